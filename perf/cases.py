@@ -408,13 +408,20 @@ def _run_init(s):
     return dict(planes=planes, branch=branch, beta=beta, y=y, **pca)
 
 
+def _rotations(q):
+    """Rotation matrices [n, 3, 3] of quaternions q [4, n] (w, x, y, z) of any length."""
+    w, x, y, z = q / q.norm(dim=0)
+    return torch.stack([1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y), 2 * (x * y + w * z), 1 - 2 * (x * x + z * z),
+                        2 * (y * z - w * x), 2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)], 1).reshape(-1, 3, 3)
+
+
 def _mlp_batch(n, seed):
     """Features as the voxel fit makes them (log variances, a rotation, colour, log footprint) and
     small residual targets."""
     gen = _gen(seed)
     x = torch.randn(n, 16, generator=gen, device=DEV)
     x[:, 0:3] = (-7 + 1.5 * x[:, 0:3]).sort(dim=1).values
-    x[:, 3:12] = torch.linalg.qr(x[:, 3:12].reshape(n, 3, 3))[0].reshape(n, 9)
+    x[:, 3:12] = _rotations(x[:, 3:7].T).reshape(n, 9)
     x[:, 12:15] = torch.rand(n, 3, generator=gen, device=DEV)
     x[:, 15] = -3.5 + 0.5 * x[:, 15]
     y = torch.zeros(n, 16, device=DEV)
@@ -930,10 +937,7 @@ def _exact_map_update(case, seed):
 
 
 def _planar64(p):
-    q = p[6:10].double()
-    w, x, y, z = q / q.norm(dim=0)
-    R = torch.stack([1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y), 2 * (x * y + w * z), 1 - 2 * (x * x + z * z),
-                     2 * (y * z - w * x), 2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)], 1).reshape(-1, 3, 3)
+    R = _rotations(p[6:10].double())
     lam = torch.ones(p.shape[1], 3, dtype=torch.float64, device=DEV)
     lam.scatter_(1, p[3:6].argmin(0)[:, None], 1e-3)
     return (R * lam[:, None, :]) @ R.transpose(1, 2)
@@ -970,7 +974,9 @@ def _exact_gicp(case, seed):
         R, t = T[:3, :3].to(DEV), T[:3, 3].to(DEV)
         x = R @ src[:, ok].double() + t[:, None]
         r = (tar[:, at[ok]].double() - x).T
-        W = torch.linalg.inv(ct[at[ok]] + R @ cs[ok] @ R.T)
+        a, b, c = (ct[at[ok]] + R @ cs[ok] @ R.T).unbind(1)       # inverse of the 3 x 3 rows
+        W = torch.stack([torch.linalg.cross(b, c), torch.linalg.cross(c, a), torch.linalg.cross(a, b)], 2)
+        W = W / (a * torch.linalg.cross(b, c)).sum(1)[:, None, None]
         J = torch.zeros(len(ok), 3, 6, dtype=torch.float64, device=DEV)
         J[:, 0, 0] = J[:, 1, 1] = J[:, 2, 2] = -1
         J[:, 0, 4], J[:, 0, 5], J[:, 1, 3] = -x[2], x[1], x[2]
