@@ -1164,7 +1164,7 @@ gs_status gs_map_update(const gs_gaussians* in, const gs_gaussians* m_in, const 
 
 
 // ---------------------------------------------------------------------------------------
-// f3: Gaussian-GICP loop registration (gicp.cu); host side: 6 x 6 solves and SE(3) updates.
+// f3: Gaussian-GICP loop registration (gicp.cu), and the SE(3) helpers of the pose twists.
 // ---------------------------------------------------------------------------------------
 static GicpMap gicp_map(const gs_gaussians* g) {
     GicpMap m;
@@ -1314,34 +1314,6 @@ gs_status gs_twist_grad(const float* xi, const float* g_left, int32_t n_views, f
     return GS_OK;
 }
 
-// Solves H x = b (6 x 6, symmetric positive definite) by Cholesky; false if not positive.
-static bool solve6(const double H[36], const double b[6], double x[6]) {
-    double L[36] = {0};
-    for (int i = 0; i < 6; i++)
-        for (int j = 0; j <= i; j++) {
-            double s = H[6 * i + j];
-            for (int k = 0; k < j; k++) s -= L[6 * i + k] * L[6 * j + k];
-            if (i == j) {
-                if (!(s > 0)) return false;
-                L[6 * i + i] = sqrt(s);
-            } else {
-                L[6 * i + j] = s / L[6 * j + j];
-            }
-        }
-    double y[6];
-    for (int i = 0; i < 6; i++) {
-        double s = b[i];
-        for (int k = 0; k < i; k++) s -= L[6 * i + k] * y[k];
-        y[i] = s / L[6 * i + i];
-    }
-    for (int i = 5; i >= 0; i--) {
-        double s = y[i];
-        for (int k = i + 1; k < 6; k++) s -= L[6 * k + i] * x[k];
-        x[i] = s / L[6 * i + i];
-    }
-    return true;
-}
-
 gs_status gs_gicp_register(const gs_gaussians* src, const uint8_t* src_flag, const gs_gaussians* tar,
                            const uint8_t* tar_flag, const double T_init[12], float d_corr, int32_t max_iters,
                            double eps, gs_gicp_result* result, void* scratch, size_t scratch_bytes, void* stream) {
@@ -1353,49 +1325,16 @@ gs_status gs_gicp_register(const gs_gaussians* src, const uint8_t* src_flag, con
     if (tar->n >= (int64_t)0x7FFFFFFFll || src->n >= (int64_t)0x7FFFFFFFll) return fail(GS_ERR_INVALID_ARG, "sizes must be < 2^31");
     if (scratch_bytes < gicp_scratch_bytes(tar->n)) return fail(GS_ERR_INVALID_ARG, "scratch too small");
     cudaStream_t st = (cudaStream_t)stream;
-    const GicpMap gs_src = gicp_map(src), gs_tar = gicp_map(tar);
-    GS_CUDA(launch_gicp_build(gs_tar, tar_flag, d_corr, scratch, st));
-    double T[16];
-    for (int r = 0; r < 3; r++)
-        for (int c = 0; c < 4; c++) T[4 * r + c] = T_init[4 * r + c];
-    T[12] = T[13] = T[14] = 0; T[15] = 1;
-    double acc[29];
-    auto evaluate = [&]() -> cudaError_t {
-        const double R[9] = {T[0], T[1], T[2], T[4], T[5], T[6], T[8], T[9], T[10]};
-        const double t[3] = {T[3], T[7], T[11]};
-        return launch_gicp_normal_eq(gs_src, src_flag, gs_tar, d_corr, R, t, scratch, acc, st);
-    };
-    int it = 0;
-    bool converged = false;
-    for (it = 1; it <= max_iters; it++) {
-        GS_CUDA(evaluate());
-        if (acc[28] < 6) break;
-        double H[36], g[6], xi[6];
-        int k = 0;
-        for (int r = 0; r < 6; r++)
-            for (int c = r; c < 6; c++) { H[6 * r + c] = acc[k]; H[6 * c + r] = acc[k]; k++; }
-        for (int r = 0; r < 6; r++) g[r] = -acc[21 + r];
-        if (!solve6(H, g, xi)) break;
-        double E[16], Tn[16];
-        se3_exp(xi, E);
-        for (int r = 0; r < 4; r++)
-            for (int c = 0; c < 4; c++) {
-                double v = 0;
-                for (int e = 0; e < 4; e++) v += E[4 * r + e] * T[4 * e + c];
-                Tn[4 * r + c] = v;
-            }
-        for (int k2 = 0; k2 < 16; k2++) T[k2] = Tn[k2];
-        double nrm = 0;
-        for (int r = 0; r < 6; r++) nrm += xi[r] * xi[r];
-        if (sqrt(nrm) < eps) { converged = true; break; }
-    }
-    GS_CUDA(evaluate());
-    for (int r = 0; r < 3; r++)
-        for (int c = 0; c < 4; c++) result->T[4 * r + c] = T[4 * r + c];
-    result->cost = acc[27];
-    result->n_corr = (int64_t)acc[28];
-    result->iters = it > max_iters ? max_iters : it;
-    result->converged = converged ? 1 : 0;
+    double T0[12];
+    for (int k = 0; k < 12; k++) T0[k] = T_init[k];
+    GicpOutcome out;
+    GS_CUDA(launch_gicp_register(gicp_map(src), src_flag, gicp_map(tar), tar_flag, T0, d_corr, max_iters, eps, scratch,
+                                 scratch_bytes, &out, st));
+    for (int k = 0; k < 12; k++) result->T[k] = out.T[k];
+    result->cost = out.cost;
+    result->n_corr = out.n_corr;
+    result->iters = out.iters;
+    result->converged = out.converged;
     return GS_OK;
 }
 

@@ -209,12 +209,16 @@ size_t gicp_scratch_bytes(int64_t n_tar);
 cudaError_t launch_gicp_target_set(const GicpMap& map, const GicpView* views, int n_views, float near_z, float dmax2,
                                    const uint8_t* source_flag, uint8_t* target_flag, void* scratch,
                                    unsigned long long* count_host, cudaStream_t st);
-// builds the target hash (once per registration)
-cudaError_t launch_gicp_build(const GicpMap& tar, const uint8_t* tar_flag, float d_corr, void* scratch, cudaStream_t st);
-// accumulates H (21, upper triangle row-major), g (6), cost, count for transform (R, t) into
-// 29 doubles copied to acc_host
-cudaError_t launch_gicp_normal_eq(const GicpMap& src, const uint8_t* src_flag, const GicpMap& tar, float d_corr,
-                                  const double* R, const double* t, void* scratch, double* acc_host, cudaStream_t st);
+struct GicpOutcome {
+    double T[12];
+    double cost;
+    int64_t n_corr;
+    int iters, converged;
+};
+// The registration from T0 (row-major 3 x 4) to its end; synchronises the stream.
+cudaError_t launch_gicp_register(const GicpMap& src, const uint8_t* src_flag, const GicpMap& tar, const uint8_t* tar_flag,
+                                 const double (&T0)[12], float d_corr, int max_iters, double eps, void* scratch,
+                                 size_t scratch_bytes, GicpOutcome* out, cudaStream_t st);
 
 cudaError_t launch_project(const ProjectArgs& a, int deg, cudaStream_t st);
 cudaError_t launch_project_bwd(const ProjectBwdArgs& a, int deg, cudaStream_t st);
