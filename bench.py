@@ -338,7 +338,7 @@ def run_gpu(args, rank, world):
         torch.cuda.synchronize()
         c = step.ws.counters()
         print(json.dumps({"profile_step": args.profile_step, "status": int(c.status), "pairs": int(c.n_pairs),
-                          "kernels_per_step": kernels_per_step(step.ws.layout)}), flush=True)
+                          "kernels_per_step": launches_per_step(step.ws.layout)}), flush=True)
         sys.exit(0 if c.status == 0 else 1)
     stages = ["project", "bin_sort", "render_fwd", "composite_bwd", "project_bwd_adam"]
     st = torch.cuda.current_stream()
@@ -415,7 +415,7 @@ def run_gpu(args, rank, world):
         return dict(f1=None, f23=None, a9=None, total_ms=total_ms, stage_ms=stage_ms, n_pairs=n_pairs, loss0=loss0,
                     loss_end=loss_end, tune=tune, adam_steps=adam_steps, eager_ms=None, h2d_ms=None, work=work,
                     clocks=clk.summary(), e2e_s=None, px=sum(w * h for w, h in SIZES), h2d=0, d2h=0, sc=sc,
-                    cams=cams, trgb=trgb, tdep=tdep, n=n, kernels=kernels_per_step(step.ws.layout),
+                    cams=cams, trgb=trgb, tdep=tdep, n=n, kernels=launches_per_step(step.ws.layout),
                     sms=torch.cuda.get_device_properties(dev).multi_processor_count)
     f1 = f1_measure(args, step, cams, trgb, tdep, planes0, cap, st, dev)
     f23 = f23_measure(step, cams, dev)
@@ -463,7 +463,7 @@ def run_gpu(args, rank, world):
                 tune=tune, adam_steps=adam_steps, eager_ms=eager_ms, h2d_ms=h2d_ms, work=work,
                 clocks=clk.summary(), e2e_s=e_dt, px=px, h2d=int(h_rgb.numel() * 4 + h_dep.numel() * 4),
                 d2h=int(h_loss.numel() * 4), sc=sc, cams=cams, trgb=trgb, tdep=tdep, n=n,
-                kernels=kernels_per_step(step.ws.layout),
+                kernels=launches_per_step(step.ws.layout),
                 sms=torch.cuda.get_device_properties(dev).multi_processor_count)
 
 
@@ -659,13 +659,24 @@ def tile_sort_passes(L):
 
 
 def kernels_per_step(L):
-    """Kernels one gs_step launches (the graph replays exactly these)."""
+    """Kernels of one step with every scan and sort pass as separate kernels (upsweep, scan,
+    downsweep): what launches_per_step's single-pass forms replace."""
     # view table, project, entry count / scan / compaction, 4 depth-sort passes of 3
     # kernels, pair count / scan / offsets / emission, 3 per tile-sort pass, ranges, 3
     # tile-order kernels, loss count + composite, gradient-record clear (with the loss terms
     # and the Adam counter) + composite backward, projection backward entry, SH and geometry
-    # (+ Adam) parts (38 with two tile-sort passes, as the ncu launch list of one step shows)
+    # (+ Adam) parts (38 with two tile-sort passes)
     return 1 + 1 + 3 + 3 * 4 + 4 + 3 * tile_sort_passes(L) + 1 + 3 + 2 + 2 + 3
+
+
+def launches_per_step(L, sms=152):
+    """Kernels one gs_step launches (the graph replays exactly these)."""
+    # setup (view table and clears), project, entry compaction (a count kernel before it once its
+    # blocks of 64 words are more than 4 per SM), 4 depth-sort passes, pair offsets, emission, the
+    # tile-sort passes, ranges, 2 tile-order kernels, loss count + composite, gradient-record
+    # clear + composite backward, projection backward entry, SH and geometry (+ Adam) parts
+    blocks = -(-(L.n_views * -(-L.n // 32)) // 64)
+    return 1 + 1 + (1 if blocks <= 4 * sms else 2) + 4 + 2 + tile_sort_passes(L) + 1 + 2 + 2 + 2 + 3
 
 
 # Algorithmic FP32 work per evaluated fragment, (pixel, Gaussian) pairs tested: 20 operations in

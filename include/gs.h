@@ -134,7 +134,7 @@ typedef struct {
     size_t vis_bits;     /* uint32 [n_views][ceil(n/32)]: bit i % 32 of word
                             v * ceil(n/32) + i / 32 is set when Gaussian i covers a tile of
                             view v (its record in proj is then valid); other bits are 0 */
-    size_t scan_tmp;     /* uint32 scratch of the scans */
+    size_t scan_tmp;     /* uint64 look-back words of the scans */
     size_t ekeys0, ekeys1; /* uint32 [n_views*n] ping-pong: bits(z) of the visible entries */
     size_t evals0, evals1; /* uint32 [n_views*n] ping-pong: their compact indices (positions
                               in `entries`); after gs_bin_sort evals0 lists the entries by depth */
@@ -146,7 +146,7 @@ typedef struct {
                             its tile that hold pixels with alpha >= alpha_min (written by
                             gs_render_fwd, read by the backward) */
     size_t emit_tmp;     /* uint32 scratch of the pair emission */
-    size_t sort_tmp;     /* uint32 scratch of the radix sorts */
+    size_t sort_tmp;     /* scratch of the radix sorts: digit counts, tickets, look-back words */
     size_t ranges;       /* uint32 [total_tiles][2] [first, last+1) in the sorted pairs */
     size_t T_final;      /* float [total_pixels] */
     size_t n_contrib;    /* uint32 [total_pixels] tile-list position after the last added */
@@ -160,8 +160,9 @@ typedef struct {
                             view directions (projection backward: SH part -> geometry part) */
     size_t visible;      /* uint8 [n]: 1 if the Gaussian covers a tile of any view */
     size_t entries;      /* uint32 [n_views*n]: the visible entries in (view, Gaussian) order */
-    size_t erect;        /* uint32 [n_views*n][2]: per visible entry, in the order of `entries`,
-                            its tile rectangle (first global tile id, wx | wy << 16) */
+    size_t erect;        /* uint32 [n_views*n][4]: per visible entry, in the order of `entries`,
+                            its tile rectangle (first global tile id, wx | wy << 16), view * n +
+                            index and a pad word */
     size_t tile_order;   /* uint32 [total_tiles]: compositing work order, largest pair count
                             first (power-of-two buckets), then scratch */
     size_t render_mask;  /* uint8 [total_pixels]: the step's interior mask (mask_erode >= 0) */

@@ -1,6 +1,7 @@
 // extern "C" entry points declared in include/gs.h: argument checks, workspace layout and
 // the launch sequence of each stage.  Host code only; all arithmetic of the step runs in
 // the kernels of project.cu, binsort.cu, render.cu and adam.cu.
+#include <cassert>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -33,6 +34,12 @@ static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // loss accumulators: double [GS_MAX_VIEWS][3] sums, then uint32 [GS_MAX_VIEWS][2] counts
 constexpr size_t kLossAccBytes = sizeof(double) * 3 * GS_MAX_VIEWS + sizeof(uint32_t) * 2 * GS_MAX_VIEWS;
+
+// sort_tmp: the digit counts of the passes of the two sorts, the tickets of their passes and of
+// the two scans, then the look-back words (all cleared by the binning's setup)
+constexpr size_t kSortHist = sizeof(uint32_t) * 2 * kSortMaxPasses * kSortMaxBins;
+constexpr size_t kSortTickets = sizeof(uint32_t) * (2 * kSortMaxPasses + 2);
+constexpr size_t kSortHead = (kSortHist + kSortTickets + 255) & ~(size_t)255;
 
 struct Geometry {
     int total_tiles = 0;
@@ -141,7 +148,7 @@ static gs_status layout(int64_t n, int32_t n_views, const gs_camera* cams, const
     L.loss_acc = take(kLossAccBytes);
     L.proj = take(sizeof(float) * 12 * (size_t)VN);
     L.vis_bits = take(sizeof(uint32_t) * (size_t)n_views * (size_t)((n + 31) / 32));
-    L.scan_tmp = take(sizeof(uint32_t) * ((size_t)VN / kScanBlock + 2));
+    L.scan_tmp = take(sizeof(unsigned long long) * (entry_scan_words(n, n_views) + pair_scan_words(n, n_views)));
     L.ekeys0 = take(sizeof(uint32_t) * (size_t)VN);
     L.ekeys1 = take(sizeof(uint32_t) * (size_t)VN);
     L.evals0 = take(sizeof(uint32_t) * (size_t)VN);
@@ -152,7 +159,12 @@ static gs_status layout(int64_t n, int32_t n_views, const gs_camera* cams, const
     L.vals1 = take(sizeof(uint32_t) * (size_t)max_pairs);
     L.pair_mask = take((size_t)max_pairs);
     L.emit_tmp = take(sizeof(uint32_t) * ((size_t)max_pairs / kEmitChunk + 2));
-    L.sort_tmp = take(sizeof(uint32_t) * ((size_t)kSortMaxBins * kSortMaxGrid + kSortMaxBins));
+    int shifts[16], bits[16];
+    const int np = pair_sort_passes(G.total_tiles, shifts, bits);
+    {
+        const size_t le = sort_lookback_bytes(VN, 8), lp = sort_lookback_bytes(max_pairs, np > 0 ? bits[np - 1] : 8);
+        L.sort_tmp = take(kSortHead + (le > lp ? le : lp));
+    }
     L.ranges = take(sizeof(uint32_t) * 2 * (size_t)G.total_tiles);
     L.T_final = take(sizeof(float) * (size_t)G.total_pixels);
     L.n_contrib = take(sizeof(uint32_t) * (size_t)G.total_pixels);
@@ -160,15 +172,14 @@ static gs_status layout(int64_t n, int32_t n_views, const gs_camera* cams, const
     L.geo2d = take(sizeof(float) * 12 * (size_t)VN);
     L.dirgrad = take(sizeof(float) * 3 * (size_t)n);
     L.entries = take(sizeof(uint32_t) * (size_t)VN);
-    L.erect = take(sizeof(uint32_t) * 2 * (size_t)VN);
+    L.erect = take(sizeof(uint32_t) * 4 * (size_t)VN);
     L.visible = take((size_t)n);
-    L.tile_order = take(sizeof(uint32_t) * ((size_t)G.total_tiles + 2 * 34));
+    L.tile_order = take(sizeof(uint32_t) * ((size_t)G.total_tiles + kOrderTmpWords));
     L.render_mask = take((size_t)G.total_pixels);
     L.has_ssim = o->lambda_ssim > 0.f ? 1 : 0;
     L.ssim_tmp = take(L.has_ssim ? sizeof(float) * 9 * (size_t)G.total_pixels : 0);
     L.total = off;
-    int shifts[16], bits[16];
-    L.sorted_buf = pair_sort_passes(G.total_tiles, shifts, bits) & 1;
+    L.sorted_buf = np & 1;
     L.total_tiles = G.total_tiles;
     L.total_pixels = G.total_pixels;
     L.max_pairs = max_pairs;
@@ -192,21 +203,71 @@ static Opts to_opts(const gs_render_opts* o) {
     return r;
 }
 
-struct ViewsParam {
+// A call's setup: the view table, and the words its stages expect to be zero, in one launch.
+struct SetupParam {
     int n;
+    int n_clear;
     View v[GS_MAX_VIEWS];
+    struct { uint32_t* p; uint32_t words; } clear[10];
 };
+static_assert(sizeof(SetupParam) + 8 <= 4096, "kernel parameters");
 
-__global__ void setup_views_kernel(View* dst, const __grid_constant__ ViewsParam p) {
-    for (int i = threadIdx.x; i < p.n; i += blockDim.x) dst[i] = p.v[i];
+__global__ void __launch_bounds__(256) setup_kernel(View* dst, const __grid_constant__ SetupParam p) {
+    if (blockIdx.x == 0)
+        for (int i = threadIdx.x; i < p.n; i += blockDim.x) dst[i] = p.v[i];
+    for (int k = 0; k < p.n_clear; k++) {
+            // 16 bytes a store where the range is aligned, which the large ones are
+            uint32_t* q = p.clear[k].p;
+            const uint32_t words = p.clear[k].words, quads = (reinterpret_cast<uintptr_t>(q) & 15) ? 0u : words / 4;
+            const uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+            for (uint32_t i = i0; i < quads; i += step) reinterpret_cast<uint4*>(q)[i] = make_uint4(0u, 0u, 0u, 0u);
+            for (uint32_t i = 4 * quads + i0; i < words; i += step) q[i] = 0u;
+        }
 }
 
-static gs_status upload_views(void* ws, const gs_ws_layout& L, const Geometry& G, int n_views, cudaStream_t st) {
-    ViewsParam p;
+static void setup_add(SetupParam& p, void* ptr, size_t bytes) {
+    if (bytes == 0) return;
+    assert(p.n_clear < (int)(sizeof(p.clear) / sizeof(p.clear[0])));
+    p.clear[p.n_clear].p = static_cast<uint32_t*>(ptr);
+    p.clear[p.n_clear++].words = (uint32_t)(bytes / sizeof(uint32_t));
+}
+
+// What a call's stages expect to be zero.
+enum { kSetupProject = 1, kSetupBin = 2, kSetupLoss = 4 };
+
+static SetupParam setup_param(void* ws, const gs_ws_layout& L, const Geometry& G, int what, float* grad_twist = nullptr) {
+    SetupParam p;
     memset(&p, 0, sizeof(p));
-    p.n = n_views;
-    memcpy(p.v, G.views, sizeof(View) * n_views);
-    setup_views_kernel<<<1, 32, 0, st>>>(at<View>(ws, L.views), p);
+    p.n = L.n_views;
+    memcpy(p.v, G.views, sizeof(View) * L.n_views);
+    Counters* c = at<Counters>(ws, L.counters);
+    if (what & kSetupProject) setup_add(p, c, kCountersResetBytes);
+    if (what & kSetupBin) {
+        // entry and pair counts (written by the last chunk of a scan, if there is one)
+        setup_add(p, &c->n_entries32, 12);
+        setup_add(p, &c->n_entries, 8);
+        setup_add(p, at<char>(ws, L.scan_tmp),
+                  sizeof(unsigned long long) * (entry_scan_words(L.n, L.n_views) + pair_scan_words(L.n, L.n_views)));
+        setup_add(p, at<char>(ws, L.sort_tmp), L.ranges - L.sort_tmp);   // (the region's padding too)
+        setup_add(p, at<char>(ws, L.ranges), sizeof(uint32_t) * 2 * (size_t)L.total_tiles);
+        setup_add(p, at<uint32_t>(ws, L.tile_order) + L.total_tiles, sizeof(uint32_t) * kOrderTmpWords);
+    }
+    if (what & kSetupLoss) setup_add(p, at<char>(ws, L.loss_acc), kLossAccBytes);
+    if (grad_twist) setup_add(p, grad_twist, sizeof(float) * 6 * L.n_views);
+    return p;
+}
+
+static int setup_grid(const SetupParam& p) {
+    uint32_t words = 0;
+    for (int k = 0; k < p.n_clear; k++) words = p.clear[k].words > words ? p.clear[k].words : words;
+    const uint32_t g = (words + 2047) / 2048;   // two 16-byte stores a thread
+    return g < 1 ? 1 : (g > 128 ? 128 : (int)g);
+}
+
+static gs_status run_setup(void* ws, const gs_ws_layout& L, const Geometry& G, int what, cudaStream_t st,
+                           float* grad_twist = nullptr) {
+    const SetupParam p = setup_param(ws, L, G, what, grad_twist);
+    setup_kernel<<<setup_grid(p), 256, 0, st>>>(at<View>(ws, L.views), p);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }
@@ -245,8 +306,6 @@ static gs_status geometry_for(const gs_ws_layout* L, const gs_camera* cams, cons
 // ---------------------------------------------------------------------------------------
 static cudaError_t run_project(const gs_gaussians* g, const gs_render_opts* opts, const gs_ws_layout* L, void* ws,
                                cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(at<Counters>(ws, L->counters), 0, kCountersResetBytes, st);
-    if (e != cudaSuccess) return e;
     ProjectArgs a;
     a.n = g->n;
     a.n_views = L->n_views;
@@ -270,11 +329,19 @@ static cudaError_t run_bin_sort(const gs_render_opts* opts, const gs_ws_layout* 
     b.max_pairs = L->max_pairs;
     b.proj = at<float4>(ws, L->proj);
     b.vis_bits = at<uint32_t>(ws, L->vis_bits);
-    b.scan_tmp = at<uint32_t>(ws, L->scan_tmp);
+    uint32_t* tickets = reinterpret_cast<uint32_t*>(at<char>(ws, L->sort_tmp) + kSortHist);
+    b.entry_scan = at<unsigned long long>(ws, L->scan_tmp);
+    b.pair_scan = b.entry_scan + entry_scan_words(L->n, L->n_views);
+    b.tickets = tickets + 2 * kSortMaxPasses;
+    int shifts[16], bits[16];
+    const int np = pair_sort_passes(L->total_tiles, shifts, bits);
+    b.ehist = at<uint32_t>(ws, L->sort_tmp);
+    b.phist = b.ehist + kSortMaxPasses * kSortMaxBins;
+    b.phist_mask = np > 0 ? (1u << bits[0]) - 1u : 0u;
     b.ekeys = at<uint32_t>(ws, L->ekeys0);
     b.evals = at<uint32_t>(ws, L->evals0);
     b.entries = at<uint32_t>(ws, L->entries);
-    b.erect = at<uint2>(ws, L->erect);
+    b.erect = at<uint4>(ws, L->erect);
     b.sorted_evals = at<uint32_t>(ws, L->evals0);   // 4 passes: the entry sort ends in buffer 0
     b.pkeys = at<uint32_t>(ws, L->keys0);
     b.pvals = at<uint32_t>(ws, L->vals0);
@@ -286,15 +353,16 @@ static cudaError_t run_bin_sort(const gs_render_opts* opts, const gs_ws_layout* 
     if (e != cudaSuccess) return e;
     SortArgs sa;
     sa.hist = at<uint32_t>(ws, L->sort_tmp);
-    sa.digit_tot = sa.hist + (size_t)kSortMaxBins * kSortMaxGrid;
+    sa.tickets = tickets;
+    sa.lookback = reinterpret_cast<unsigned long long*>(at<char>(ws, L->sort_tmp) + kSortHead);
     sa.counters = cnt;
-    sa.grid = sort_grid();
     // 1. entries by depth
     sa.keys[0] = at<uint32_t>(ws, L->ekeys0);
     sa.keys[1] = at<uint32_t>(ws, L->ekeys1);
     sa.vals[0] = at<uint32_t>(ws, L->evals0);
     sa.vals[1] = at<uint32_t>(ws, L->evals1);
     sa.count = &cnt->n_entries;
+    sa.capacity = (int64_t)L->n_views * L->n;
     const int depth_shifts[4] = {0, 8, 16, 24}, depth_bits[4] = {8, 8, 8, 8};
     if ((e = launch_sort32(sa, 4, depth_shifts, depth_bits, st)) != cudaSuccess) return e;
     // 2. pairs emitted in depth order, then by tile
@@ -304,12 +372,11 @@ static cudaError_t run_bin_sort(const gs_render_opts* opts, const gs_ws_layout* 
     sa.vals[0] = at<uint32_t>(ws, L->vals0);
     sa.vals[1] = at<uint32_t>(ws, L->vals1);
     sa.count = &cnt->n_pairs;
-    int shifts[16], bits[16];
-    const int np = pair_sort_passes(L->total_tiles, shifts, bits);
+    sa.capacity = L->max_pairs;
+    sa.hist += kSortMaxPasses * kSortMaxBins;
+    sa.tickets += kSortMaxPasses;
+    sa.tag = 1 + kSortMaxPasses;   // (the two sorts share the look-back words)
     if ((e = launch_sort32(sa, np, shifts, bits, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(at<uint32_t>(ws, L->ranges), 0, sizeof(uint32_t) * 2 * (size_t)L->total_tiles, st)) !=
-        cudaSuccess)
-        return e;
     RangeArgs r;
     r.keys = static_cast<const uint32_t*>(sa.keys[np & 1]);
     r.ranges = at<uint2>(ws, L->ranges);
@@ -359,7 +426,6 @@ static cudaError_t run_objective(const gs_render_opts* opts, const gs_ws_layout*
                                  float* loss_out, cudaStream_t st) {
     ObjArgs o = obj_args(opts, L, G, ws);
     cudaError_t e;
-    if ((e = cudaMemsetAsync(o.sums, 0, kLossAccBytes, st)) != cudaSuccess) return e;
     if ((e = launch_loss_count(o.views, L->n_views, G.pix, target_depth, mask, const_cast<uint32_t*>(o.counts), st)) !=
         cudaSuccess)
         return e;
@@ -436,7 +502,6 @@ static cudaError_t run_fwd(const gs_render_opts* opts, const gs_ws_layout* L, co
     const bool fused = target_rgb && !separate;
     cudaError_t e;
     if (fused) {
-        if ((e = cudaMemsetAsync(sums, 0, kLossAccBytes, st)) != cudaSuccess) return e;
         if ((e = launch_loss_count(at<View>(ws, L->views), L->n_views, G.pix, target_depth, mask, counts, st)) !=
             cudaSuccess)
             return e;
@@ -629,7 +694,7 @@ static gs_status run_step(gs_gaussians* params, gs_gaussians* grads, gs_gaussian
     } else if (host_in) {
         GS_CUDA(upload_targets(io, L, st));
     }
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, kSetupProject | kSetupBin | kSetupLoss, st, io->grad_twist)) != GS_OK) return s;
     GS_CUDA(run_project(params, opts, L, ws, st));
     GS_CUDA(run_bin_sort(opts, L, ws, st));
     if (branch) GS_CUDA(cudaStreamWaitEvent(st, cb->join, 0));   // targets needed from here on
@@ -649,9 +714,7 @@ static gs_status run_step_tail(gs_gaussians* params, gs_gaussians* grads, gs_gau
         // kernel for forward, backward, projection backward and Adam
         double* sums = at<double>(ws, L->loss_acc);
         uint32_t* counts = reinterpret_cast<uint32_t*>(sums + 3 * GS_MAX_VIEWS);
-        GS_CUDA(cudaMemsetAsync(sums, 0, kLossAccBytes, st));
         GS_CUDA(launch_loss_count(at<View>(ws, L->views), L->n_views, G.pix, io->target_depth, io->mask, counts, st));
-        if (io->grad_twist) GS_CUDA(cudaMemsetAsync(io->grad_twist, 0, sizeof(float) * 6 * L->n_views, st));
         const float* dl_dd = io->target_depth ? io->dl_ddepth : nullptr;
         const FwdArgs fa_ = fwd_args(opts, L, ws, io->out_rgb, io->out_depth, nullptr, io->target_rgb, io->target_depth,
                                      io->mask, io->dl_drgb, io->target_depth ? io->dl_ddepth : nullptr);
@@ -670,7 +733,6 @@ static gs_status run_step_tail(gs_gaussians* params, gs_gaussians* grads, gs_gau
     GS_CUDA(run_fwd(opts, L, G, ws, io->out_rgb, io->out_depth, nullptr, io->target_rgb, io->target_depth, io->mask,
                     io->dl_drgb, io->target_depth ? io->dl_ddepth : nullptr, io->loss_out, st,
                     io->optimize ? &lf : nullptr));
-    if (io->grad_twist) GS_CUDA(cudaMemsetAsync(io->grad_twist, 0, sizeof(float) * 6 * L->n_views, st));
     const float* dl_dd = io->target_depth ? io->dl_ddepth : nullptr;
     if (io->optimize) {
         Counters* c = at<Counters>(ws, L->counters);
@@ -700,13 +762,14 @@ static gs_status check_step(gs_gaussians* params, gs_gaussians* grads, gs_gaussi
     return geometry_for(L, cams, opts, G);
 }
 
-// Captured step: the graph, its executable and the node of the view-table upload, whose
-// by-value camera argument gs_graph_set_cameras rewrites.
+// Captured step: the graph, its executable and the setup node, whose by-value view table
+// gs_graph_set_cameras rewrites.
 struct GraphState {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphNode_t views_node = nullptr;
     cudaKernelNodeParams views_params;
+    SetupParam setup;   // its argument as captured
     gs_render_opts opts;
     gs_ws_layout layout;
     void* ws = nullptr;
@@ -804,7 +867,7 @@ gs_status gs_project(const gs_gaussians* g, const gs_camera* cams, const gs_rend
     Geometry G;
     if ((s = geometry_for(L, cams, opts, G)) != GS_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, kSetupProject, st)) != GS_OK) return s;
     GS_CUDA(run_project(g, opts, L, ws, st));
     return GS_OK;
 }
@@ -815,7 +878,7 @@ gs_status gs_bin_sort(const gs_camera* cams, const gs_render_opts* opts, const g
     Geometry G;
     if ((s = geometry_for(L, cams, opts, G)) != GS_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, kSetupBin, st)) != GS_OK) return s;
     GS_CUDA(run_bin_sort(opts, L, ws, st));
     return GS_OK;
 }
@@ -833,7 +896,7 @@ gs_status gs_render_fwd(const gs_camera* cams, const gs_render_opts* opts, const
     if (target_depth && !target_rgb) return fail(GS_ERR_INVALID_ARG, "target_depth needs target_rgb");
     if (target_depth && !dl_ddepth) return fail(GS_ERR_INVALID_ARG, "the depth loss needs dl_ddepth");
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, kSetupLoss, st)) != GS_OK) return s;
     GS_CUDA(run_fwd(opts, L, G, ws, out_rgb, out_depth, out_T, target_rgb, target_depth, mask, dl_drgb, dl_ddepth,
                     loss_out, st));
     return GS_OK;
@@ -847,7 +910,7 @@ gs_status gs_render_mask(const gs_camera* cams, const gs_render_opts* opts, cons
     if ((s = geometry_for(L, cams, opts, G)) != GS_OK) return s;
     if (!mask_out) return fail(GS_ERR_INVALID_ARG, "mask_out is NULL");
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, 0, st)) != GS_OK) return s;
     GS_CUDA(run_render_mask(opts, L, G, ws, caller_mask, mask_out, st));
     return GS_OK;
 }
@@ -862,7 +925,7 @@ gs_status gs_objective(const gs_camera* cams, const gs_render_opts* opts, const 
     if (!rgb || !target_rgb || !dl_drgb || !loss_out) return fail(GS_ERR_INVALID_ARG, "rgb, target_rgb, dl_drgb and loss_out are required");
     if (target_depth && (!depth || !dl_ddepth)) return fail(GS_ERR_INVALID_ARG, "the depth term needs depth and dl_ddepth");
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, kSetupLoss, st)) != GS_OK) return s;
     GS_CUDA(run_objective(opts, L, G, ws, rgb, depth, target_rgb, target_depth, mask, dl_drgb, dl_ddepth, loss_out, st));
     return GS_OK;
 }
@@ -880,7 +943,7 @@ gs_status gs_render_bwd(const gs_gaussians* g, const gs_camera* cams, const gs_r
     Geometry G;
     if ((s = geometry_for(L, cams, opts, G)) != GS_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, 0, st)) != GS_OK) return s;
     GS_CUDA(run_bwd(g, opts, L, ws, dl_drgb, dl_ddepth, grads, grad_twist, st));
     return GS_OK;
 }
@@ -893,7 +956,7 @@ gs_status gs_composite_bwd(const gs_camera* cams, const gs_render_opts* opts, co
     Geometry G;
     if ((s = geometry_for(L, cams, opts, G)) != GS_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, 0, st)) != GS_OK) return s;
     GS_CUDA(run_composite_bwd(opts, L, ws, dl_drgb, dl_ddepth, st));
     return GS_OK;
 }
@@ -909,7 +972,7 @@ gs_status gs_project_bwd(const gs_gaussians* g, const gs_camera* cams, const gs_
     Geometry G;
     if ((s = geometry_for(L, cams, opts, G)) != GS_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, 0, st)) != GS_OK) return s;
     GS_CUDA(run_project_bwd(g, opts, L, ws, grads, grad_twist, st));
     return GS_OK;
 }
@@ -927,7 +990,7 @@ gs_status gs_project_bwd_adam(gs_gaussians* params, const gs_camera* cams, const
     Geometry G;
     if ((s = geometry_for(L, cams, opts, G)) != GS_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    if ((s = upload_views(ws, *L, G, L->n_views, st)) != GS_OK) return s;
+    if ((s = run_setup(ws, *L, G, 0, st)) != GS_OK) return s;
     FusedAdam fa{params, m, v, update_mask, lr, b1, b2, eps, step, nullptr};
     GS_CUDA(run_project_bwd(params, opts, L, ws, nullptr, grad_twist, st, &fa));
     return GS_OK;
@@ -993,6 +1056,7 @@ gs_status gs_graph_create(gs_graph* out, gs_gaussians* params, gs_gaussians* gra
         return s != GS_OK ? s : fail(GS_ERR_CUDA, "cudaStreamEndCapture: %s", cudaGetErrorString(ec));
     }
     gst->graph = graph;
+    gst->setup = setup_param(ws, *L, G, kSetupProject | kSetupBin | kSetupLoss, io->grad_twist);
     size_t nn = 0;
     cudaGraphGetNodes(graph, nullptr, &nn);
     cudaGraphNode_t* nodes = new cudaGraphNode_t[nn ? nn : 1];
@@ -1002,7 +1066,7 @@ gs_status gs_graph_create(gs_graph* out, gs_gaussians* params, gs_gaussians* gra
         if (cudaGraphNodeGetType(nodes[i], &t) != cudaSuccess || t != cudaGraphNodeTypeKernel) continue;
         cudaKernelNodeParams kp;
         if (cudaGraphKernelNodeGetParams(nodes[i], &kp) != cudaSuccess) continue;
-        if (kp.func == reinterpret_cast<void*>(setup_views_kernel)) {
+        if (kp.func == reinterpret_cast<void*>(setup_kernel)) {
             gst->views_node = nodes[i];
             gst->views_params = kp;
         }
@@ -1032,9 +1096,7 @@ gs_status gs_graph_set_cameras(gs_graph g, const gs_camera* cams) {
     Geometry G;
     gs_status s = geometry_for(&gst->layout, cams, &gst->opts, G);
     if (s != GS_OK) return s;
-    ViewsParam p;
-    memset(&p, 0, sizeof(p));
-    p.n = gst->layout.n_views;
+    SetupParam p = gst->setup;
     memcpy(p.v, G.views, sizeof(View) * p.n);
     View* dst = at<View>(gst->ws, gst->layout.views);
     void* args[2] = {&dst, &p};

@@ -11,12 +11,12 @@
 // Both sorts are stable, so pass 2 keeps the depth order within a tile and pass 1 keeps
 // (view, index) order between equal depths: the result is the order above.
 //
-// The sorts run on a fixed grid (a multiple of the SM count) whose blocks each own a
-// contiguous run of chunks; element counts are read on the device, so no host round trip
-// is needed between the stages and the whole sequence can be captured in a CUDA graph.
-// Every pass: per-block digit histograms (upsweep), a per-digit scan over the blocks (one
-// warp per digit), then a stable scatter (downsweep) that ranks each chunk with warp
-// ballot counting and writes digit runs contiguously.
+// Element counts are read on the device, so no host round trip is needed between the stages and
+// the whole sequence can be captured in a CUDA graph.  A sort pass is one kernel: every block
+// counts the digits of its run of chunks, gets the counts of the blocks before it by look-back
+// (gs_internal.cuh), and scatters its chunks, ranked by warp ballots, in digit runs; the digit
+// totals a pass needs are counted by the kernel before it.  With separate histogram, scan and
+// scatter kernels a pass took 20 us however few the keys (launches and latency).
 #include "gs_kernels.cuh"
 
 namespace gs {
@@ -52,81 +52,137 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_1024(uint32_t x, uint32
     return r;
 }
 
-// One block: exclusive scan of nb block sums in place; the total goes to *total_out and
-// sets GS_ERR_CAPACITY when it exceeds max_total (max_total < 0: no limit).
-__global__ void __launch_bounds__(kScanThreads) scan_blocks_kernel(uint32_t* __restrict__ bsum, int nb,
-                                                                  unsigned long long* total_out,
-                                                                  uint32_t* total32_out, Counters* c,
-                                                                  int64_t max_total) {
-    __shared__ uint32_t s[33];
-    if (c->status != 0) return;
+// ----------------------------------------------------------------------------------------
+// Entry compaction.  The projection leaves one bit word per view and 32 Gaussians (vis_bits,
+// each view padded to whole words).  A block of kEntryThreads threads takes WPW words per warp;
+// each warp writes the entries of its words, one word at a time with a lane per slot, so entries
+// stay in (view, index) order.  32 words per warp on large maps; 8 (two rounds of gathers
+// instead of eight) shorten the chain of dependent gathers where few blocks are resident anyway.
+// The blocks' first positions come from a look-back scan while the blocks are about one wave
+// (9 us in all at 10k slots, 25 us with separate count and scan kernels), else from a count
+// kernel whose last block scans the totals: a look-back stalls each further wave of blocks (58
+// against 49 us at 16M slots).
+// ----------------------------------------------------------------------------------------
+constexpr int kEntryThreads = 256;
+constexpr int kEntryWarps = kEntryThreads / 32;
+static_assert(kEntryMinWords == 8 * kEntryWarps && kEntryThreads == 32 * kEntryWarps, "words per block of the short form");
+
+// Entries of every block's words (blocks of `wpb` words), and their exclusive scan by the last
+// block to finish; the total goes to the counters.  A thread counts four words.
+constexpr int kCountWords = 4 * kEntryThreads;
+
+__global__ void __launch_bounds__(kEntryThreads) entry_count_kernel(BinArgs a, int64_t n_words, int wpb, int n_blocks) {
+    constexpr int GT = kEntryMinWords / 4;   // threads per kEntryMinWords words
+    __shared__ uint32_t s[kEntryThreads / GT], s_w[33];
+    __shared__ bool last;
+    if (a.counters->status != 0) return;
+    const int64_t word = (int64_t)blockIdx.x * kCountWords + 4 * threadIdx.x;
+    uint32_t sum = 0;
+    if (word + 3 < n_words) {
+        const uint4 q = *reinterpret_cast<const uint4*>(a.vis_bits + word);
+        sum = __popc(q.x) + __popc(q.y) + __popc(q.z) + __popc(q.w);
+    } else {
+        for (int64_t k = word; k < n_words; k++) sum += __popc(a.vis_bits[k]);
+    }
+#pragma unroll
+    for (int o = GT / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (threadIdx.x % GT == 0) s[threadIdx.x / GT] = sum;
+    __syncthreads();
+    const int per = kCountWords / wpb, groups = wpb / kEntryMinWords;   // totals of this block; groups of each
+    if ((int)threadIdx.x < per) {
+        uint32_t t = 0;
+        for (int k = 0; k < groups; k++) t += s[threadIdx.x * groups + k];
+        const int64_t b = (int64_t)blockIdx.x * per + threadIdx.x;
+        if (b < n_blocks) a.entry_scan[b] = t;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&a.tickets[0], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     unsigned long long carry = 0;
-    for (int base = 0; base < nb; base += kScanThreads) {
-        const int j = base + threadIdx.x;
-        const uint32_t x = j < nb ? bsum[j] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_exclusive_scan_1024(x, s, tot);
-        if (j < nb) bsum[j] = (uint32_t)(carry + ex);
+    constexpr int PT = 8;   // totals per thread and round
+    for (int base = 0; base < n_blocks; base += PT * kEntryThreads) {
+        uint32_t x[PT], sum8 = 0, tot;
+#pragma unroll
+        for (int k = 0; k < PT; k++) {
+            const int j = base + (int)threadIdx.x * PT + k;
+            x[k] = j < n_blocks ? (uint32_t)__ldcg(&a.entry_scan[j]) : 0u;
+            sum8 += x[k];
+        }
+        unsigned long long run = carry + block_exclusive_scan_1024(sum8, s_w, tot);
+#pragma unroll
+        for (int k = 0; k < PT; k++) {
+            const int j = base + (int)threadIdx.x * PT + k;
+            if (j < n_blocks) a.entry_scan[j] = run;
+            run += x[k];
+        }
         carry += tot;
     }
     if (threadIdx.x == 0) {
-        *total_out = carry;
-        if (total32_out) *total32_out = (uint32_t)carry;
-        if (max_total >= 0 && carry > (unsigned long long)max_total) set_status(c, GS_ERR_CAPACITY);
+        a.counters->n_entries = carry;
+        a.counters->n_entries32 = (uint32_t)carry;
     }
 }
 
-// ----------------------------------------------------------------------------------------
-// Entry compaction.  The projection leaves one bit word per view and 32 Gaussians (vis_bits,
-// each view padded to whole words).  A block of kEntryThreads threads covers as many words:
-// the count kernel writes the block's entry total; the totals are scanned; the compaction
-// kernel gives each word its offset by a block scan of the word counts, and each warp writes
-// the entries of 32 words, one word at a time with a lane per slot, so entries stay in (view,
-// index) order.  Blocks of 256 (four resident per SM) rather than 1024 (one, at the
-// compaction's registers) shorten the ragged end of the grid.
-// ----------------------------------------------------------------------------------------
-constexpr int kEntryThreads = 256;
-
-__global__ void __launch_bounds__(kEntryThreads) entry_count_kernel(const uint32_t* __restrict__ bits, int64_t n_words,
-                                                                   uint32_t* __restrict__ bsum) {
-    __shared__ uint32_t s[kEntryThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t word = (int64_t)blockIdx.x * kEntryThreads + threadIdx.x;
-    const uint32_t sum = warp_sum((uint32_t)__popc(word < n_words ? bits[word] : 0u));
-    if (lane == 0) s[w] = sum;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        uint32_t t = threadIdx.x < (kEntryThreads >> 5) ? s[threadIdx.x] : 0u;
-        t = warp_sum(t);
-        if (threadIdx.x == 0) bsum[blockIdx.x] = t;
-    }
-}
-
+template <int WPW, bool LOOKBACK>
 __global__ void __launch_bounds__(kEntryThreads, 4) entry_compact_kernel(BinArgs a, int64_t n_words) {
+    constexpr int WPB = WPW * kEntryWarps;   // words per block
     __shared__ uint32_t s[33];
-    __shared__ uint32_t s_off[kEntryThreads], s_word[kEntryThreads];
+    __shared__ uint32_t s_off[WPB], s_word[WPB];
+    __shared__ uint32_t s_base, s_chunk;
+    __shared__ uint32_t s_hist[kSortBins];
+    __shared__ bool s_ok;
+    static_assert(kEntryThreads == kSortBins, "a thread per digit");
     if (a.counters->status != 0) return;
-    const int64_t word = (int64_t)blockIdx.x * kEntryThreads + threadIdx.x;
-    const uint32_t b = word < n_words ? a.vis_bits[word] : 0u;
+    s_hist[threadIdx.x] = 0;
+    if (LOOKBACK) {
+        if (threadIdx.x == 0) s_chunk = atomicAdd(&a.tickets[0], 1u);
+        __syncthreads();
+    }
+    const int64_t chunk = LOOKBACK ? s_chunk : blockIdx.x, word = chunk * WPB + threadIdx.x;
+    const uint32_t b = (int)threadIdx.x < WPB && word < n_words ? a.vis_bits[word] : 0u;
     const uint32_t nw = (uint32_t)((a.n + 31) >> 5);   // words per view
     uint32_t tot;
-    const uint32_t off = block_exclusive_scan_1024((uint32_t)__popc(b), s, tot) + a.scan_tmp[blockIdx.x];
-    s_off[threadIdx.x] = off;
-    s_word[threadIdx.x] = b;
+    const uint32_t off = block_exclusive_scan_1024((uint32_t)__popc(b), s, tot);
+    if (!LOOKBACK) {
+        if (threadIdx.x == 0) {
+            s_base = (uint32_t)a.entry_scan[chunk];
+            s_ok = true;
+        }
+    } else if (threadIdx.x < 32) {
+        bool ok = true;
+        const unsigned long long before = lb_scan_warp(a.entry_scan, chunk, tot, a.counters, ok);
+        if (threadIdx.x == 0) {
+            s_base = (uint32_t)before;
+            s_ok = ok;
+            if (ok && chunk == gridDim.x - 1) {
+                a.counters->n_entries = before + tot;
+                a.counters->n_entries32 = (uint32_t)(before + tot);
+            }
+        }
+    }
+    if ((int)threadIdx.x < WPB) {
+        s_off[threadIdx.x] = off;
+        s_word[threadIdx.x] = b;
+    }
     __syncthreads();
+    if (!s_ok) return;
+    const uint32_t base = s_base;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t ltm;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(ltm));
     // four bit words per iteration: their record gathers are issued together
-    for (int k = 0; k < 32; k += 4) {
+    for (int k = 0; k < WPW; k += 4) {
         bool hit[4];
         float4 g0[4];
         int grx[4], gry[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const int lw = w * 32 + k + u;
+            const int lw = w * WPW + k + u;
             hit[u] = (s_word[lw] >> lane) & 1u;
-            const uint32_t gw = (uint32_t)blockIdx.x * kEntryThreads + lw;   // < V * nw
+            const uint32_t gw = (uint32_t)(chunk * WPB) + lw;   // < V * nw
             const uint32_t v = gw / nw;
             const uint32_t idx = v * (uint32_t)a.n + (gw - v * nw) * 32 + lane;
             if (hit[u]) {
@@ -137,11 +193,11 @@ __global__ void __launch_bounds__(kEntryThreads, 4) entry_compact_kernel(BinArgs
         }
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-            const int lw = w * 32 + k + u;
+            const int lw = w * WPW + k + u;
             const uint32_t bw = s_word[lw];
             if (hit[u]) {
-                const uint32_t pos = s_off[lw] + (uint32_t)__popc(bw & ltm);
-                const uint32_t gw = (uint32_t)blockIdx.x * kEntryThreads + lw;
+                const uint32_t pos = base + s_off[lw] + (uint32_t)__popc(bw & ltm);
+                const uint32_t gw = (uint32_t)(chunk * WPB) + lw;
                 const uint32_t v = gw / nw;
                 const uint32_t idx = v * (uint32_t)a.n + (gw - v * nw) * 32 + lane;
                 const float4 r0 = g0[u];
@@ -152,23 +208,40 @@ __global__ void __launch_bounds__(kEntryThreads, 4) entry_compact_kernel(BinArgs
                 int xa = 0, xb = 0, ya = 0, yb = 0;
                 tile_span(r0.x, rx, a.tile, V.tiles_x, xa, xb);
                 tile_span(r0.y, ry, a.tile, V.tiles_y, ya, yb);
-                a.ekeys[pos] = __float_as_uint(r0.z);   // z > 0: bits are monotone
+                const uint32_t zk = __float_as_uint(r0.z);   // z > 0: bits are monotone
+                a.ekeys[pos] = zk;
+                atomicAdd(&s_hist[zk & 255u], 1u);   // the depth sort's first digit
                 a.evals[pos] = pos;
                 a.entries[pos] = idx;
-                a.erect[pos] = make_uint2((uint32_t)(V.tile_off + ya * V.tiles_x + xa),
-                                          (uint32_t)(xb - xa + 1) | ((uint32_t)(yb - ya + 1) << 16));
+                a.erect[pos] = make_uint4((uint32_t)(V.tile_off + ya * V.tiles_x + xa),
+                                          (uint32_t)(xb - xa + 1) | ((uint32_t)(yb - ya + 1) << 16), idx, 0u);
             }
         }
     }
+    __syncthreads();
+    if (s_hist[threadIdx.x]) atomicAdd(&a.ehist[threadIdx.x], s_hist[threadIdx.x]);
+}
+
+size_t entry_scan_words(int64_t n, int n_views) {
+    return (size_t)(((int64_t)n_views * ((n + 31) >> 5) + kEntryMinWords - 1) / kEntryMinWords) + 1;
 }
 
 cudaError_t launch_entries(const BinArgs& a, cudaStream_t st) {
     const int64_t n_words = (int64_t)a.n_views * ((a.n + 31) >> 5);
-    const int nb = (int)((n_words + kEntryThreads - 1) / kEntryThreads);
-    if (nb > 0) entry_count_kernel<<<nb, kEntryThreads, 0, st>>>(a.vis_bits, n_words, a.scan_tmp);
-    scan_blocks_kernel<<<1, kScanThreads, 0, st>>>(a.scan_tmp, nb, &a.counters->n_entries, &a.counters->n_entries32,
-                                                   a.counters, -1);
-    if (nb > 0) entry_compact_kernel<<<nb, kEntryThreads, 0, st>>>(a, n_words);
+    if (n_words == 0) return cudaSuccess;
+    // the short form while its blocks fit the device a few times over (4 resident per SM)
+    const int64_t small = (n_words + kEntryMinWords - 1) / kEntryMinWords, sms = device_sms();
+    if (small <= 4 * sms) {
+        entry_compact_kernel<8, true><<<(unsigned)small, kEntryThreads, 0, st>>>(a, n_words);
+        return cudaGetLastError();
+    }
+    const int wpb = small <= 16 * sms ? kEntryMinWords : 32 * kEntryWarps;
+    const int nb = (int)((n_words + wpb - 1) / wpb);
+    entry_count_kernel<<<(unsigned)((n_words + kCountWords - 1) / kCountWords), kEntryThreads, 0, st>>>(a, n_words, wpb, nb);
+    if (wpb == kEntryMinWords)
+        entry_compact_kernel<8, false><<<nb, kEntryThreads, 0, st>>>(a, n_words);
+    else
+        entry_compact_kernel<32, false><<<nb, kEntryThreads, 0, st>>>(a, n_words);
     return cudaGetLastError();
 }
 
@@ -176,80 +249,105 @@ cudaError_t launch_entries(const BinArgs& a, cudaStream_t st) {
 // Pair emission from the depth-sorted entries: the tile counts of their rectangles, taken
 // in that order, are scanned into pair offsets (total = pair count), then each entry writes
 // one (global tile id, view * n + index) pair per covered tile, tiles in row-major order.
-// The rectangles and indices are read from the compact per-entry arrays of the compaction
-// (12 bytes an entry, which stay in L2), not from the projected records.
+// The rectangles and indices are read from the compact per-entry records of the compaction (16
+// bytes, one gather an entry), not from the projected records.
 // ----------------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t rect_count(uint2 r) { return (r.y & 0xFFFFu) * (r.y >> 16); }
 
-// The entry count is known only on the device, so the scans over the depth-sorted entries
-// cover the capacity (n_views * n) in chunks of kScanBlock entries, taken in turn by a grid of
-// resident blocks: a chunk past the last entry costs one store, not a block launch.
-//
-// Pair count of each chunk.  Also writes, in depth order, each entry's tile rectangle and
-// index (srt), which the offsets and the emission then read without the gather through the
-// sorted compact indices.
-__global__ void __launch_bounds__(kScanThreads) pair_count_kernel(BinArgs a, int nb) {
-    __shared__ uint32_t s[33];
-    const int64_t E = (int64_t)a.counters->n_entries;
-    const int64_t VN = (int64_t)a.n_views * a.n;
-    for (int ch = blockIdx.x; ch < nb; ch += gridDim.x) {
-        const int64_t base = (int64_t)ch * kScanBlock;
-        if (base >= E) {   // (the same for the whole block)
-            if (threadIdx.x == 0) a.scan_tmp[ch] = 0u;
-            continue;
-        }
-        uint32_t sum = 0;
+// Pair offsets of the depth-sorted entries (poff[e] = pairs of the entries before e), for every
+// output chunk of kEmitChunk pairs the entry holding its first pair, and each entry's tile
+// rectangle and index in depth order (srt), which the emission then reads without the gather
+// through the sorted compact indices.  The entry count is known only on the device: resident
+// blocks take chunks of kPairScanChunk entries in turn.
+__global__ void __launch_bounds__(kPairScanThreads) pair_offsets_kernel(BinArgs a) {
+    __shared__ uint32_t s[33], s_chunk;
+    __shared__ unsigned long long s_base;
+    __shared__ bool s_ok;
+    if (a.counters->status != 0) return;
+    const int64_t E = (int64_t)a.counters->n_entries, VN = (int64_t)a.n_views * a.n;
+    const int64_t n_chunks = (E + kPairScanChunk - 1) / kPairScanChunk;
+    const uint64_t emit_chunks = ((uint64_t)a.max_pairs + kEmitChunk - 1) / kEmitChunk;
+    for (;;) {
+        if (threadIdx.x == 0) s_chunk = atomicAdd(&a.tickets[1], 1u);
+        __syncthreads();
+        const int64_t ch = s_chunk;
+        if (ch >= n_chunks) return;
+        // thread t takes entries 4 t .. 4 t + 3 of the chunk
+        const int64_t e0 = ch * kPairScanChunk + (int64_t)threadIdx.x * kPairScanItems;
+        uint32_t c[kPairScanItems], t[kPairScanItems], sum = 0;
+        if (e0 + kPairScanItems <= E) {
+            const uint4 q = *reinterpret_cast<const uint4*>(a.sorted_evals + e0);
+            c[0] = q.x; c[1] = q.y; c[2] = q.z; c[3] = q.w;
+        } else {
 #pragma unroll
-        for (int k = 0; k < kScanItems; k++) {
-            const int64_t j = base + (int64_t)k * kScanThreads + threadIdx.x;
-            if (j < E) {
-                const uint32_t c = a.sorted_evals[j];
-                const uint2 r = a.erect[c];
-                a.srt[j] = r.x;
-                a.srt[VN + j] = r.y;
-                a.srt[2 * VN + j] = a.entries[c];
-                sum += rect_count(r);
+            for (int k = 0; k < kPairScanItems; k++) c[k] = e0 + k < E ? a.sorted_evals[e0 + k] : 0u;
+        }
+        uint4 r[kPairScanItems];   // one 16-byte gather an entry
+#pragma unroll
+        for (int k = 0; k < kPairScanItems; k++) r[k] = e0 + k < E ? a.erect[c[k]] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int k = 0; k < kPairScanItems; k++) {
+            t[k] = rect_count(make_uint2(r[k].x, r[k].y));
+            sum += t[k];
+            if (e0 + k < E) {
+                a.srt[e0 + k] = r[k].x;
+                a.srt[VN + e0 + k] = r[k].y;
+                a.srt[2 * VN + e0 + k] = r[k].z;
             }
         }
-        sum = warp_sum(sum);
-        if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = sum;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            uint32_t t = threadIdx.x < (kScanThreads >> 5) ? s[threadIdx.x] : 0u;
-            t = warp_sum(t);
-            if (threadIdx.x == 0) a.scan_tmp[ch] = t;
-        }
-        __syncthreads();   // s is written again for the next chunk
-    }
-}
-
-// Pair offsets of the depth-sorted entries (poff[e] = pairs of the entries before e), and
-// for every output chunk of kEmitChunk pairs the entry holding its first pair.
-__global__ void __launch_bounds__(kScanThreads) pair_offsets_kernel(BinArgs a, int nb) {
-    __shared__ uint32_t s[33];
-    if (a.counters->status != 0) return;
-    const int64_t E = (int64_t)a.counters->n_entries;
-    for (int ch = blockIdx.x; ch < nb && (int64_t)ch * kScanBlock < E; ch += gridDim.x) {
-        const int64_t base = (int64_t)ch * kScanBlock + (int64_t)threadIdx.x * kScanItems;
-        uint32_t t[kScanItems], sum = 0;
-#pragma unroll
-        for (int k = 0; k < kScanItems; k++) {
-            t[k] = base + k < E ? rect_count(make_uint2(0u, a.srt[(int64_t)a.n_views * a.n + base + k])) : 0u;
-            sum += t[k];
-        }
         uint32_t tot;
-        uint32_t off = block_exclusive_scan_1024(sum, s, tot) + a.scan_tmp[ch];   // (ends with a barrier)
+        const uint32_t local = block_exclusive_scan_1024(sum, s, tot);
+        if (threadIdx.x < 32) {
+            bool ok = true;
+            const unsigned long long before = lb_scan_warp(a.pair_scan, ch, tot, a.counters, ok);
+            if (threadIdx.x == 0) {
+                s_base = before;
+                s_ok = ok;
+                if (ok && ch == n_chunks - 1) {
+                    a.counters->n_pairs = before + tot;
+                    if (before + tot > (unsigned long long)a.max_pairs) set_status(a.counters, GS_ERR_CAPACITY);
+                }
+            }
+        }
+        __syncthreads();
+        if (!s_ok) return;
+        unsigned long long off = s_base + local;
 #pragma unroll
-        for (int k = 0; k < kScanItems; k++) {
-            if (base + k < E) {
-                a.poff[base + k] = off;
-                // chunk starts c * kEmitChunk inside [off, off + t)
-                for (uint32_t c = (off + kEmitChunk - 1) / kEmitChunk; c * (uint64_t)kEmitChunk < (uint64_t)off + t[k];
-                     c++)
-                    a.chunk_first[c] = (uint32_t)(base + k);
+        for (int k = 0; k < kPairScanItems; k++) {
+            if (e0 + k < E) {
+                a.poff[e0 + k] = (uint32_t)off;
+                // chunk starts c * kEmitChunk inside [off, off + t), of the chunks that exist
+                for (uint64_t m = (off + kEmitChunk - 1) / kEmitChunk; m < emit_chunks && m * kEmitChunk < off + t[k]; m++)
+                    a.chunk_first[m] = (uint32_t)(e0 + k);
             }
             off += t[k];
         }
+    }
+}
+
+size_t pair_scan_words(int64_t n, int n_views) { return (size_t)(((int64_t)n_views * n) / kPairScanChunk) + 2; }
+
+// Adds one to bin d of a shared histogram for every valid lane: once, with the count, where the
+// valid lanes share the digit -- the rule for a depth's or a tile id's upper digits -- instead of
+// 32 serial additions to one address.  All lanes of the warp call it.
+// hist_add_all: every lane is valid.
+__device__ __forceinline__ void hist_add_all(uint32_t* h, uint32_t d) {
+    const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
+    if (__all_sync(0xffffffffu, d == d0)) {
+        if ((threadIdx.x & 31) == 0) atomicAdd(&h[d0], 32u);
+    } else {
+        atomicAdd(&h[d], 1u);
+    }
+}
+__device__ __forceinline__ void hist_add(uint32_t* h, uint32_t d, bool valid) {
+    const uint32_t v = __ballot_sync(0xffffffffu, valid);
+    if (!v) return;
+    const int lead = __ffs(v) - 1;
+    const uint32_t d0 = __shfl_sync(0xffffffffu, d, lead);
+    if (__all_sync(0xffffffffu, !valid || d == d0)) {
+        if ((int)(threadIdx.x & 31) == lead) atomicAdd(&h[d0], (uint32_t)__popc(v));
+    } else if (valid) {
+        atomicAdd(&h[d], 1u);
     }
 }
 
@@ -265,7 +363,9 @@ __global__ void __launch_bounds__(kEmitThreads) pair_emit_kernel(BinArgs a) {
     __shared__ __align__(16) uint16_t s_own[kEmitChunk];   // slot -> local entry index
     __shared__ uint32_t s_wmax[kEmitThreads / 32];
     __shared__ uint16_t s_view_tx[GS_MAX_VIEWS];   // tiles per row of each view
+    __shared__ uint32_t s_hist[kSortMaxBins];      // the tile sort's first digit
     if (a.counters->status != 0) return;
+    for (int k = threadIdx.x; k < kSortMaxBins; k += kEmitThreads) s_hist[k] = 0;
     for (int v = threadIdx.x; v < a.n_views; v += blockDim.x) s_view_tx[v] = (uint16_t)a.views[v].tiles_x;
     const uint64_t P = a.counters->n_pairs;
     const int64_t E = (int64_t)a.counters->n_entries;
@@ -328,20 +428,25 @@ __global__ void __launch_bounds__(kEmitThreads) pair_emit_kernel(BinArgs a) {
             const uint32_t j = s_own[p - p0];
             const uint32_t kk = (uint32_t)p - s_off[j], wx = s_wx[j];
             const uint32_t ty = kk / wx, tx = kk - ty * wx;
-            a.pkeys[p] = s_t0[j] + ty * (uint32_t)s_tx[j] + tx;
+            const uint32_t tile = s_t0[j] + ty * (uint32_t)s_tx[j] + tx;
+            a.pkeys[p] = tile;
             a.pvals[p] = s_id[j];
+            if (a.phist_mask) atomicAdd(&s_hist[tile & a.phist_mask], 1u);
         }
         __syncthreads();
     }
+    __syncthreads();
+    for (int k = threadIdx.x; k < kSortMaxBins; k += kEmitThreads)
+        if (s_hist[k]) atomicAdd(&a.phist[k], s_hist[k]);
 }
 
 // Blocks of `kernel` resident on the device at once (occupancy times SMs), kept per device.
 template <class Kernel>
-static int resident_grid(int (&cache)[kMaxDevices], Kernel kernel, int threads) {
+static int resident_grid(int (&cache)[kMaxDevices], Kernel kernel, int threads, size_t smem = 0) {
     const int d = current_device();
     if (d >= 0 && cache[d] > 0) return cache[d];
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess || per_sm < 1)
         per_sm = 1;
     const int g = per_sm * device_sms();
     if (d >= 0) cache[d] = g;
@@ -349,18 +454,11 @@ static int resident_grid(int (&cache)[kMaxDevices], Kernel kernel, int threads) 
 }
 
 cudaError_t launch_emit(const BinArgs& a, cudaStream_t st) {
-    static int g_count[kMaxDevices] = {}, g_offsets[kMaxDevices] = {}, g_emit[kMaxDevices] = {};
-    const int64_t total = (int64_t)a.n_views * a.n;   // upper bound of the entry count
-    const int nb = (int)((total + kScanBlock - 1) / kScanBlock);
+    static int g_offsets[kMaxDevices] = {}, g_emit[kMaxDevices] = {};
+    const int64_t nb = ((int64_t)a.n_views * a.n + kPairScanChunk - 1) / kPairScanChunk;   // at most
     if (nb > 0) {
-        const int g = resident_grid(g_count, pair_count_kernel, kScanThreads);
-        pair_count_kernel<<<g < nb ? g : nb, kScanThreads, 0, st>>>(a, nb);
-    }
-    scan_blocks_kernel<<<1, kScanThreads, 0, st>>>(a.scan_tmp, nb, &a.counters->n_pairs, nullptr, a.counters,
-                                                   a.max_pairs);
-    if (nb > 0) {
-        const int g = resident_grid(g_offsets, pair_offsets_kernel, kScanThreads);
-        pair_offsets_kernel<<<g < nb ? g : nb, kScanThreads, 0, st>>>(a, nb);
+        const int64_t g = resident_grid(g_offsets, pair_offsets_kernel, kPairScanThreads);
+        pair_offsets_kernel<<<(unsigned)(g < nb ? g : nb), kPairScanThreads, 0, st>>>(a);
     }
     // one chunk of kEmitChunk pairs per block and turn; the pair count is known only on the
     // device, so the grid is the resident one (capped by the capacity's chunks)
@@ -376,17 +474,8 @@ cudaError_t launch_emit(const BinArgs& a, cudaStream_t st) {
 // ----------------------------------------------------------------------------------------
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kItemsPerWarp = kSortChunk / kSortWarps;   // 512
-constexpr int kUpThreads = 512;                          // upsweep block (same chunk range, more warps)
-constexpr int kUpWarps = kUpThreads / 32;
-constexpr int kUpItems = kSortChunk / kUpThreads;        // 8
-
-__device__ __forceinline__ void chunk_span(unsigned long long count, int grid, int b, int64_t& lo, int64_t& hi) {
-    const int64_t P = (int64_t)count;
-    const int64_t nch = (P + kSortChunk - 1) / kSortChunk;
-    const int64_t c0 = nch * b / grid, c1 = nch * (b + 1) / grid;
-    lo = c0 * kSortChunk;
-    hi = min(c1 * kSortChunk, P);
-}
+constexpr int kHistThreads = 512;
+constexpr int kHistItems = kSortChunk / kHistThreads;    // 8
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
     uint32_t m;
@@ -401,70 +490,29 @@ __device__ __forceinline__ uint32_t digit_of(K k, int shift, uint32_t mask) {
     return (uint32_t)(k >> shift) & ((1u << BITS) - 1u) & mask;
 }
 
-// Per-block digit histograms over the block's chunks: every thread loads its kUpItems keys of
-// a chunk first, then adds them to its warp's private histogram with shared-memory atomics.
-template <typename K, int BITS>
-__global__ void __launch_bounds__(kUpThreads) sort_upsweep_kernel(SortArgs a, int in_buf, int shift) {
-    constexpr int BINS = 1 << BITS;
-    __shared__ uint32_t h[kUpWarps][BINS];
+// Digit counts of one pass of 8-bit digits (a sort whose keys no kernel of the library counts).
+__global__ void __launch_bounds__(kHistThreads) sort_count_kernel(SortArgs a, int shift) {
+    __shared__ uint32_t h[kSortBins];
     if (a.counters->status != 0) return;
-    for (int t = threadIdx.x; t < kUpWarps * BINS; t += blockDim.x) (&h[0][0])[t] = 0;
+    const int64_t count = (int64_t)*a.count;
+    for (int t = threadIdx.x; t < kSortBins; t += kHistThreads) h[t] = 0;
     __syncthreads();
-    int64_t lo, hi;
-    chunk_span(*a.count, a.grid, blockIdx.x, lo, hi);
-    const K* keys = static_cast<const K*>(in_buf ? a.keys[1] : a.keys[0]);
-    uint32_t* hw = h[threadIdx.x >> 5];
-    for (int64_t base = lo; base < hi; base += kSortChunk) {
-        K k[kUpItems];
+    const unsigned long long* keys = static_cast<const unsigned long long*>(a.keys[0]);
+    for (int64_t base = (int64_t)blockIdx.x * kSortChunk; base < count; base += (int64_t)gridDim.x * kSortChunk) {
+        unsigned long long k[kHistItems];
 #pragma unroll
-        for (int j = 0; j < kUpItems; j++) {
-            const int64_t idx = base + (int64_t)j * kUpThreads + threadIdx.x;
-            k[j] = idx < hi ? keys[idx] : (K)0;
+        for (int j = 0; j < kHistItems; j++) {
+            const int64_t i = base + (int64_t)j * kHistThreads + threadIdx.x;
+            k[j] = i < count ? keys[i] : 0ull;
         }
 #pragma unroll
-        for (int j = 0; j < kUpItems; j++) {
-            const int64_t idx = base + (int64_t)j * kUpThreads + threadIdx.x;
-            if (idx < hi) atomicAdd(&hw[digit_of<BITS>(k[j], shift, a.digit_mask)], 1u);
-        }
+        for (int j = 0; j < kHistItems; j++)
+            hist_add(h, (uint32_t)(k[j] >> shift) & 255u & a.digit_mask,
+                     base + (int64_t)j * kHistThreads + threadIdx.x < count);
     }
     __syncthreads();
-    for (int d = threadIdx.x; d < BINS; d += blockDim.x) {
-        uint32_t s = 0;
-#pragma unroll
-        for (int w = 0; w < kUpWarps; w++) s += h[w][d];
-        a.hist[(int64_t)d * a.grid + blockIdx.x] = s;
-    }
-}
-
-// One warp per digit: exclusive prefix of the digit's block counts (in place) and the
-// digit total.  8 warps per block.
-__global__ void __launch_bounds__(256) sort_scan_kernel(SortArgs a) {
-    if (a.counters->status != 0) return;
-    const int lane = threadIdx.x & 31;
-    const int d = blockIdx.x * 8 + (threadIdx.x >> 5);
-    uint32_t* row = a.hist + (int64_t)d * a.grid;
-    constexpr int C = kSortMaxGrid / 32;
-    uint32_t x[C];
-#pragma unroll
-    for (int c = 0; c < C; c++) {
-        const int b = c * 32 + lane;
-        x[c] = b < a.grid ? row[b] : 0u;
-    }
-    uint32_t carry = 0;
-#pragma unroll
-    for (int c = 0; c < C; c++) {
-        if (c * 32 >= a.grid) break;
-        uint32_t inc = x[c];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        const int b = c * 32 + lane;
-        if (b < a.grid) row[b] = carry + inc - x[c];
-        carry += __shfl_sync(0xffffffffu, inc, 31);
-    }
-    if (lane == 0) a.digit_tot[d] = carry;
+    for (int t = threadIdx.x; t < kSortBins; t += kHistThreads)
+        if (h[t]) atomicAdd(&a.hist[t], h[t]);
 }
 
 // Digit-indexed shared arrays are stored at dix(d) = d with its low 5 bits XORed with the next
@@ -483,10 +531,12 @@ struct SortSmem {
     K keys[kSortChunk + kSortChunk / 32];
     uint32_t vals[kSortChunk + kSortChunk / 32];
     uint32_t wcnt[kSortWarps][BINS];
-    uint32_t run[BINS];
-    uint32_t tot[BINS];
+    uint32_t run[BINS];      // next output position of each digit
+    uint32_t gpos[BINS];     // the same for the chunk being written, less cstart
     uint32_t cstart[BINS];
+    uint32_t next[kSortMaxBins];   // digit counts: of the block's run, then of the next pass
     uint32_t scan_w[33];
+    uint32_t ticket;
 };
 
 // Exclusive scan of DPT consecutive values per thread over the block (kSortThreads threads);
@@ -526,42 +576,94 @@ __device__ __forceinline__ void block_exclusive_scan_dpt(const uint32_t (&x)[DPT
     __syncthreads();
 }
 
-// resident downsweep blocks per SM (and the grid of every sort pass: this many per SM)
-constexpr int kSortBlocksPerSM = 3;   // (2 and 4 measured slower on GB300)
+constexpr int kSortBlocksPerSM = kSortThreads == 256 ? 3 : 2;
 
+// Blocks of a pass: at most the resident ones, which bounds the look-back.
+static int sort_grid(int64_t capacity) {
+    int64_t g = (int64_t)device_sms() * kSortBlocksPerSM;
+    if (g > kSortMaxGrid) g = kSortMaxGrid;
+    const int64_t chunks = sort_chunks(capacity);
+    return (int)(chunks < 1 ? 1 : (chunks < g ? chunks : g));
+}
+
+constexpr int kLbBatch = 8;   // look-back words loaded at a time
+
+// Sum of the words col[j << bits], j = last, last - 1, ..., first, up to and including the first
+// that holds an inclusive prefix (state 2).  ok is cleared if a wait gave up.
+template <typename W>
+__device__ __forceinline__ uint32_t lb_sum(const W* col, int bits, int64_t last, int64_t first, uint32_t tag,
+                                           const Counters* c, bool& ok) {
+    uint32_t sum = 0;
+    int spin = 0;
+    for (int64_t j = last; j >= first && ok; j -= kLbBatch) {
+        W wd[kLbBatch];
+#pragma unroll
+        for (int u = 0; u < kLbBatch; u++) wd[u] = j - u >= first ? lb_load(col + ((size_t)(j - u) << bits)) : (W)0;
+        bool full = false;
+#pragma unroll
+        for (int u = 0; u < kLbBatch; u++) {
+            if (full || j - u < first || !ok) continue;
+            uint32_t st = lb_state(wd[u], tag);
+            while (st == 0) {
+                if (++spin > kLbSpin || ((spin & 1023) == 0 && *(const volatile uint32_t*)&c->status != 0)) {
+                    ok = false;
+                    break;
+                }
+                wd[u] = lb_load(col + ((size_t)(j - u) << bits));
+                st = lb_state(wd[u], tag);
+            }
+            if (!ok) continue;
+            sum += (uint32_t)lb_value(wd[u]);
+            full = st == 2;
+        }
+        if (full) break;
+    }
+    return sum;
+}
+
+// One pass.  Block t (in ticket order, so that the blocks it waits for are running) owns a
+// contiguous run of chunks.  It counts the run's digits and publishes them, ranks its first chunk,
+// and then sums the counts of the blocks before it (a thread per digit), by when those mostly are
+// there; then it scatters its chunks one after another.  Blocks form groups of kSortGroup whose
+// last block publishes the group's counts and then its inclusive prefix, so that a block reads
+// at most 15 + grid / 16 words a digit: reading the words of every block in flight instead took
+// most of the pass.  At 7k / 356k / 1.9M entries a pass takes 9 / 12 / 27 us, at 8.7M pairs 77 to 90
+// (separate kernels: 20 / 26 / 38, 76).  (Chunks dealt out one by one, each with a look-back of its own, lose at large
+// counts: a look-back step is about a microsecond across the two dies, 85 against 60 us a pass at
+// 8.7M pairs.)  The next pass's digits are counted on the way out.
 template <typename K, int BITS>
-__global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSM) sort_downsweep_kernel(SortArgs a, int in_buf, int shift) {
+__global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSM)
+    sort_pass_kernel(SortArgs a, int in_buf, int shift, int pass, int next_shift, uint32_t next_mask) {
     constexpr int BINS = 1 << BITS;
-    constexpr int DPT = BINS / kSortThreads;   // digits per thread: 1 or 2
-    static_assert(DPT * kSortThreads == BINS, "whole digits per thread");
+    constexpr int DPT = (BINS + kSortThreads - 1) / kSortThreads;   // digits per thread
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem<K, BITS>& S = *reinterpret_cast<SortSmem<K, BITS>*>(smem_raw);
     if (a.counters->status != 0) return;
-    int64_t lo, hi;
-    chunk_span(*a.count, a.grid, blockIdx.x, lo, hi);
+    const int64_t count = (int64_t)*a.count, nch = sort_chunks(count);
+    if (threadIdx.x == 0) S.ticket = atomicAdd(&a.tickets[pass], 1u);
+    for (int t = threadIdx.x; t < kSortMaxBins; t += kSortThreads) S.next[t] = 0;
     // (selects, not a runtime index into the parameter arrays, which would go to local memory)
     const K* kin = static_cast<const K*>(in_buf ? a.keys[1] : a.keys[0]);
     const uint32_t* vin = in_buf ? a.vals[1] : a.vals[0];
     K* kout = static_cast<K*>(in_buf ? a.keys[0] : a.keys[1]);
     uint32_t* vout = in_buf ? a.vals[0] : a.vals[1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int d0 = threadIdx.x * DPT;   // this thread's digits d0 .. d0 + DPT - 1
+    const int d0 = threadIdx.x * DPT;   // this thread's digits d0 .. d0 + DPT - 1 (if below BINS)
+    const uint32_t tag = a.tag + (uint32_t)pass;
+    uint32_t dbase[DPT];                // first output position of each digit
     {
-        // start of this block's run of each digit: digit offset + count in earlier blocks
-        uint32_t x[DPT], ex[DPT];
+        uint32_t x[DPT];
 #pragma unroll
-        for (int q = 0; q < DPT; q++) x[q] = a.digit_tot[d0 + q];
-        block_exclusive_scan_dpt<DPT>(x, ex, S.scan_w);
-#pragma unroll
-        for (int q = 0; q < DPT; q++) S.run[dix(d0 + q)] = ex[q] + a.hist[(int64_t)(d0 + q) * a.grid + blockIdx.x];
+        for (int q = 0; q < DPT; q++) x[q] = d0 + q < BINS ? a.hist[pass * kSortMaxBins + d0 + q] : 0u;
+        block_exclusive_scan_dpt<DPT>(x, dbase, S.scan_w);   // (begins and ends with barriers)
     }
+    const int64_t blocks = nch < gridDim.x ? nch : gridDim.x, t = S.ticket;
+    if (t >= blocks) return;   // (the same for the whole block)
+    const int64_t lo = nch * t / blocks * kSortChunk, end = nch * (t + 1) / blocks * kSortChunk, hi = end < count ? end : count;
     const uint32_t ltm = lanemask_lt();
-    for (int64_t base = lo; base < hi; base += kSortChunk) {
-        const int m = (int)(hi - base < kSortChunk ? hi - base : kSortChunk);
-        for (int t = threadIdx.x; t < kSortWarps * BINS; t += blockDim.x) (&S.wcnt[0][0])[t] = 0;
-        K key[kSortItems];
-        uint32_t val[kSortItems];
-        uint32_t rank[kSortItems];
+    K key[kSortItems];
+    uint32_t val[kSortItems];
+    auto load = [&](int64_t base, int m) {
         // all loads first: the chunk's reads are in flight together
 #pragma unroll
         for (int j = 0; j < kSortItems; j++) {
@@ -570,116 +672,206 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSM) sort_downsweep
             key[j] = valid ? kin[base + item] : (K)0;
             val[j] = valid ? vin[base + item] : 0u;
         }
+    };
+    auto chunk_size = [&](int64_t base) { return (int)(hi - base < kSortChunk ? hi - base : kSortChunk); };
+    // the digits of the run, two chunks' keys in flight at a time (of a single chunk, from the
+    // registers it is ranked from below)
+    if (hi - lo > kSortChunk) {
+        for (int64_t base = lo; base < hi; base += 2 * kSortChunk) {
+            K k[2][kSortItems];
+#pragma unroll
+            for (int j = 0; j < 2 * kSortItems; j++) {
+                const int64_t i = base + (int64_t)j * kSortThreads + threadIdx.x;
+                k[j / kSortItems][j % kSortItems] = i < hi ? kin[i] : (K)0;
+            }
+            if (base + 2 * kSortChunk <= hi) {
+#pragma unroll
+                for (int j = 0; j < 2 * kSortItems; j++)
+                    hist_add_all(S.next, digit_of<BITS>(k[j / kSortItems][j % kSortItems], shift, a.digit_mask));
+            } else {
+#pragma unroll
+                for (int j = 0; j < 2 * kSortItems; j++)
+                    hist_add(S.next, digit_of<BITS>(k[j / kSortItems][j % kSortItems], shift, a.digit_mask),
+                             base + (int64_t)j * kSortThreads + threadIdx.x < hi);
+            }
+        }
+    }
+    load(lo, chunk_size(lo));
+    if (hi - lo <= kSortChunk) {
+#pragma unroll
+        for (int j = 0; j < kSortItems; j++)
+            hist_add(S.next, digit_of<BITS>(key[j], shift, a.digit_mask), w * kItemsPerWarp + j * 32 + lane < chunk_size(lo));
+    }
+    __syncthreads();
+    lbword* const groups = a.lookback;
+    uint32_t* const words = reinterpret_cast<uint32_t*>(groups + kSortGroupBytes / sizeof(lbword));
+    uint32_t mine[DPT];
+#pragma unroll
+    for (int q = 0; q < DPT; q++) {
+        if (d0 + q >= BINS) continue;
+        mine[q] = S.next[d0 + q];
+        lb_store(words + ((size_t)t << BITS) + d0 + q, tag, 1, mine[q]);
+        S.next[d0 + q] = 0;
+    }
+    bool ok = true;
+    for (int64_t base = lo; base < hi; base += kSortChunk) {
+        const int m = chunk_size(base);
+        for (int k = threadIdx.x; k < kSortWarps * BINS; k += kSortThreads) (&S.wcnt[0][0])[k] = 0;
+        if (base != lo) load(base, m);
+        uint32_t rank[kSortItems / 2];   // two 16-bit ranks a word
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < kSortItems; j++) {
             const int item = w * kItemsPerWarp + j * 32 + lane;
             const bool valid = item < m;
-            const uint32_t d = valid ? digit_of<BITS>(key[j], shift, a.digit_mask) : (uint32_t)BINS;
+            const uint32_t dg = valid ? digit_of<BITS>(key[j], shift, a.digit_mask) : (uint32_t)BINS;
             // lanes holding the same digit: one ballot per digit bit, and one for validity (a
             // fixed cost; __match_any_sync is slower when a warp holds many distinct digits)
             uint32_t peers = __ballot_sync(0xffffffffu, valid);
             if (!valid) peers = ~peers;
 #pragma unroll
             for (int bit = 0; bit < BITS; bit++) {
-                const bool set = (d >> bit) & 1u;
+                const bool set = (dg >> bit) & 1u;
                 const uint32_t bb = __ballot_sync(0xffffffffu, set);
                 peers &= set ? bb : ~bb;
             }
             uint32_t r = __popc(peers & ltm);
-            if (valid) r += S.wcnt[w][dix(d)];
+            if (valid) r += S.wcnt[w][dix(dg)];
             __syncwarp();
-            if (valid && lane == 31 - __clz(peers)) S.wcnt[w][dix(d)] += __popc(peers);
+            if (valid && lane == 31 - __clz(peers)) S.wcnt[w][dix(dg)] += __popc(peers);
             __syncwarp();
-            rank[j] = r;
+            rank[j / 2] = j % 2 ? rank[j / 2] | r << 16 : r;
         }
         __syncthreads();
-        {
-            // per digit: prefix over warps and the chunk total, then the chunk's digit starts
-            uint32_t tot[DPT], cs[DPT];
+        // per digit: prefix over warps and the chunk total, then the chunk's digit starts
+        uint32_t tot[DPT], cs[DPT];
 #pragma unroll
-            for (int q = 0; q < DPT; q++) {
-                uint32_t run = 0;
+        for (int q = 0; q < DPT; q++) {
+            tot[q] = 0;
+            if (d0 + q >= BINS) continue;
 #pragma unroll
-                for (int ww = 0; ww < kSortWarps; ww++) {
-                    const uint32_t c = S.wcnt[ww][dix(d0 + q)];
-                    S.wcnt[ww][dix(d0 + q)] = run;
-                    run += c;
-                }
-                tot[q] = run;
-                S.tot[dix(d0 + q)] = run;
+            for (int ww = 0; ww < kSortWarps; ww++) {
+                const uint32_t c = S.wcnt[ww][dix(d0 + q)];
+                S.wcnt[ww][dix(d0 + q)] = tot[q];
+                tot[q] += c;
             }
-            block_exclusive_scan_dpt<DPT>(tot, cs, S.scan_w);
-#pragma unroll
-            for (int q = 0; q < DPT; q++) S.cstart[dix(d0 + q)] = cs[q];
         }
+        block_exclusive_scan_dpt<DPT>(tot, cs, S.scan_w);
+#pragma unroll
+        for (int q = 0; q < DPT; q++)
+            if (d0 + q < BINS) S.cstart[dix(d0 + q)] = cs[q];
         __syncthreads();
 #pragma unroll
         for (int j = 0; j < kSortItems; j++) {
             const int item = w * kItemsPerWarp + j * 32 + lane;
             if (item < m) {
-                const uint32_t d = digit_of<BITS>(key[j], shift, a.digit_mask);
-                const int pos = skew((int)(S.cstart[dix(d)] + S.wcnt[w][dix(d)] + rank[j]));
+                const uint32_t dg = digit_of<BITS>(key[j], shift, a.digit_mask);
+                const int pos = skew((int)(S.cstart[dix(dg)] + S.wcnt[w][dix(dg)] + (rank[j / 2] >> (16 * (j % 2)) & 0xFFFFu)));
                 S.keys[pos] = key[j];
                 S.vals[pos] = val[j];
             }
         }
-        __syncthreads();
-        for (int k = threadIdx.x; k < m; k += blockDim.x) {
-            const K kk = S.keys[skew(k)];
-            const uint32_t d = digit_of<BITS>(kk, shift, a.digit_mask);
-            const int64_t g = (int64_t)S.run[dix(d)] + (k - (int)S.cstart[dix(d)]);
-            kout[g] = kk;
-            vout[g] = S.vals[skew(k)];
+        if (base == lo) {
+            // counts of the blocks before this one: those of its group, then the groups before
+            const int64_t g = t / kSortGroup;
+            const bool last = t % kSortGroup == kSortGroup - 1;
+#pragma unroll
+            for (int q = 0; q < DPT; q++) {
+                const int d = d0 + q;
+                if (d >= BINS) continue;
+                uint32_t before = lb_sum(words + d, BITS, t - 1, g * kSortGroup, tag, a.counters, ok);
+                if (last && ok)
+                    lb_store(groups + ((size_t)g << BITS) + d, tag, g == 0 ? 2u : 1u, (unsigned long long)(before + mine[q]));
+                if (g > 0 && ok) {
+                    before += lb_sum(groups + d, BITS, g - 1, 0, tag, a.counters, ok);
+                    if (last && ok) lb_store(groups + ((size_t)g << BITS) + d, tag, 2, (unsigned long long)(before + mine[q]));
+                }
+                S.run[d] = dbase[q] + before;
+            }
+            if (__syncthreads_or(!ok)) {
+                if (threadIdx.x == 0) set_status(a.counters, GS_ERR_TIMEOUT);
+                return;
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < DPT; q++) {
+            if (d0 + q >= BINS) continue;
+            const uint32_t r = S.run[d0 + q];
+            S.gpos[dix(d0 + q)] = r - cs[q];
+            S.run[d0 + q] = r + tot[q];
         }
         __syncthreads();
-#pragma unroll
-        for (int q = 0; q < DPT; q++) S.run[dix(d0 + q)] += S.tot[dix(d0 + q)];
+        auto put = [&](int k) {
+            const K kk = S.keys[skew(k)];
+            const uint32_t g = S.gpos[dix(digit_of<BITS>(kk, shift, a.digit_mask))] + (uint32_t)k;   // (mod 2^32)
+            kout[g] = kk;
+            vout[g] = S.vals[skew(k)];
+            return kk;
+        };
+        if (m == kSortChunk) {
+#pragma unroll 4
+            for (int k = threadIdx.x; k < kSortChunk; k += kSortThreads) {
+                const K kk = put(k);
+                if (next_mask) hist_add_all(S.next, (uint32_t)(kk >> next_shift) & next_mask);
+            }
+        } else {
+            for (int k0 = 0; k0 < m; k0 += kSortThreads) {
+                const int k = k0 + (int)threadIdx.x;
+                K kk = 0;
+                if (k < m) kk = put(k);
+                if (next_mask) hist_add(S.next, (uint32_t)(kk >> next_shift) & next_mask, k < m);
+            }
+        }
+        __syncthreads();
     }
-}
-
-static int g_sort_grid[kMaxDevices] = {};
-int sort_grid() {
-    const int d = current_device();
-    if (d >= 0 && g_sort_grid[d] > 0) return g_sort_grid[d];
-    const int g = device_sms() * kSortBlocksPerSM;
-    const int grid = g < kSortMaxGrid ? g : kSortMaxGrid;
-    if (d >= 0) g_sort_grid[d] = grid;
-    return grid;
+    if (next_mask)
+        for (int k = threadIdx.x; k < kSortMaxBins; k += kSortThreads)
+            if (S.next[k]) atomicAdd(&a.hist[(pass + 1) * kSortMaxBins + k], S.next[k]);
 }
 
 // One pass (in_buf -> in_buf ^ 1) with BITS-bit digits at `shift`.
 template <typename K, int BITS>
-static cudaError_t launch_pass(const SortArgs& a, int in_buf, int shift, cudaStream_t st) {
+static cudaError_t launch_pass(const SortArgs& a, int in_buf, int shift, int pass, int next_shift, uint32_t next_mask,
+                               cudaStream_t st) {
     static bool attr_set[kMaxDevices] = {};
     const size_t smem = sizeof(SortSmem<K, BITS>);
-    if (a.grid < 1 || a.grid > kSortMaxGrid) return cudaErrorInvalidValue;
     cudaError_t e = once_per_device(attr_set, [&] {
-        return cudaFuncSetAttribute(sort_downsweep_kernel<K, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem);
+        return cudaFuncSetAttribute(sort_pass_kernel<K, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
-    sort_upsweep_kernel<K, BITS><<<a.grid, kUpThreads, 0, st>>>(a, in_buf, shift);
-    sort_scan_kernel<<<(1 << BITS) / 8, 256, 0, st>>>(a);
-    sort_downsweep_kernel<K, BITS><<<a.grid, kSortThreads, smem, st>>>(a, in_buf, shift);
+    sort_pass_kernel<K, BITS><<<sort_grid(a.capacity), kSortThreads, smem, st>>>(a, in_buf, shift, pass, next_shift,
+                                                                              next_mask);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sort32(const SortArgs& a, int n_passes, const int* shifts, const int* bits, cudaStream_t st) {
+template <typename K>
+static cudaError_t launch_passes(const SortArgs& a, int n_passes, const int* shifts, const int* bits, cudaStream_t st) {
+    if (n_passes > kSortMaxPasses) return cudaErrorInvalidValue;
     for (int p = 0; p < n_passes; p++) {
-        const cudaError_t e = bits[p] == 9 ? launch_pass<uint32_t, 9>(a, p & 1, shifts[p], st)
-                                           : launch_pass<uint32_t, 8>(a, p & 1, shifts[p], st);
+        const bool more = p + 1 < n_passes;
+        const int ns = more ? shifts[p + 1] : 0;
+        const uint32_t nm = more ? ((1u << bits[p + 1]) - 1u) & a.digit_mask : 0u;
+        cudaError_t e = cudaErrorInvalidValue;
+        if (bits[p] == 8) e = launch_pass<K, 8>(a, p & 1, shifts[p], p, ns, nm, st);
+        if constexpr (sizeof(K) == 4)
+            if (bits[p] == 9) e = launch_pass<K, 9>(a, p & 1, shifts[p], p, ns, nm, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
+cudaError_t launch_sort32(const SortArgs& a, int n_passes, const int* shifts, const int* bits, cudaStream_t st) {
+    return launch_passes<uint32_t>(a, n_passes, shifts, bits, st);
+}
+
 cudaError_t launch_sort64(const SortArgs& a, int n_passes, const int* shifts, cudaStream_t st) {
-    for (int p = 0; p < n_passes; p++) {
-        const cudaError_t e = launch_pass<unsigned long long, 8>(a, p & 1, shifts[p], st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    const int bits[kSortMaxPasses] = {8, 8, 8, 8, 8, 8, 8, 8};
+    return launch_passes<unsigned long long>(a, n_passes, shifts, bits, st);
+}
+
+cudaError_t launch_sort_count64(const SortArgs& a, int shift, cudaStream_t st) {
+    sort_count_kernel<<<sort_grid(a.capacity), kHistThreads, 0, st>>>(a, shift);
+    return cudaGetLastError();
 }
 
 // ----------------------------------------------------------------------------------------
@@ -722,7 +914,7 @@ __global__ void __launch_bounds__(256) ranges_kernel(RangeArgs a) {
 
 cudaError_t launch_ranges(const RangeArgs& a, int n_tiles, cudaStream_t st) {
     (void)n_tiles;
-    ranges_kernel<<<sort_grid() * 4, 256, 0, st>>>(a);
+    ranges_kernel<<<device_sms() * 12, 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -731,15 +923,16 @@ cudaError_t launch_ranges(const RangeArgs& a, int n_tiles, cudaStream_t st) {
 // power-of-two buckets (bucket b holds counts in [2^(b-1), 2^b)), so that the largest tiles
 // are scheduled first and the tail of the launch is made of short items.
 // ----------------------------------------------------------------------------------------
-constexpr int kOrderBuckets = 34;
-
 __device__ __forceinline__ int order_bucket(uint2 r) {
     const uint32_t c = r.y - r.x;
     return c ? 33 - __clz(c) : 0;   // 0 = empty, 1..33
 }
 
-__global__ void tile_order_hist_kernel(const uint2* ranges, int n_tiles, uint32_t* cnt, const Counters* c) {
+// Bucket counts; the last block to finish turns them into the buckets' first positions, largest
+// counts first (tmp: counts, then positions, then the blocks done).
+__global__ void tile_order_hist_kernel(const uint2* ranges, int n_tiles, uint32_t* tmp, const Counters* c) {
     __shared__ uint32_t h[kOrderBuckets];
+    __shared__ bool last;
     for (int b = threadIdx.x; b < kOrderBuckets; b += blockDim.x) h[b] = 0;
     __syncthreads();
     if (c->status == 0)
@@ -747,16 +940,21 @@ __global__ void tile_order_hist_kernel(const uint2* ranges, int n_tiles, uint32_
             atomicAdd(&h[order_bucket(ranges[t])], 1u);
     __syncthreads();
     for (int b = threadIdx.x; b < kOrderBuckets; b += blockDim.x)
-        if (h[b]) atomicAdd(&cnt[b], h[b]);
-}
-
-// cursor[b] = number of items in buckets above b (largest counts first)
-__global__ void tile_order_scan_kernel(const uint32_t* cnt, uint32_t* cursor) {
-    if (threadIdx.x != 0) return;
-    uint32_t run = 0;
-    for (int b = kOrderBuckets - 1; b >= 0; b--) {
-        cursor[b] = run;
-        run += cnt[b];
+        if (h[b]) atomicAdd(&tmp[b], h[b]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&tmp[2 * kOrderBuckets], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int b = threadIdx.x; b < kOrderBuckets; b += blockDim.x) h[b] = __ldcg(&tmp[b]);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t run = 0;
+        for (int b = kOrderBuckets - 1; b >= 0; b--) {
+            tmp[kOrderBuckets + b] = run;
+            run += h[b];
+        }
     }
 }
 
@@ -780,11 +978,8 @@ __global__ void tile_order_scatter_kernel(const uint2* ranges, int n_tiles, uint
 cudaError_t launch_tile_order(const uint2* ranges, int n_tiles, uint32_t* order, uint32_t* tmp, const Counters* c,
                               cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(tmp, 0, sizeof(uint32_t) * 2 * kOrderBuckets, st);
-    if (e != cudaSuccess) return e;
     const int blocks = (n_tiles + 255) / 256 < 1024 ? (n_tiles + 255) / 256 : 1024;
     tile_order_hist_kernel<<<blocks, 256, 0, st>>>(ranges, n_tiles, tmp, c);
-    tile_order_scan_kernel<<<1, 32, 0, st>>>(tmp, tmp + kOrderBuckets);
     tile_order_scatter_kernel<<<blocks, 256, 0, st>>>(ranges, n_tiles, tmp + kOrderBuckets, order, c);
     return cudaGetLastError();
 }

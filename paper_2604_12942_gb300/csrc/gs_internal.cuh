@@ -14,13 +14,18 @@ constexpr float kLn2 = 0.69314718055994530942f;
 constexpr float kLog2e = 1.44269504088896340736f;
 constexpr int kSortBins = 256;                    // 8-bit digits (64-bit keys)
 constexpr int kSortMaxBins = 512;                 // up to 9-bit digits (32-bit keys)
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;                     // per thread per chunk
+constexpr int kSortThreads = 512;
+constexpr int kSortItems = 8;                      // per thread per chunk
+constexpr int kSortGroup = 16;                     // blocks per look-back group
+constexpr int kSortMaxGrid = 512;                  // blocks of a sort pass (at most)
 constexpr int kSortChunk = kSortThreads * kSortItems;
-constexpr int kSortMaxGrid = 512;                 // blocks of a sort pass (at most)
-constexpr int kScanThreads = 1024;
-constexpr int kScanItems = 4;
-constexpr int kScanBlock = kScanThreads * kScanItems;
+constexpr int kSortMaxPasses = 8;
+__host__ __device__ __forceinline__ int64_t sort_chunks(int64_t n) { return (n + kSortChunk - 1) / kSortChunk; }
+constexpr int kPairScanThreads = 512;
+constexpr int kPairScanItems = 4;                 // depth-sorted entries per thread
+constexpr int kPairScanChunk = kPairScanThreads * kPairScanItems;
+constexpr int kEntryMinWords = 64;                // visibility words per block of the compaction (at least)
+constexpr int kOrderBuckets = 34;                 // tile_order: power-of-two pair counts
 constexpr int kEmitThreads = 256;
 constexpr int kEmitChunk = 2048;                  // pairs per chunk of the balanced emission
 
@@ -406,6 +411,98 @@ __device__ __forceinline__ void project_view(const float* mu, const Cov3& cv, fl
     P.u = V.fx * x * iz + V.cx;
     P.v = V.fy * y * iz + V.cy;
     P.culled = !(ok && P.rx > 0 && P.ry > 0);
+}
+
+// ---------------------------------------------------------------------------------------
+// Decoupled look-back: one pass over chunks taken in ticket order, each publishing its total
+// (state 1) and, once the totals before it are summed, its inclusive prefix (state 2) in one
+// 64-bit word: (tag * 4 + state) << 56 | value.  A chunk only waits for chunks with smaller
+// tickets, whose blocks are running, so every wait ends; a wait is bounded all the same and
+// then sets GS_ERR_TIMEOUT.  Words start at 0; the passes of one sort share words by tags.
+// ---------------------------------------------------------------------------------------
+typedef unsigned long long lbword;
+constexpr int kLbSpin = 1 << 20;   // polls of a wait (about a second)
+
+__device__ __forceinline__ void lb_store(lbword* p, uint32_t tag, uint32_t state, unsigned long long v) {
+    const lbword w = ((lbword)(tag * 4 + state) << 56) | v;
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+}
+__device__ __forceinline__ lbword lb_load(const lbword* p) {
+    lbword w;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+    return w;
+}
+// state of a word under `tag`: 0 while it is not published
+__device__ __forceinline__ uint32_t lb_state(lbword w, uint32_t tag) {
+    const uint32_t t = (uint32_t)(w >> 56);
+    return (t >> 2) == tag ? (t & 3u) : 0u;
+}
+__device__ __forceinline__ unsigned long long lb_value(lbword w) { return w & ((1ull << 56) - 1); }
+// the same in 32 bits, for totals below 2^24 (state and tag in the top byte)
+__device__ __forceinline__ void lb_store(uint32_t* p, uint32_t tag, uint32_t state, uint32_t v) {
+    const uint32_t w = ((tag * 4 + state) << 24) | v;
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(w) : "memory");
+}
+__device__ __forceinline__ uint32_t lb_load(const uint32_t* p) {
+    uint32_t w;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(p) : "memory");
+    return w;
+}
+__device__ __forceinline__ uint32_t lb_state(uint32_t w, uint32_t tag) {
+    const uint32_t t = w >> 24;
+    return (t >> 2) == tag ? (t & 3u) : 0u;
+}
+__device__ __forceinline__ uint32_t lb_value(uint32_t w) { return w & 0xFFFFFFu; }
+
+// One warp: publishes the chunk's total, sums the totals of the chunks before it (128 at a time:
+// the chunks of the first wave publish together and none has a prefix yet) and publishes the
+// inclusive prefix.  Returns the exclusive prefix; ok is cleared if a wait gave up (the status
+// word is then set).
+__device__ __forceinline__ unsigned long long lb_scan_warp(lbword* words, int64_t chunk, unsigned long long total,
+                                                           Counters* c, bool& ok) {
+    const int lane = threadIdx.x & 31;
+    if (chunk == 0) {
+        if (lane == 0) lb_store(words, 0, 2, total);
+        return 0;
+    }
+    if (lane == 0) lb_store(words + chunk, 0, 1, total);
+    unsigned long long before = 0;
+    int spin = 0;
+    bool done = false;
+    for (int64_t base = chunk - 1; !done; base -= 128) {
+        lbword w[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int64_t j = base - 32 * u - lane;
+            w[u] = j >= 0 ? lb_load(words + j) : (lbword)2 << 56;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (done) continue;
+            for (;;) {
+                const uint32_t st = lb_state(w[u], 0);
+                const uint32_t ready = __ballot_sync(0xffffffffu, st != 0), full = __ballot_sync(0xffffffffu, st == 2);
+                const uint32_t need = full ? (full & -full) | ((full & -full) - 1) : 0xffffffffu;
+                if ((ready & need) == need) {
+                    unsigned long long v = (need >> lane) & 1u ? lb_value(w[u]) : 0ull;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    before += v;
+                    done = full != 0;
+                    break;
+                }
+                if (++spin > kLbSpin || ((spin & 1023) == 0 && *(volatile uint32_t*)&c->status != 0)) {
+                    if (lane == 0) set_status(c, GS_ERR_TIMEOUT);
+                    ok = false;
+                    return before;
+                }
+                const int64_t j = base - 32 * u - lane;
+                if (j >= 0) w[u] = lb_load(words + j);
+            }
+        }
+    }
+    if (lane == 0) lb_store(words + chunk, 0, 2, before + total);
+    return before;
 }
 
 template <typename T>

@@ -53,11 +53,15 @@ struct BinArgs {
     int64_t max_pairs;
     const float4* proj;
     const uint32_t* vis_bits;     // [V][ceil(n/32)] per-view visibility words (ProjectArgs)
-    uint32_t* scan_tmp;           // block sums of the scans
+    unsigned long long *entry_scan, *pair_scan;   // look-back words of the two scans (cleared)
+    uint32_t *ehist, *phist;      // digit counts of the first pass of each sort (cleared)
+    uint32_t phist_mask;          // its digit of a pair: tile id & phist_mask (0: no sort follows)
+    uint32_t* tickets;            // [2] chunks taken by the two scans (cleared)
     uint32_t* ekeys;              // compaction output: bits(z) of each entry
     uint32_t* evals;              //   and its compact index (the value the depth sort carries)
     uint32_t* entries;            //   view * n + Gaussian index of each entry, (view, Gaussian) order
-    uint2* erect;                 //   its tile rectangle: (first global tile id, wx | wy << 16)
+    uint4* erect;                 //   its tile rectangle and index: (first global tile id,
+                                  //   wx | wy << 16, view * n + Gaussian index, 0)
     const uint32_t* sorted_evals; // compact indices of the entries in depth order
     uint32_t* pkeys;              // emission output: global tile id of each pair
     uint32_t* pvals;              //   and the entry's view * n + Gaussian index
@@ -68,18 +72,30 @@ struct BinArgs {
     Counters* counters;
 };
 
-// Stable LSD radix sort of (key, value) pairs with 8-bit digits; pass p reads buffer
-// (p & 1) of keys / vals and writes the other.  Keys are uint32 or uint64 per the launcher.
+// Stable LSD radix sort of (key, value) pairs; pass p reads buffer (p & 1) of keys / vals and
+// writes the other.  Keys are uint32 or uint64 per the launcher.  hist (but for the
+// first pass's counts, which the caller's kernels or launch_sort_count64 fill in), tickets and the look-back
+// words must be zero when the sort starts; sorts with different tags can share the words.
 struct SortArgs {
     void* keys[2];
     uint32_t* vals[2];
-    uint32_t* hist;            // [256][grid] block histograms, then block offsets
-    uint32_t* digit_tot;       // [256] digit totals
-    const Counters* counters;  // status word (a set status skips the sort)
+    uint32_t* hist;            // [passes][kSortMaxBins] digit counts of every pass
+    uint32_t* tickets;         // [passes] blocks started
+    unsigned long long* lookback;   // sort_lookback_bytes(capacity, bits of the largest digit)
+    Counters* counters;        // status word (a set status skips the sort)
     const unsigned long long* count;   // element count, read on the device
-    int grid;
+    int64_t capacity;          // upper bound of it (grid sizes)
+    uint32_t tag = 1;          // look-back tags tag .. tag + passes - 1 (below 64)
     uint32_t digit_mask = 0xFFFFFFFFu;  // ANDed into every digit of the pass (a partial top digit)
 };
+// a 64-bit word per digit of every group of kSortGroup blocks (at a place of their own whatever the
+// sort, so that no sort's words of one kind are read as the other kind by the next), then a
+// 32-bit word per digit of every block
+constexpr size_t kSortGroupBytes = sizeof(unsigned long long) * (kSortMaxGrid / kSortGroup) * kSortMaxBins;
+inline size_t sort_lookback_bytes(int64_t capacity, int bits) {
+    const int64_t c = sort_chunks(capacity), blocks = c < kSortMaxGrid ? c : kSortMaxGrid;
+    return kSortGroupBytes + ((sizeof(uint32_t) * (size_t)blocks) << bits);
+}
 
 struct RangeArgs {
     const uint32_t* keys;      // sorted global tile ids
@@ -223,15 +239,22 @@ cudaError_t launch_gicp_register(const GicpMap& src, const uint8_t* src_flag, co
 cudaError_t launch_project(const ProjectArgs& a, int deg, cudaStream_t st);
 cudaError_t launch_project_bwd(const ProjectBwdArgs& a, int deg, cudaStream_t st);
 // Compaction of the visible entries (their vis_bits set) in (view, Gaussian) order with their
-// depth keys; the count goes to c->n_entries.
+// depth keys; the count goes to c->n_entries (zero before the call).
 cudaError_t launch_entries(const BinArgs& a, cudaStream_t st);
-// Pair offsets over the depth-sorted entries (total to c->n_pairs, GS_ERR_CAPACITY above
-// max_pairs) and emission of one (tile id, entry) pair per covered tile.
+// look-back words of the two scans
+size_t entry_scan_words(int64_t n, int n_views);
+size_t pair_scan_words(int64_t n, int n_views);
+// Pair offsets over the depth-sorted entries (total to c->n_pairs, zero before the call;
+// GS_ERR_CAPACITY above max_pairs) and emission of one (tile id, entry) pair per covered tile.
 cudaError_t launch_emit(const BinArgs& a, cudaStream_t st);
 // 32-bit keys: pass p takes bits[p]-bit digits (8 or 9) at shifts[p]; 64-bit keys: 8-bit digits.
 cudaError_t launch_sort32(const SortArgs& a, int n_passes, const int* shifts, const int* bits, cudaStream_t st);
 cudaError_t launch_sort64(const SortArgs& a, int n_passes, const int* shifts, cudaStream_t st);
+// digit counts of the first pass of a 64-bit sort (8 bits at `shift`)
+cudaError_t launch_sort_count64(const SortArgs& a, int shift, cudaStream_t st);
 cudaError_t launch_ranges(const RangeArgs& a, int n_tiles, cudaStream_t st);
+// tmp: kOrderTmpWords words, zero before the call
+constexpr int kOrderTmpWords = 2 * kOrderBuckets + 1;
 cudaError_t launch_tile_order(const uint2* ranges, int n_tiles, uint32_t* order, uint32_t* tmp, const Counters* c,
                               cudaStream_t st);
 cudaError_t launch_loss_count(const View* views, int n_views, const int64_t* pix_counts_host,
@@ -261,8 +284,5 @@ cudaError_t launch_step_persistent(const FwdArgs& fwd, const BwdArgs& bwd, const
                                    int total_tiles, float lambda_rgb, float lambda_depth, int has_depth,
                                    float* loss_out, float b1, float b2, long long spin_limit, int skip_block,
                                    cudaStream_t st, int* grid_out);
-cudaError_t launch_setup_views(View* dst, const View* src_host, int n_views, cudaStream_t st);
-
-int sort_grid();
 
 }  // namespace gs

@@ -273,6 +273,13 @@ struct PcaWs {
 
 static size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// digit counts, tickets and look-back words of the sort
+constexpr size_t kPcaSortCounts = sizeof(uint32_t) * kSortMaxPasses * kSortMaxBins;
+constexpr size_t kPcaSortHead = kPcaSortCounts + 256;
+constexpr size_t kPcaSortRegion = sizeof(uint32_t) * (512 * 512 + 512);
+static_assert(kPcaSortHead + kSortGroupBytes + (size_t)kSortMaxGrid * 4 * kSortBins <= kPcaSortRegion,
+              "sort_lookback_bytes of any size");
+
 static PcaWs pca_layout(int64_t n) {
     PcaWs L;
     size_t off = 0;
@@ -282,7 +289,7 @@ static PcaWs pca_layout(int64_t n) {
     L.keys1 = take(8 * (size_t)n);
     L.vals0 = take(4 * (size_t)n);
     L.vals1 = take(4 * (size_t)n);
-    L.hist = take(sizeof(uint32_t) * ((size_t)kSortMaxBins * kSortMaxGrid + kSortMaxBins));
+    L.hist = take(kPcaSortRegion);
     L.total = off;
     return L;
 }
@@ -303,15 +310,19 @@ cudaError_t launch_voxel_pca(const float* pts, const float* rgb, int64_t n, cons
     sa.vals[0] = reinterpret_cast<uint32_t*>(b + L.vals0);
     sa.vals[1] = reinterpret_cast<uint32_t*>(b + L.vals1);
     sa.hist = reinterpret_cast<uint32_t*>(b + L.hist);
-    sa.digit_tot = sa.hist + (size_t)kSortMaxBins * kSortMaxGrid;
+    sa.tickets = reinterpret_cast<uint32_t*>(b + L.hist + kPcaSortCounts);
+    sa.lookback = reinterpret_cast<unsigned long long*>(b + L.hist + kPcaSortHead);
     sa.counters = cnt;
     sa.count = &cnt->n_pairs;
-    sa.grid = sort_grid();
+    sa.capacity = n;
+    cudaError_t e = cudaMemsetAsync(b + L.hist, 0, kPcaSortHead + sort_lookback_bytes(n, 8), st);
+    if (e != cudaSuccess) return e;
     const int blocks = (int)((n + 255) / 256);
     point_depth_kernel<<<blocks, 256, 0, st>>>(pts, n, fs, depth, inside);
     voxel_key_kernel<<<blocks, 256, 0, st>>>(pts, n, voxel, vkeys, sa.vals[0], cnt);
     int shifts[8] = {0, 8, 16, 24, 32, 40, 48, 56};
-    cudaError_t e = launch_sort64(sa, 8, shifts, st);   // 63-bit keys, result back in buffer 0
+    if ((e = launch_sort_count64(sa, shifts[0], st)) != cudaSuccess) return e;
+    e = launch_sort64(sa, 8, shifts, st);   // 63-bit keys, result back in buffer 0
     if (e != cudaSuccess) return e;
     PcaArgs a;
     a.n = n;

@@ -182,7 +182,7 @@ static cudaError_t launch_project_bwd_t(const ProjectBwdArgs& a, int deg, cudaSt
 cudaError_t launch_project_bwd(const ProjectBwdArgs& a, int deg, cudaStream_t st) {
     // entry part (persistent grid over the device-side entry count), then the row part's SH
     // and geometry kernels
-    project_bwd_entry_kernel<<<sort_grid() * 4, kEntryThreads, 0, st>>>(a);
+    project_bwd_entry_kernel<<<device_sms() * 12, kEntryThreads, 0, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return a.fused_adam ? launch_project_bwd_t<true>(a, deg, st) : launch_project_bwd_t<false>(a, deg, st);

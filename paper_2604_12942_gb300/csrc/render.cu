@@ -1060,7 +1060,7 @@ __global__ void __launch_bounds__(256) clear_grad2d_kernel(BwdArgs a, Counters* 
 
 cudaError_t launch_render_bwd(const BwdArgs& a, int total_tiles, cudaStream_t st, Counters* adam_ctr, float b1,
                               float b2, const LossFinal& lf) {
-    clear_grad2d_kernel<<<sort_grid() * 4, 256, 0, st>>>(a, adam_ctr, b1, b2, lf);
+    clear_grad2d_kernel<<<device_sms() * 12, 256, 0, st>>>(a, adam_ctr, b1, b2, lf);
     if (total_tiles <= 0) return cudaGetLastError();
     // 16 x 16 tiles: one independent warp per 8 x 8 region (8 x 8 tiles are one warp already)
     if (a.op.tile == 16) {

@@ -20,17 +20,19 @@
 namespace gs {
 
 constexpr int64_t kNoAllocMaxPairs = int64_t(1) << 20;
-// The sort grid never exceeds kSortMaxGrid blocks (sort_grid() caps it), and each block of a
-// pass owns one histogram row: the scratch holds exactly that many rows.
-constexpr int kNoAllocMaxGrid = kSortMaxGrid;
+// A pass at a time: its look-back words (a chunk's digits each) and its digit counts.
 constexpr size_t kNoAllocCounters = 256;
-constexpr size_t kNoAllocHist = sizeof(uint32_t) * ((size_t)kSortBins * kNoAllocMaxGrid + kSortBins);
+constexpr size_t kNoAllocTickets = 192;   // in the counters' slot
+constexpr size_t kNoAllocLookback = 524288;
+constexpr size_t kNoAllocHist = kNoAllocLookback + sizeof(uint32_t) * kSortBins;
+static_assert(kSortGroupBytes + kNoAllocMaxPairs / kSortChunk * 4 * kSortBins <= kNoAllocLookback,
+              "sort_lookback_bytes of the largest call");
 constexpr size_t kNoAllocKeys = sizeof(unsigned long long) * (size_t)kNoAllocMaxPairs;
 constexpr size_t kNoAllocVals = sizeof(uint32_t) * (size_t)kNoAllocMaxPairs;
 constexpr size_t kNoAllocBytes = kNoAllocCounters + kNoAllocHist + kNoAllocKeys + kNoAllocVals;
 
 static_assert(kNoAllocBytes == 13108480, "the size stated in gs.h");
-static_assert(sizeof(Counters) <= kNoAllocCounters, "counter block");
+static_assert(sizeof(Counters) <= kNoAllocTickets, "counter block");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -57,12 +59,19 @@ static cudaError_t noalloc_scratch(void** out) {
 }
 
 // The sort kernels read the pair count and the status word from a Counters block; here it
-// lives at the start of the scratch and is rewritten by every call.
-__global__ void noalloc_init_kernel(Counters* c, unsigned long long n) {
+// lives at the start of the scratch.  Every pass starts from zero digit counts, tickets and
+// look-back words.
+__global__ void __launch_bounds__(kSortBins) noalloc_init_kernel(Counters* c, uint32_t* hist, uint32_t* tickets,
+                                                                 unsigned long long* lookback, uint32_t words,
+                                                                 unsigned long long n) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < words; i += gridDim.x * blockDim.x) lookback[i] = 0ull;
+    if (blockIdx.x != 0) return;
+    hist[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         c->status = 0;
         c->n_entries32 = 0;
         c->n_pairs = n;
+        tickets[0] = 0;
     }
 }
 
@@ -103,10 +112,10 @@ extern "C" gs_status gs_sort_pairs_noalloc(const uint64_t* keys_in, const uint32
     cudaStream_t st = (cudaStream_t)stream;
     unsigned char* b = static_cast<unsigned char*>(base);
     Counters* cnt = reinterpret_cast<Counters*>(b);
-    uint32_t* hist = reinterpret_cast<uint32_t*>(b + kNoAllocCounters);
+    uint32_t* tickets = reinterpret_cast<uint32_t*>(b + kNoAllocTickets);
+    uint32_t* hist = reinterpret_cast<uint32_t*>(b + kNoAllocCounters + kNoAllocLookback);
     unsigned long long* k_tmp = reinterpret_cast<unsigned long long*>(b + kNoAllocCounters + kNoAllocHist);
     uint32_t* v_tmp = reinterpret_cast<uint32_t*>(b + kNoAllocCounters + kNoAllocHist + kNoAllocKeys);
-    noalloc_init_kernel<<<1, 32, 0, st>>>(cnt, (unsigned long long)n);
     const int passes = (key_bits + 7) / 8;
     // Pass 0 reads the caller's input; the passes then alternate between the output and
     // the scratch copy so that the last one writes the output.
@@ -115,10 +124,11 @@ extern "C" gs_status gs_sort_pairs_noalloc(const uint64_t* keys_in, const uint32
     uint32_t* vdst[2] = {(passes & 1) ? vals_out : v_tmp, (passes & 1) ? v_tmp : vals_out};
     SortArgs a;
     a.hist = hist;
-    a.digit_tot = hist + (size_t)kSortBins * kNoAllocMaxGrid;
+    a.tickets = tickets;
+    a.lookback = reinterpret_cast<unsigned long long*>(b + kNoAllocCounters);
     a.counters = cnt;
     a.count = &cnt->n_pairs;
-    a.grid = sort_grid();   // <= kSortMaxGrid = kNoAllocMaxGrid
+    a.capacity = n;
     for (int p = 0; p < passes; p++) {
         const int shift = 8 * p;
         if (p == 0) {
@@ -133,7 +143,11 @@ extern "C" gs_status gs_sort_pairs_noalloc(const uint64_t* keys_in, const uint32
         // the last pass takes only the key bits below key_bits
         const int top = key_bits - shift;
         a.digit_mask = top >= 8 ? 0xFFFFFFFFu : (1u << top) - 1u;
-        e = launch_sort64(a, 1, &shift, st);
+        const uint32_t words = (uint32_t)(sort_lookback_bytes(n, 8) / sizeof(unsigned long long));
+        noalloc_init_kernel<<<(int)((words + 4 * kSortBins - 1) / (4 * kSortBins)), kSortBins, 0, st>>>(
+            cnt, hist, tickets, a.lookback, words, (unsigned long long)n);
+        e = launch_sort_count64(a, shift, st);
+        if (e == cudaSuccess) e = launch_sort64(a, 1, &shift, st);
         if (e != cudaSuccess) return record_error(GS_ERR_CUDA, cudaGetErrorString(e));
     }
     return GS_OK;
