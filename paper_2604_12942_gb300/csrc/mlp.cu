@@ -22,29 +22,51 @@ constexpr int kLdIn = kIn + 8, kLdHid = kHid + 8;   // padded smem strides (bf16
 
 typedef __nv_bfloat16 bf16;
 
-__device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
-    return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
+__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
+    return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(lo)) |
+           ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(hi)) << 16);
 }
 
-// acc += A (16x16) * B (16x8) with A(m, k) = A0[m*sam + k*sak] and B(k, n) = B0[k*sbk + n*sbn]
-// (BF16 in shared memory), FP32 accumulate.  Fragment layout of mma.m16n8k16 (row.col):
-// lane = 4 g + t; A regs {(g, 2t..2t+1), (g+8, 2t..), (g, 2t+8..), (g+8, 2t+8..)}, B regs
-// {(2t..2t+1, g), (2t+8.., g)}, C {(g, 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1)}.
-__device__ __forceinline__ void mma_tile(float acc[4], const bf16* A0, int sam, int sak, const bf16* B0, int sbk,
-                                         int sbn) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    auto A = [&](int m, int k) { return A0[m * sam + k * sak]; };
-    auto B = [&](int k, int n) { return B0[k * sbk + n * sbn]; };
-    const uint32_t a0 = pack2(A(g, 2 * t), A(g, 2 * t + 1));
-    const uint32_t a1 = pack2(A(g + 8, 2 * t), A(g + 8, 2 * t + 1));
-    const uint32_t a2 = pack2(A(g, 2 * t + 8), A(g, 2 * t + 9));
-    const uint32_t a3 = pack2(A(g + 8, 2 * t + 8), A(g + 8, 2 * t + 9));
-    const uint32_t b0 = pack2(B(2 * t, g), B(2 * t + 1, g));
-    const uint32_t b1 = pack2(B(2 * t + 8, g), B(2 * t + 9, g));
+// Fragment layout of mma.m16n8k16 (row.col): lane = 4 g + t; A regs {(g, 2t..2t+1), (g+8, 2t..),
+// (g, 2t+8..), (g+8, 2t+8..)}, B regs {(2t..2t+1, g), (2t+8.., g)}, C {(g, 2t), (g, 2t+1),
+// (g+8, 2t), (g+8, 2t+1)}.  So the results of two neighbouring column tiles are, rounded to BF16,
+// the A registers of the k step over the same 16 columns: a warp's 16 rows pass from layer to
+// layer in registers, and only weights come from shared memory (ldmatrix, four 8 x 8 blocks an
+// instruction; rows padded by 16 bytes keep it free of bank conflicts).  Gathering every
+// fragment element by element from shared memory took 377 us for 400k rows, most of it those
+// loads; this form takes 203, bound by the erf of 384 activations a row (about 120 us of issue
+// slots).  The k steps are summed in the same order, so the outputs are the same bits; tcgen05
+// sums in another order, which moves BF16 roundings of the activations.
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                  "{%0,%1,%2,%3};\n"
-                 : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const bf16* p) {
+    const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(s) : "memory");
+}
+__device__ __forceinline__ void ldsm4_trans(uint32_t (&r)[4], const bf16* p) {
+    const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(p));
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(s) : "memory");
+}
+// B of two column tiles (n0, n0 + 8) and one k step from M[n][k] or, transposed, from M[k][n]:
+// r = {b0, b1} of the first, {b0, b1} of the second
+__device__ __forceinline__ void load_b(uint32_t (&r)[4], const bf16* M, int ld, int n0, int k0) {
+    const int lane = threadIdx.x & 31;
+    ldsm4(r, M + (n0 + (lane & 7) + (lane >> 4) * 8) * ld + k0 + ((lane >> 3) & 1) * 8);
+}
+__device__ __forceinline__ void load_b_trans(uint32_t (&r)[4], const bf16* M, int ld, int n0, int k0) {
+    const int lane = threadIdx.x & 31;
+    ldsm4_trans(r, M + (k0 + (lane & 7) + ((lane >> 3) & 1) * 8) * ld + n0 + (lane >> 4) * 8);
+}
+// A of rows m0.. and one k step from M[k][m]
+__device__ __forceinline__ void load_a_trans(uint32_t (&r)[4], const bf16* M, int ld, int m0, int k0) {
+    const int lane = threadIdx.x & 31;
+    ldsm4_trans(r, M + (k0 + (lane & 7) + (lane >> 4) * 8) * ld + m0 + ((lane >> 3) & 1) * 8);
 }
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
@@ -52,219 +74,307 @@ __device__ __forceinline__ float gelu_grad(float z) {
     return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * expf(-0.5f * z * z) * 0.3989422804014327f;
 }
 
-struct MlpSmem {
+// Two adjacent floats; vec: the pointer is 8-byte aligned (checked on the host per buffer).
+__device__ __forceinline__ float2 ld2(const float* p, bool vec) {
+    return vec ? *reinterpret_cast<const float2*>(p) : make_float2(p[0], p[1]);
+}
+__device__ __forceinline__ void st2(float* p, float a, float b, bool vec) {
+    if (vec) *reinterpret_cast<float2*>(p) = make_float2(a, b);
+    else { p[0] = a; p[1] = b; }
+}
+__device__ __forceinline__ void add2(float* p, float a, float b, bool vec) {
+    if (vec) atomicAdd(reinterpret_cast<float2*>(p), make_float2(a, b));
+    else { atomicAdd(p, a); atomicAdd(p + 1, b); }
+}
+
+struct WeightSmem {
     bf16 w1[kHid * kLdIn];
-    bf16 w2[kHid * kLdHid];
-    bf16 w3[kHid * kLdHid];
+    bf16 w2[2][kHid * kLdHid];   // W2, W3
     bf16 w4[kOut * kLdHid];
     float b[kNB];
-    bf16 a0[kRows * kLdIn];
-    bf16 a1[kRows * kLdHid];
-    bf16 a2[kRows * kLdHid];
-    bf16 a3[kRows * kLdHid];
 };
 
-__device__ void load_weights(MlpSmem& S, const bf16* w, const float* b) {
-    for (int e = threadIdx.x; e < kHid * kIn; e += blockDim.x) S.w1[(e / kIn) * kLdIn + e % kIn] = w[woff(0) + e];
-    for (int e = threadIdx.x; e < kHid * kHid; e += blockDim.x) {
-        S.w2[(e / kHid) * kLdHid + e % kHid] = w[woff(1) + e];
-        S.w3[(e / kHid) * kLdHid + e % kHid] = w[woff(2) + e];
+// vec: w is 16-byte aligned
+__device__ void load_weights(WeightSmem& S, const bf16* w, const float* b, bool vec) {
+    // eight elements of one matrix row at a time (the rows' padded strides are multiples of 8)
+    for (int e = threadIdx.x; e < kNW / 8; e += blockDim.x) {
+        const int i = 8 * e;
+        bf16* dst;
+        if (i < woff(1)) dst = S.w1 + (i / kIn) * kLdIn + i % kIn;
+        else if (i < woff(3)) {
+            const int j = i - woff(1), m = j / (kHid * kHid), q = j % (kHid * kHid);
+            dst = S.w2[m] + (q / kHid) * kLdHid + q % kHid;
+        } else dst = S.w4 + ((i - woff(3)) / kHid) * kLdHid + (i - woff(3)) % kHid;
+        if (vec) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(w + i);
+        else
+            for (int k = 0; k < 8; k++) dst[k] = w[i + k];
     }
-    for (int e = threadIdx.x; e < kOut * kHid; e += blockDim.x) S.w4[(e / kHid) * kLdHid + e % kHid] = w[woff(3) + e];
     for (int e = threadIdx.x; e < kNB; e += blockDim.x) S.b[e] = b[e];
 }
 
-// One layer for the warp's 16 rows: out[r][n] = sum_k in[r][k] W[n][k] + bias[n].  The
-// result goes through `epi(row, col, value)` (each lane owns 4 values per 8-column tile).
-template <int K, int N, typename Epi>
-__device__ __forceinline__ void warp_layer(const bf16* in, int ldin, const bf16* W, int ldw, const float* bias, int r0,
-                                           Epi epi) {
+// BF16 input rows r0 .. r0 + 15 as the A registers of the first layer (rows past n are zero)
+__device__ __forceinline__ void load_x(uint32_t (&a)[4], const float* x, int64_t r0, int64_t n, bool vec) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-#pragma unroll 2
-    for (int n0 = 0; n0 < N; n0 += 8) {
-        float acc[4] = {bias[n0 + 2 * t], bias[n0 + 2 * t + 1], bias[n0 + 2 * t], bias[n0 + 2 * t + 1]};
 #pragma unroll
-        for (int k0 = 0; k0 < K; k0 += 16) mma_tile(acc, in + r0 * ldin + k0, ldin, 1, W + n0 * ldw + k0, 1, ldw);
-        epi(r0 + g, n0 + 2 * t, acc[0]);
-        epi(r0 + g, n0 + 2 * t + 1, acc[1]);
-        epi(r0 + g + 8, n0 + 2 * t, acc[2]);
-        epi(r0 + g + 8, n0 + 2 * t + 1, acc[3]);
+    for (int q = 0; q < 4; q++) {
+        const int64_t row = r0 + g + (q & 1) * 8;
+        const float2 v = row < n ? ld2(x + row * kIn + 2 * t + (q >> 1) * 8, vec) : make_float2(0.f, 0.f);
+        a[q] = pack2(v.x, v.y);
     }
 }
 
-// Forward of the warp's 16 rows from S.a0; hidden activations (BF16) kept in S.a1..a3,
-// pre-activations optionally stored (FP32) for the backward, outputs through `out`.
+// Forward of the warp's 16 rows; the pre-activations go to z1..z3 (each [n][128], null: not
+// stored), the output layer's two column tiles (C layout) through out(c0, c1).
 template <typename Out>
-__device__ __forceinline__ void warp_forward(MlpSmem& S, int r0, float* z1, float* z2, float* z3, int64_t row_base,
-                                             int64_t n, Out out) {
-    auto hid = [&](bf16* dst, float* zst) {
-        return [=, &S](int r, int c, float v) {
-            dst[r * kLdHid + c] = __float2bfloat16_rn(gelu(v));
-            if (zst && row_base + r < n) zst[(row_base + r) * kHid + c] = v;
-        };
+__device__ __forceinline__ void warp_forward(const WeightSmem& S, const uint32_t (&x)[4], float* const (&z)[3], int64_t r0,
+                                             int64_t n, bool vec, Out out) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    uint32_t A[8][4], B[8][4];
+    auto bias = [&](float (&c)[4], const float* b, int n0) {
+        c[0] = c[2] = b[n0 + 2 * t];
+        c[1] = c[3] = b[n0 + 2 * t + 1];
     };
-    warp_layer<kIn, kHid>(S.a0, kLdIn, S.w1, kLdIn, S.b + boff(0), r0, hid(S.a1, z1));
-    __syncwarp();
-    warp_layer<kHid, kHid>(S.a1, kLdHid, S.w2, kLdHid, S.b + boff(1), r0, hid(S.a2, z2));
-    __syncwarp();
-    warp_layer<kHid, kHid>(S.a2, kLdHid, S.w3, kLdHid, S.b + boff(2), r0, hid(S.a3, z3));
-    __syncwarp();
-    warp_layer<kHid, kOut>(S.a3, kLdHid, S.w4, kLdHid, S.b + boff(3), r0, out);
-}
-
-__device__ __forceinline__ void load_input_rows(MlpSmem& S, const float* x, int64_t row_base, int64_t n) {
-    for (int e = threadIdx.x; e < kRows * kIn; e += blockDim.x) {
-        const int r = e / kIn, c = e % kIn;
-        const int64_t row = row_base + r;
-        S.a0[r * kLdIn + c] = __float2bfloat16_rn(row < n ? x[row * kIn + c] : 0.f);
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) mlp_infer_kernel(const bf16* w, const float* b, const float* x, int64_t n,
-                                                             float* y) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    MlpSmem& S = *reinterpret_cast<MlpSmem*>(smem_raw);
-    load_weights(S, w, b);
-    const int r0 = (threadIdx.x >> 5) * 16;
-    for (int64_t base = (int64_t)blockIdx.x * kRows; base < n; base += (int64_t)gridDim.x * kRows) {
-        __syncthreads();
-        load_input_rows(S, x, base, n);
-        __syncthreads();
-        warp_forward(S, r0, nullptr, nullptr, nullptr, base, n, [&](int r, int c, float v) {
-            if (base + r < n) y[(base + r) * kOut + c] = v;
-        });
-    }
-}
-
-// Training, pass 1: forward with stored pre-activations and hidden activations; output
-// gradient g4 = 2 (y - t) / (n * 11) on the 11 used outputs; loss sum.
-__global__ void __launch_bounds__(kThreads) mlp_train_fwd_kernel(const bf16* w, const float* b, const float* x,
-                                                                 const float* t, int64_t n, float* z1, float* z2,
-                                                                 float* z3, float* g4, double* loss_sum) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    MlpSmem& S = *reinterpret_cast<MlpSmem*>(smem_raw);
-    load_weights(S, w, b);
-    const int r0 = (threadIdx.x >> 5) * 16;
-    double lsum = 0.0;
-    const float scale = 2.f / ((float)n * (float)kOutUsed);
-    for (int64_t base = (int64_t)blockIdx.x * kRows; base < n; base += (int64_t)gridDim.x * kRows) {
-        __syncthreads();
-        load_input_rows(S, x, base, n);
-        __syncthreads();
-        warp_forward(S, r0, z1, z2, z3, base, n, [&](int r, int c, float v) {
-            const int64_t row = base + r;
-            if (row >= n) return;
-            float gv = 0.f;
-            if (c < kOutUsed) {
-                const float d = v - t[row * kOut + c];
-                lsum += (double)d * (double)d;
-                gv = scale * d;
+    // the hidden layer's columns 16 j .. 16 j + 15 from their two tiles' sums
+    auto activate = [&](uint32_t (&dst)[4], const float (&c0)[4], const float (&c1)[4], float* zl, int j) {
+        if (zl) {
+            const int c = 16 * j + 2 * t;
+            if (r0 + g < n) {
+                st2(zl + (r0 + g) * kHid + c, c0[0], c0[1], vec);
+                st2(zl + (r0 + g) * kHid + c + 8, c1[0], c1[1], vec);
             }
-            g4[row * kOut + c] = gv;
-        });
+            if (r0 + g + 8 < n) {
+                st2(zl + (r0 + g + 8) * kHid + c, c0[2], c0[3], vec);
+                st2(zl + (r0 + g + 8) * kHid + c + 8, c1[2], c1[3], vec);
+            }
+        }
+        dst[0] = pack2(gelu(c0[0]), gelu(c0[1]));
+        dst[1] = pack2(gelu(c0[2]), gelu(c0[3]));
+        dst[2] = pack2(gelu(c1[0]), gelu(c1[1]));
+        dst[3] = pack2(gelu(c1[2]), gelu(c1[3]));
+    };
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+        float c0[4], c1[4];
+        uint32_t w[4];
+        bias(c0, S.b + boff(0), 16 * j);
+        bias(c1, S.b + boff(0), 16 * j + 8);
+        load_b(w, S.w1, kLdIn, 16 * j, 0);
+        mma16816(c0, x, w[0], w[1]);
+        mma16816(c1, x, w[2], w[3]);
+        activate(A[j], c0, c1, z[0], j);
     }
-    lsum = warp_sum(lsum);
-    if ((threadIdx.x & 31) == 0 && lsum != 0.0) atomicAdd(loss_sum, lsum);
+#pragma unroll 1
+    for (int l = 1; l <= 2; l++) {
+        const bf16* W = S.w2[l - 1];
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            float c0[4], c1[4];
+            bias(c0, S.b + boff(l), 16 * j);
+            bias(c1, S.b + boff(l), 16 * j + 8);
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                uint32_t w[4];
+                load_b(w, W, kLdHid, 16 * j, 16 * k);
+                mma16816(c0, A[k], w[0], w[1]);
+                mma16816(c1, A[k], w[2], w[3]);
+            }
+            activate(B[j], c0, c1, z[l], j);
+        }
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+#pragma unroll
+            for (int q = 0; q < 4; q++) A[j][q] = B[j][q];
+    }
+    float c0[4], c1[4];
+    bias(c0, S.b + boff(3), 0);
+    bias(c1, S.b + boff(3), 8);
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+        uint32_t w[4];
+        load_b(w, S.w4, kLdHid, 0, 16 * k);
+        mma16816(c0, A[k], w[0], w[1]);
+        mma16816(c1, A[k], w[2], w[3]);
+    }
+    out(c0, c1);
 }
 
-struct BwdSmem {
-    bf16 w1[kHid * kLdIn];
-    bf16 w2[kHid * kLdHid];
-    bf16 w3[kHid * kLdHid];
-    bf16 w4[kOut * kLdHid];
-    bf16 act[kRows * kLdHid];     // a_{l-1} of the current layer (BF16, recomputed input side)
-    bf16 g[kRows * kLdHid];       // g_l (BF16 operand)
-    bf16 gn[kRows * kLdHid];      // g_{l-1} being formed
+// A warp takes 16 rows at a time; no barrier after the weights are in place.
+__global__ void __launch_bounds__(kThreads, 2) mlp_infer_kernel(const bf16* w, const float* b, const float* x, int64_t n,
+                                                                float* y, bool vec_w, bool vec) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    WeightSmem& S = *reinterpret_cast<WeightSmem*>(smem_raw);
+    load_weights(S, w, b, vec_w);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    float* const none[3] = {nullptr, nullptr, nullptr};
+    for (int64_t r0 = ((int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * 16; r0 < n;
+         r0 += (int64_t)gridDim.x * (kThreads / 32) * 16) {
+        uint32_t a[4];
+        load_x(a, x, r0, n, vec);
+        warp_forward(S, a, none, r0, n, vec, [&](const float (&c0)[4], const float (&c1)[4]) {
+            if (r0 + g < n) {
+                st2(y + (r0 + g) * kOut + 2 * t, c0[0], c0[1], vec);
+                st2(y + (r0 + g) * kOut + 2 * t + 8, c1[0], c1[1], vec);
+            }
+            if (r0 + g + 8 < n) {
+                st2(y + (r0 + g + 8) * kOut + 2 * t, c0[2], c0[3], vec);
+                st2(y + (r0 + g + 8) * kOut + 2 * t + 8, c1[2], c1[3], vec);
+            }
+        });
+    }
+}
+
+struct TrainSmem {
+    WeightSmem w;
+    bf16 g[kRows * kLdHid];     // g_l of the block's rows, [row][output]
+    bf16 act[kRows * kLdHid];   // a_{l-1}, [row][input]
 };
 
-// Training, pass 2: per CTA rows, layer by layer from the output: weight / bias gradients
-// (g_l^T a_{l-1}, reduced over the CTA's rows and added atomically) and the gradient of the
-// previous layer's pre-activation g_{l-1} = (g_l W_l) * gelu'(z_{l-1}).
-__global__ void __launch_bounds__(kThreads) mlp_train_bwd_kernel(const bf16* w, const float* x, int64_t n,
-                                                                 const float* z1, const float* z2, const float* z3,
-                                                                 const float* g4, float* gw, float* gb) {
+// One training pass over the block's 128 rows, a warp's 16 rows in registers: the forward with the
+// pre-activations stored, the output gradient g = 2 (y - t) / (n * 11) on the 11 used outputs and
+// the loss sum, then layer by layer from the output the weight / bias gradients (g_l^T a_{l-1},
+// summed over the block's rows and added atomically) and the gradient of the previous layer's
+// pre-activation g_{l-1} = (g_l W_l) * gelu'(z_{l-1}).  Only the weight gradients mix rows of
+// different warps: g_l and a_{l-1} pass through shared memory for them, and a column of ones as
+// one more B operand gives the bias gradient.  Forward and backward in one kernel read back the
+// pre-activations their own lanes wrote.  16384 rows: 202 us a step with two kernels that
+// gathered their fragments element by element, 80 us with this one.
+__global__ void __launch_bounds__(kThreads, 1) mlp_train_kernel(const bf16* w, const float* b, const float* x,
+                                                                const float* tgt, int64_t n, float* z1, float* z2,
+                                                                float* z3, float* gw, float* gb, double* loss_sum,
+                                                                bool vec_w, bool vec) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    BwdSmem& S = *reinterpret_cast<BwdSmem*>(smem_raw);
-    for (int e = threadIdx.x; e < kHid * kIn; e += blockDim.x) S.w1[(e / kIn) * kLdIn + e % kIn] = w[woff(0) + e];
-    for (int e = threadIdx.x; e < kHid * kHid; e += blockDim.x) {
-        S.w2[(e / kHid) * kLdHid + e % kHid] = w[woff(1) + e];
-        S.w3[(e / kHid) * kLdHid + e % kHid] = w[woff(2) + e];
-    }
-    for (int e = threadIdx.x; e < kOut * kHid; e += blockDim.x) S.w4[(e / kHid) * kLdHid + e % kHid] = w[woff(3) + e];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gq = lane >> 2, tq = lane & 3;
-    const float* zs[4] = {nullptr, z1, z2, z3};
-    const bf16* Ws[4] = {S.w1, S.w2, S.w3, S.w4};
-    const int lds[4] = {kLdIn, kLdHid, kLdHid, kLdHid};
+    TrainSmem& S = *reinterpret_cast<TrainSmem*>(smem_raw);
+    load_weights(S.w, w, b, vec_w);
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    float* const zs[3] = {z1, z2, z3};
+    const float scale = 2.f / ((float)n * (float)kOutUsed);
+    double lsum = 0.0;
+    uint32_t* const gw32 = reinterpret_cast<uint32_t*>(S.g);
+    uint32_t* const aw32 = reinterpret_cast<uint32_t*>(S.act);
+    constexpr int LW = kLdHid / 2;   // row stride in words
+    const int row0 = warp * 16 + g;  // this lane's rows of the block: row0, row0 + 8
     for (int64_t base = (int64_t)blockIdx.x * kRows; base < n; base += (int64_t)gridDim.x * kRows) {
-        __syncthreads();
-        // g4 of the rows (16 columns)
-        for (int e = threadIdx.x; e < kRows * kOut; e += blockDim.x) {
-            const int r = e / kOut, c = e % kOut;
-            const int64_t row = base + r;
-            S.g[r * kLdHid + c] = __float2bfloat16_rn(row < n ? g4[row * kOut + c] : 0.f);
-        }
-        for (int l = 3; l >= 0; l--) {
-            const int out_dim = l == 3 ? kOut : kHid, in_dim = l == 0 ? kIn : kHid;
-            // a_{l-1}: the network input (l = 0) or gelu(z_l) of the previous layer, as BF16
-            for (int e = threadIdx.x; e < kRows * in_dim; e += blockDim.x) {
-                const int r = e / in_dim, c = e % in_dim;
-                const int64_t row = base + r;
-                float v = 0.f;
-                if (row < n) v = (l == 0) ? x[row * kIn + c] : gelu(zs[l][row * kHid + c]);
-                S.act[r * kLdHid + c] = __float2bfloat16_rn(v);
-            }
-            __syncthreads();
-            // bias gradient: column sums of g_l
-            for (int c = threadIdx.x; c < out_dim; c += blockDim.x) {
-                float s = 0.f;
-                for (int r = 0; r < kRows; r++) s += __bfloat162float(S.g[r * kLdHid + c]);
-                if (s != 0.f) atomicAdd(&gb[boff(l) + c], s);
-            }
-            // weight gradient gW[o][i] = sum_r g[r][o] a[r][i]: M = out, N = in, K = rows
-            const int mt = out_dim / 16, nt = in_dim / 8;
-            for (int tile = warp; tile < mt * nt; tile += kThreads / 32) {
-                const int o0 = (tile / nt) * 16, i0 = (tile % nt) * 8;
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-                for (int r0 = 0; r0 < kRows; r0 += 16)
-                    mma_tile(acc, S.g + r0 * kLdHid + o0, 1, kLdHid, S.act + r0 * kLdHid + i0, kLdHid, 1);
-                float* dst = gw + woff(l);
-                atomicAdd(&dst[(o0 + gq) * in_dim + i0 + 2 * tq], acc[0]);
-                atomicAdd(&dst[(o0 + gq) * in_dim + i0 + 2 * tq + 1], acc[1]);
-                atomicAdd(&dst[(o0 + gq + 8) * in_dim + i0 + 2 * tq], acc[2]);
-                atomicAdd(&dst[(o0 + gq + 8) * in_dim + i0 + 2 * tq + 1], acc[3]);
-            }
-            if (l == 0) break;
-            // g_{l-1} = (g_l W_l) * gelu'(z_l): rows x in_dim, K = out_dim (each warp its 16 rows)
-            const int r0 = warp * 16;
-            for (int i0 = 0; i0 < in_dim; i0 += 8) {
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int k0 = 0; k0 < out_dim; k0 += 16)
-                    mma_tile(acc, S.g + r0 * kLdHid + k0, kLdHid, 1, Ws[l] + k0 * lds[l] + i0, lds[l], 1);
-                const int rr[4] = {r0 + gq, r0 + gq, r0 + gq + 8, r0 + gq + 8};
-                const int cc[4] = {i0 + 2 * tq, i0 + 2 * tq + 1, i0 + 2 * tq, i0 + 2 * tq + 1};
+        const int64_t r0 = base + warp * 16;
+        uint32_t xa[4], G[8][4];
+        load_x(xa, x, r0, n, vec);
+        warp_forward(S.w, xa, zs, r0, n, vec, [&](const float (&c0)[4], const float (&c1)[4]) {
+            float gv[8];
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const int64_t row = base + rr[q];
-                    const float zz = row < n ? zs[l][row * kHid + cc[q]] : 0.f;
-                    S.gn[rr[q] * kLdHid + cc[q]] = __float2bfloat16_rn(acc[q] * gelu_grad(zz));
+            for (int q = 0; q < 8; q++) {
+                const int64_t row = r0 + g + ((q >> 1) & 1) * 8;
+                const int c = 2 * t + (q & 1) + (q >> 2) * 8;
+                gv[q] = 0.f;
+                if (row < n && c < kOutUsed) {
+                    const float d = (q < 4 ? c0[q & 3] : c1[q & 3]) - tgt[row * kOut + c];
+                    lsum += (double)d * (double)d;
+                    gv[q] = scale * d;
                 }
             }
-            __syncthreads();
-            for (int e = threadIdx.x; e < kRows * kHid; e += blockDim.x) {
-                const int r = e / kHid, c = e % kHid;
-                S.g[r * kLdHid + c] = S.gn[r * kLdHid + c];
+            G[0][0] = pack2(gv[0], gv[1]);
+            G[0][1] = pack2(gv[2], gv[3]);
+            G[0][2] = pack2(gv[4], gv[5]);
+            G[0][3] = pack2(gv[6], gv[7]);
+        });
+#pragma unroll 1
+        for (int l = 3; l >= 0; l--) {
+            const int out_dim = l == 3 ? kOut : kHid, in_dim = l == 0 ? kIn : kHid;
+            const int nk = out_dim / 16;
+            __syncthreads();   // the last layer's products have read g and act
+#pragma unroll
+            for (int k = 0; k < 8; k++) {
+                if (k >= nk) break;
+                gw32[row0 * LW + 8 * k + t] = G[k][0];
+                gw32[(row0 + 8) * LW + 8 * k + t] = G[k][1];
+                gw32[row0 * LW + 8 * k + t + 4] = G[k][2];
+                gw32[(row0 + 8) * LW + 8 * k + t + 4] = G[k][3];
+            }
+            if (l == 0) {
+                aw32[row0 * LW + t] = xa[0];
+                aw32[(row0 + 8) * LW + t] = xa[1];
+                aw32[row0 * LW + t + 4] = xa[2];
+                aw32[(row0 + 8) * LW + t + 4] = xa[3];
+            } else {
+                // a_{l-1} = gelu(z_l) into shared memory and g_{l-1} into registers
+                const float* zl = zs[l - 1];
+                const bf16* W = l == 3 ? S.w.w4 : S.w.w2[l - 1];
+                uint32_t H[8][4];
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+                    for (int k = 0; k < 8; k++) {
+                        if (k >= nk) break;
+                        uint32_t wb[4];
+                        load_b_trans(wb, W, kLdHid, 16 * j, 16 * k);
+                        mma16816(c[0], G[k], wb[0], wb[1]);
+                        mma16816(c[1], G[k], wb[2], wb[3]);
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const int col = 16 * j + 8 * h + 2 * t;
+#pragma unroll
+                        for (int r = 0; r < 2; r++) {
+                            const int64_t row = r0 + g + 8 * r;
+                            const float2 zz = row < n ? ld2(zl + row * kHid + col, vec) : make_float2(0.f, 0.f);
+                            const float av0 = row < n ? gelu(zz.x) : 0.f, av1 = row < n ? gelu(zz.y) : 0.f;
+                            aw32[(row0 + 8 * r) * LW + 8 * j + 4 * h + t] = pack2(av0, av1);
+                            H[j][2 * h + r] = pack2(c[h][2 * r] * gelu_grad(zz.x), c[h][2 * r + 1] * gelu_grad(zz.y));
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 8; j++)
+#pragma unroll
+                    for (int q = 0; q < 4; q++) G[j][q] = H[j][q];
             }
             __syncthreads();
+            // gW[o][i] = sum_r g[r][o] a[r][i]: tiles of 16 outputs x 16 inputs, K = the block's rows
+            const int mt = out_dim / 16, nt = in_dim / 16;
+            float* dst = gw + woff(l);
+            for (int tile = warp; tile < mt * nt; tile += kThreads / 32) {
+                const int o0 = (tile / nt) * 16, i0 = (tile % nt) * 16;
+                float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int k = 0; k < kRows / 16; k++) {
+                    uint32_t ga[4], ab[4];
+                    load_a_trans(ga, S.g, kLdHid, o0, 16 * k);
+                    load_b_trans(ab, S.act, kLdHid, i0, 16 * k);
+                    mma16816(c0, ga, ab[0], ab[1]);
+                    mma16816(c1, ga, ab[2], ab[3]);
+                }
+                add2(dst + (o0 + g) * in_dim + i0 + 2 * t, c0[0], c0[1], vec);
+                add2(dst + (o0 + g + 8) * in_dim + i0 + 2 * t, c0[2], c0[3], vec);
+                add2(dst + (o0 + g) * in_dim + i0 + 8 + 2 * t, c1[0], c1[1], vec);
+                add2(dst + (o0 + g + 8) * in_dim + i0 + 8 + 2 * t, c1[2], c1[3], vec);
+            }
+            if (warp < mt) {   // bias gradient of outputs 16 warp ..: B = ones
+                float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int k = 0; k < kRows / 16; k++) {
+                    uint32_t ga[4];
+                    load_a_trans(ga, S.g, kLdHid, 16 * warp, 16 * k);
+                    mma16816(c, ga, 0x3F803F80u, 0x3F803F80u);
+                }
+                if (t == 0) {
+                    atomicAdd(&gb[boff(l) + 16 * warp + g], c[0]);
+                    atomicAdd(&gb[boff(l) + 16 * warp + g + 8], c[2]);
+                }
+            }
         }
     }
+    lsum = warp_sum(lsum);
+    if (lane == 0 && lsum != 0.0) atomicAdd(loss_sum, lsum);
 }
 
 // Adam on the FP32 master parameters (weights then biases), BF16 copy of the weights,
-// gradients cleared.
+// gradients cleared; the step's loss (loss_out may be null).
 __global__ void mlp_adam_kernel(float* master, bf16* wq, float* bias, float* gw, float* gb, float* m, float* v, float lr,
-                                float b1, float b2, float eps, float bc1, float bc2) {
+                                float b1, float b2, float eps, float bc1, float bc2, const double* loss_sum, int64_t n,
+                                float* loss_out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && loss_out) *loss_out = (float)(*loss_sum / ((double)n * kOutUsed));
     if (i >= kNW + kNB) return;
     const bool is_w = i < kNW;
     float g = is_w ? gw[i] : gb[i - kNW];
@@ -284,9 +394,9 @@ __global__ void mlp_adam_kernel(float* master, bf16* wq, float* bias, float* gw,
     }
 }
 
-static int mlp_grid(int64_t n) {
-    const int sms = device_sms();
-    const int64_t blocks = (n + kRows - 1) / kRows;
+// blocks of kRows rows, at most `per_sm` per SM
+static int mlp_grid(int64_t n, int per_sm) {
+    const int64_t sms = (int64_t)device_sms() * per_sm, blocks = (n + kRows - 1) / kRows;
     return (int)(blocks < sms ? (blocks > 0 ? blocks : 1) : sms);
 }
 
@@ -294,20 +404,15 @@ static bool g_mlp_attr[kMaxDevices] = {};
 static cudaError_t mlp_attrs() {
     return once_per_device(g_mlp_attr, [] {
         cudaError_t e = cudaFuncSetAttribute(mlp_infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sizeof(MlpSmem));
+                                             (int)sizeof(WeightSmem));
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(mlp_train_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sizeof(MlpSmem));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(mlp_train_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sizeof(BwdSmem));
+            e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)sizeof(TrainSmem));
         return e;
     });
 }
 
-__global__ void mlp_loss_finalize_kernel(const double* s, int64_t n, float* out) {
-    if (threadIdx.x == 0) *out = (float)(*s / ((double)n * kOutUsed));
-}
+static bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 
 gs_status record_error(gs_status s, const char* msg);
 
@@ -322,14 +427,14 @@ extern "C" gs_status gs_mlp_infer(const uint16_t* w_bf16, const float* bias, con
     if (!w_bf16 || !bias || !x || !y) return record_error(GS_ERR_INVALID_ARG, "NULL buffer");
     cudaError_t e = mlp_attrs();
     if (e != cudaSuccess) return record_error(GS_ERR_CUDA, cudaGetErrorString(e));
-    mlp_infer_kernel<<<mlp_grid(n), kThreads, sizeof(MlpSmem), (cudaStream_t)stream>>>(
-        reinterpret_cast<const bf16*>(w_bf16), bias, x, n, y);
+    mlp_infer_kernel<<<mlp_grid(n, 2), kThreads, sizeof(WeightSmem), (cudaStream_t)stream>>>(
+        reinterpret_cast<const bf16*>(w_bf16), bias, x, n, y, aligned(w_bf16, 16), aligned(x, 8) && aligned(y, 8));
     e = cudaGetLastError();
     return e == cudaSuccess ? GS_OK : record_error(GS_ERR_CUDA, cudaGetErrorString(e));
 }
 
 extern "C" size_t gs_mlp_train_scratch_size(int64_t n) {
-    // z1..z3 [n][128] FP32, g4 [n][16] FP32, loss sum (double)
+    // z1..z3 [n][128] FP32, 16 unused floats a row, loss sum (double)
     return sizeof(float) * (size_t)n * (3 * 128 + 16) + 256;
 }
 
@@ -348,18 +453,18 @@ extern "C" gs_status gs_mlp_train_step(float* w_master, uint16_t* w_bf16, float*
     float* z1 = static_cast<float*>(scratch);
     float* z2 = z1 + (size_t)n * 128;
     float* z3 = z2 + (size_t)n * 128;
-    float* g4 = z3 + (size_t)n * 128;
+    float* z_end = z3 + (size_t)n * (128 + 16);
     double* lsum = reinterpret_cast<double*>(
-        (reinterpret_cast<uintptr_t>(g4 + (size_t)n * 16) + 15) & ~(uintptr_t)15);
+        (reinterpret_cast<uintptr_t>(z_end) + 15) & ~(uintptr_t)15);
     cudaMemsetAsync(lsum, 0, sizeof(double), st);
     const bf16* wq = reinterpret_cast<const bf16*>(w_bf16);
-    const int grid = mlp_grid(n);
-    mlp_train_fwd_kernel<<<grid, kThreads, sizeof(MlpSmem), st>>>(wq, bias, x, y_target, n, z1, z2, z3, g4, lsum);
-    mlp_train_bwd_kernel<<<grid, kThreads, sizeof(BwdSmem), st>>>(wq, x, n, z1, z2, z3, g4, grad_w, grad_b);
+    mlp_train_kernel<<<mlp_grid(n, 1), kThreads, sizeof(TrainSmem), st>>>(
+        wq, bias, x, y_target, n, z1, z2, z3, grad_w, grad_b, lsum, aligned(w_bf16, 16),
+        aligned(x, 8) && aligned(scratch, 8) && aligned(grad_w, 8));
     const float bc1 = (float)(1.0 - pow((double)b1, (double)step)), bc2 = (float)(1.0 - pow((double)b2, (double)step));
     mlp_adam_kernel<<<(kNW + kNB + 255) / 256, 256, 0, st>>>(w_master, reinterpret_cast<bf16*>(w_bf16), bias, grad_w,
-                                                            grad_b, adam_m, adam_v, lr, b1, b2, eps, bc1, bc2);
-    if (loss_out) mlp_loss_finalize_kernel<<<1, 32, 0, st>>>(lsum, n, loss_out);
+                                                            grad_b, adam_m, adam_v, lr, b1, b2, eps, bc1, bc2, lsum, n,
+                                                            loss_out);
     e = cudaGetLastError();
     return e == cudaSuccess ? GS_OK : record_error(GS_ERR_CUDA, cudaGetErrorString(e));
 }
