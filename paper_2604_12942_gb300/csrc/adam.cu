@@ -15,6 +15,7 @@ __device__ __forceinline__ void adam_one(float& p, float& g, float& m, float& v,
 // grid: (blocks over n in steps of 4*256, total planes).  Plane k of the packed layout
 // (means 3, log-scales 3, quats 4, opacity 1, SH 3K) maps to group pointer and row.
 __global__ void __launch_bounds__(256) adam_kernel(AdamArgs a) {
+    pdl_begin();
     int k = blockIdx.y;
     int grp = 0;
     while (k >= a.planes_of[grp]) { k -= a.planes_of[grp]; grp++; }
@@ -83,7 +84,7 @@ __global__ void __launch_bounds__(256) adam_kernel(AdamArgs a) {
 cudaError_t launch_adam(const AdamArgs& a, cudaStream_t st) {
     if (a.n <= 0) return cudaSuccess;
     const int64_t bx = (a.n + 4 * 256 - 1) / (4 * 256);
-    adam_kernel<<<dim3((unsigned)bx, a.n_planes), 256, 0, st>>>(a);
+    launch_pdl_small(adam_kernel, dim3((unsigned)bx, a.n_planes), 256, 0, st, a);
     return cudaGetLastError();
 }
 

@@ -213,6 +213,7 @@ struct SetupParam {
 static_assert(sizeof(SetupParam) + 8 <= 4096, "kernel parameters");
 
 __global__ void __launch_bounds__(256) setup_kernel(View* dst, const __grid_constant__ SetupParam p) {
+    pdl_begin();
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < p.n; i += blockDim.x) dst[i] = p.v[i];
     for (int k = 0; k < p.n_clear; k++) {
@@ -267,7 +268,7 @@ static int setup_grid(const SetupParam& p) {
 static gs_status run_setup(void* ws, const gs_ws_layout& L, const Geometry& G, int what, cudaStream_t st,
                            float* grad_twist = nullptr) {
     const SetupParam p = setup_param(ws, L, G, what, grad_twist);
-    setup_kernel<<<setup_grid(p), 256, 0, st>>>(at<View>(ws, L.views), p);
+    launch_pdl(setup_kernel, setup_grid(p), 256, 0, st, at<View>(ws, L.views), p);
     GS_CUDA(cudaGetLastError());
     return GS_OK;
 }

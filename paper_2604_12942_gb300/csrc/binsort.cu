@@ -72,6 +72,7 @@ static_assert(kEntryMinWords == 8 * kEntryWarps && kEntryThreads == 32 * kEntryW
 constexpr int kCountWords = 4 * kEntryThreads;
 
 __global__ void __launch_bounds__(kEntryThreads) entry_count_kernel(BinArgs a, int64_t n_words, int wpb, int n_blocks) {
+    pdl_begin();
     constexpr int GT = kEntryMinWords / 4;   // threads per kEntryMinWords words
     __shared__ uint32_t s[kEntryThreads / GT], s_w[33];
     __shared__ bool last;
@@ -128,6 +129,7 @@ __global__ void __launch_bounds__(kEntryThreads) entry_count_kernel(BinArgs a, i
 
 template <int WPW, bool LOOKBACK>
 __global__ void __launch_bounds__(kEntryThreads, 4) entry_compact_kernel(BinArgs a, int64_t n_words) {
+    pdl_begin();
     constexpr int WPB = WPW * kEntryWarps;   // words per block
     __shared__ uint32_t s[33];
     __shared__ uint32_t s_off[WPB], s_word[WPB];
@@ -232,16 +234,16 @@ cudaError_t launch_entries(const BinArgs& a, cudaStream_t st) {
     // the short form while its blocks fit the device a few times over (4 resident per SM)
     const int64_t small = (n_words + kEntryMinWords - 1) / kEntryMinWords, sms = device_sms();
     if (small <= 4 * sms) {
-        entry_compact_kernel<8, true><<<(unsigned)small, kEntryThreads, 0, st>>>(a, n_words);
+        launch_pdl(entry_compact_kernel<8, true>, (unsigned)small, kEntryThreads, 0, st, a, n_words);
         return cudaGetLastError();
     }
     const int wpb = small <= 16 * sms ? kEntryMinWords : 32 * kEntryWarps;
     const int nb = (int)((n_words + wpb - 1) / wpb);
-    entry_count_kernel<<<(unsigned)((n_words + kCountWords - 1) / kCountWords), kEntryThreads, 0, st>>>(a, n_words, wpb, nb);
+    launch_pdl(entry_count_kernel, (unsigned)((n_words + kCountWords - 1) / kCountWords), kEntryThreads, 0, st, a, n_words, wpb, nb);
     if (wpb == kEntryMinWords)
-        entry_compact_kernel<8, false><<<nb, kEntryThreads, 0, st>>>(a, n_words);
+        launch_pdl(entry_compact_kernel<8, false>, nb, kEntryThreads, 0, st, a, n_words);
     else
-        entry_compact_kernel<32, false><<<nb, kEntryThreads, 0, st>>>(a, n_words);
+        launch_pdl(entry_compact_kernel<32, false>, nb, kEntryThreads, 0, st, a, n_words);
     return cudaGetLastError();
 }
 
@@ -260,6 +262,7 @@ __device__ __forceinline__ uint32_t rect_count(uint2 r) { return (r.y & 0xFFFFu)
 // through the sorted compact indices.  The entry count is known only on the device: resident
 // blocks take chunks of kPairScanChunk entries in turn.
 __global__ void __launch_bounds__(kPairScanThreads) pair_offsets_kernel(BinArgs a) {
+    pdl_begin();
     __shared__ uint32_t s[33], s_chunk;
     __shared__ unsigned long long s_base;
     __shared__ bool s_ok;
@@ -357,6 +360,7 @@ __device__ __forceinline__ void hist_add(uint32_t* h, uint32_t d, bool valid) {
 // running maximum over the chunk.  A few entries
 // with very many tiles no longer serialise on one warp.
 __global__ void __launch_bounds__(kEmitThreads) pair_emit_kernel(BinArgs a) {
+    pdl_begin();
     static_assert(kEmitChunk == 8 * kEmitThreads, "each thread owns 8 consecutive slots of the chunk");
     __shared__ uint32_t s_off[kEmitChunk + 1], s_t0[kEmitChunk + 1], s_id[kEmitChunk + 1];
     __shared__ uint16_t s_wx[kEmitChunk + 1], s_tx[kEmitChunk + 1];
@@ -458,14 +462,14 @@ cudaError_t launch_emit(const BinArgs& a, cudaStream_t st) {
     const int64_t nb = ((int64_t)a.n_views * a.n + kPairScanChunk - 1) / kPairScanChunk;   // at most
     if (nb > 0) {
         const int64_t g = resident_grid(g_offsets, pair_offsets_kernel, kPairScanThreads);
-        pair_offsets_kernel<<<(unsigned)(g < nb ? g : nb), kPairScanThreads, 0, st>>>(a);
+        launch_pdl(pair_offsets_kernel, (unsigned)(g < nb ? g : nb), kPairScanThreads, 0, st, a);
     }
     // one chunk of kEmitChunk pairs per block and turn; the pair count is known only on the
     // device, so the grid is the resident one (capped by the capacity's chunks)
     const int64_t emit_chunks = (a.max_pairs + kEmitChunk - 1) / kEmitChunk;
     const int64_t ge = resident_grid(g_emit, pair_emit_kernel, kEmitThreads);
     const int64_t emit_grid = emit_chunks < ge ? emit_chunks : ge;
-    pair_emit_kernel<<<(unsigned)(emit_grid > 0 ? emit_grid : 1), kEmitThreads, 0, st>>>(a);
+    launch_pdl(pair_emit_kernel, (unsigned)(emit_grid > 0 ? emit_grid : 1), kEmitThreads, 0, st, a);
     return cudaGetLastError();
 }
 
@@ -634,6 +638,7 @@ __device__ __forceinline__ uint32_t lb_sum(const W* col, int bits, int64_t last,
 template <typename K, int BITS>
 __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSM)
     sort_pass_kernel(SortArgs a, int in_buf, int shift, int pass, int next_shift, uint32_t next_mask) {
+    pdl_begin();
     constexpr int BINS = 1 << BITS;
     constexpr int DPT = (BINS + kSortThreads - 1) / kSortThreads;   // digits per thread
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -839,7 +844,7 @@ static cudaError_t launch_pass(const SortArgs& a, int in_buf, int shift, int pas
         return cudaFuncSetAttribute(sort_pass_kernel<K, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
-    sort_pass_kernel<K, BITS><<<sort_grid(a.capacity), kSortThreads, smem, st>>>(a, in_buf, shift, pass, next_shift,
+    launch_pdl(sort_pass_kernel<K, BITS>, sort_grid(a.capacity), kSortThreads, smem, st, a, in_buf, shift, pass, next_shift,
                                                                               next_mask);
     return cudaGetLastError();
 }
@@ -881,6 +886,7 @@ cudaError_t launch_sort_count64(const SortArgs& a, int shift, cudaStream_t st) {
 // (from the previous lane, or loaded by lane 0); a start boundary j (key[j] != key[j - 1])
 // opens key[j]'s range and closes key[j - 1]'s.
 __global__ void __launch_bounds__(256) ranges_kernel(RangeArgs a) {
+    pdl_begin();
     if (a.counters->status != 0) return;
     const int64_t P = (int64_t)a.counters->n_pairs;
     const int64_t groups = (P + 3) / 4;
@@ -914,7 +920,7 @@ __global__ void __launch_bounds__(256) ranges_kernel(RangeArgs a) {
 
 cudaError_t launch_ranges(const RangeArgs& a, int n_tiles, cudaStream_t st) {
     (void)n_tiles;
-    ranges_kernel<<<device_sms() * 12, 256, 0, st>>>(a);
+    launch_pdl(ranges_kernel, device_sms() * 12, 256, 0, st, a);
     return cudaGetLastError();
 }
 
@@ -931,6 +937,7 @@ __device__ __forceinline__ int order_bucket(uint2 r) {
 // Bucket counts; the last block to finish turns them into the buckets' first positions, largest
 // counts first (tmp: counts, then positions, then the blocks done).
 __global__ void tile_order_hist_kernel(const uint2* ranges, int n_tiles, uint32_t* tmp, const Counters* c) {
+    pdl_begin();
     __shared__ uint32_t h[kOrderBuckets];
     __shared__ bool last;
     for (int b = threadIdx.x; b < kOrderBuckets; b += blockDim.x) h[b] = 0;
@@ -960,6 +967,7 @@ __global__ void tile_order_hist_kernel(const uint2* ranges, int n_tiles, uint32_
 
 __global__ void tile_order_scatter_kernel(const uint2* ranges, int n_tiles, uint32_t* cursor, uint32_t* order,
                                           const Counters* c) {
+    pdl_begin();
     const int lane = threadIdx.x & 31;
     for (int t0 = blockIdx.x * blockDim.x; t0 < n_tiles; t0 += gridDim.x * blockDim.x) {
         const int t = t0 + threadIdx.x;
@@ -979,8 +987,8 @@ cudaError_t launch_tile_order(const uint2* ranges, int n_tiles, uint32_t* order,
                               cudaStream_t st) {
     if (n_tiles <= 0) return cudaSuccess;
     const int blocks = (n_tiles + 255) / 256 < 1024 ? (n_tiles + 255) / 256 : 1024;
-    tile_order_hist_kernel<<<blocks, 256, 0, st>>>(ranges, n_tiles, tmp, c);
-    tile_order_scatter_kernel<<<blocks, 256, 0, st>>>(ranges, n_tiles, tmp + kOrderBuckets, order, c);
+    launch_pdl(tile_order_hist_kernel, blocks, 256, 0, st, ranges, n_tiles, tmp, c);
+    launch_pdl(tile_order_scatter_kernel, blocks, 256, 0, st, ranges, n_tiles, tmp + kOrderBuckets, order, c);
     return cudaGetLastError();
 }
 

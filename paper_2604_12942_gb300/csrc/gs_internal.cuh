@@ -54,6 +54,55 @@ inline int device_sms() {
     return sms > 0 ? sms : 148;
 }
 
+// Programmatic dependent launch of the kernels of a step: each starts with pdl_begin(), which
+// waits until the kernels before it have completed (every block does, before it reads or writes
+// anything and before it may exit, so that completion carries along the chain) and then lets
+// the next kernel's blocks be scheduled as soon as all of this kernel's have been, instead of
+// after its last one has finished.  That takes about 1.3 us off a kernel boundary of a stream.  A
+// graph's plain edges are cheaper than its programmatic ones (a captured step of 500k Gaussians
+// took 676 us with them, 658 without), so a captured launch is a plain one.
+//
+// It is not free for a kernel that needs an SM's shared memory: its first blocks arrive while the
+// kernel before still holds the SM to its own split of L1 and shared memory, and as blocks follow
+// blocks the split stays, with fewer blocks resident than the kernel could have.  So the kernels of
+// many blocks that live on shared memory (compositing, the SH and geometry parts, SSIM) take a
+// plain launch unless their grid is small: with all of them launched this way the step took
+// 712 against 658 us at 500k Gaussians and 1448 against 1286 at 1M, while 10k went from 181 to 150.
+__device__ __forceinline__ void pdl_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        kernel<<<grid, block, smem, st>>>(static_cast<P>(args)...);
+        return cudaGetLastError();
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// launch_pdl for a grid of at most kPdlBlocksPerSM blocks per SM, else a plain launch.
+constexpr int kPdlBlocksPerSM = 4;
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl_small(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+    if ((int64_t)grid.x * grid.y * grid.z <= (int64_t)kPdlBlocksPerSM * device_sms())
+        return launch_pdl(kernel, grid, block, smem, st, static_cast<A&&>(args)...);
+    kernel<<<grid, block, smem, st>>>(static_cast<P>(args)...);
+    return cudaGetLastError();
+}
+
 // Per-view table held in the workspace.
 struct View {
     int32_t W, H, tiles_x, tiles_y;

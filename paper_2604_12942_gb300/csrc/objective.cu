@@ -27,6 +27,7 @@ constexpr float kSsimC1 = 0.01f * 0.01f, kSsimC2 = 0.03f * 0.03f;
 // halo of r once into shared memory, then every pixel tests the disk there.
 constexpr int kMaskMaxR = 16;
 __global__ void __launch_bounds__(kObjTX * kObjTY) render_mask_kernel(ObjArgs a) {
+    pdl_begin();
     __shared__ uint8_t s_geo[kObjTY + 2 * kMaskMaxR][kObjTX + 2 * kMaskMaxR];
     __shared__ int s_w[2 * kMaskMaxR + 1];   // half-width of the disk in each row
     const View& V = a.views[blockIdx.z];
@@ -85,6 +86,7 @@ __device__ __forceinline__ void block_add2(float s0, float s1, double* dst0, dou
 
 // Masked L1 terms: the same arithmetic as the forward's fused epilogue, on a given mask.
 __global__ void __launch_bounds__(kObjTX * kObjTY) masked_l1_kernel(ObjArgs a) {
+    pdl_begin();
     const int v = blockIdx.z;
     const View& V = a.views[v];
     const int x = blockIdx.x * kObjTX + threadIdx.x, y = blockIdx.y * kObjTY + threadIdx.y;
@@ -153,6 +155,7 @@ __device__ __forceinline__ void hconv(const float (&win)[11], const float (&v)[1
 // (the gradient of lambda_ssim (1 - SSIM) / views); and at the same output pixels the L1
 // colour terms (and, with the first channel, the depth term) with the epilogue's arithmetic.
 __global__ void __launch_bounds__(kObjTX * kObjTY) ssim_fwd_kernel(ObjArgs a) {
+    pdl_begin();
     __shared__ __align__(16) float s_x[3][kInH][kInS];
     __shared__ __align__(16) float s_y[3][kInH][kInS];
     // horizontal sums of x, y, x^2 + y^2 and xy (SSIM needs E[x^2] and E[y^2] only summed)
@@ -266,6 +269,7 @@ __global__ void __launch_bounds__(kObjTX * kObjTY) ssim_fwd_kernel(ObjArgs a) {
 // dL/dC = M dL/dx, added to the L1 gradient already in dl_drgb.  The three partial maps of a
 // channel are loaded together; channels are processed one after the other.
 __global__ void __launch_bounds__(kObjTX * kObjTY) ssim_bwd_kernel(ObjArgs a) {
+    pdl_begin();
     __shared__ __align__(16) float s_p[3][kInH][kInS];
     __shared__ __align__(16) float s_h[3][kInH][kObjTX];
     const View& V = a.views[blockIdx.z];
@@ -331,7 +335,7 @@ static dim3 obj_grid(const ObjArgs& a, int tile_h) {
 
 cudaError_t launch_render_mask(const ObjArgs& a, cudaStream_t st) {
     if (a.n_views <= 0) return cudaSuccess;
-    render_mask_kernel<<<obj_grid(a, kObjTY), dim3(kObjTX, kObjTY), 0, st>>>(a);
+    launch_pdl_small(render_mask_kernel, obj_grid(a, kObjTY), dim3(kObjTX, kObjTY), 0, st, a);
     return cudaGetLastError();
 }
 
@@ -339,10 +343,10 @@ cudaError_t launch_objective(const ObjArgs& a, cudaStream_t st) {
     if (a.n_views <= 0) return cudaSuccess;
     if (a.lambda_ssim > 0.f) {
         // (the L1 terms ride along in the SSIM forward, which holds C and C~ at every pixel)
-        ssim_fwd_kernel<<<obj_grid(a, kObjH), dim3(kObjTX, kObjTY), 0, st>>>(a);
-        ssim_bwd_kernel<<<obj_grid(a, kObjH), dim3(kObjTX, kObjTY), 0, st>>>(a);
+        launch_pdl_small(ssim_fwd_kernel, obj_grid(a, kObjH), dim3(kObjTX, kObjTY), 0, st, a);
+        launch_pdl_small(ssim_bwd_kernel, obj_grid(a, kObjH), dim3(kObjTX, kObjTY), 0, st, a);
     } else {
-        masked_l1_kernel<<<obj_grid(a, kObjTY), dim3(kObjTX, kObjTY), 0, st>>>(a);
+        launch_pdl_small(masked_l1_kernel, obj_grid(a, kObjTY), dim3(kObjTX, kObjTY), 0, st, a);
     }
     return cudaGetLastError();
 }

@@ -13,6 +13,7 @@ static_assert(sizeof(View) % 4 == 0, "the view table is copied in 4-byte words")
 
 template <int DEG>
 __global__ void __launch_bounds__(128, 8) project_kernel(ProjectArgs a) {
+    pdl_begin();
     constexpr int K = (DEG + 1) * (DEG + 1);
     // the view table in shared memory: every thread walks all views, and the streamed planes
     // leave little of it in L1 (0.142 -> 0.136 ms at 2M Gaussians, 8 views)
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(128, 8) project_kernel(ProjectArgs a) {
 namespace gs {
 
 __global__ void __launch_bounds__(kEntryThreads) project_bwd_entry_kernel(ProjectBwdArgs a) {
+    pdl_begin();
     __shared__ float s_tw[GS_MAX_VIEWS * 6];
     project_bwd_entry_part(a, blockIdx.x, gridDim.x, s_tw);
 }
@@ -134,6 +136,7 @@ constexpr int kRowThreads = 64;
 
 template <int DEG, bool FUSED_ADAM>
 __global__ void __launch_bounds__(kRowThreads, 10) project_bwd_sh_kernel(ProjectBwdArgs a) {
+    pdl_begin();
     __shared__ float s_tw[GS_MAX_VIEWS * 6];
     __shared__ float s_cam[GS_MAX_VIEWS * 12];
     __shared__ float s_mv[FUSED_ADAM ? sh_mv_floats<DEG, kRowThreads>() : 1];
@@ -142,6 +145,7 @@ __global__ void __launch_bounds__(kRowThreads, 10) project_bwd_sh_kernel(Project
 
 template <int DEG, bool FUSED_ADAM>
 __global__ void __launch_bounds__(kRowThreads, 16) project_bwd_geo_kernel(ProjectBwdArgs a) {
+    pdl_begin();
     __shared__ float s_mv[FUSED_ADAM ? geo_mv_floats<kRowThreads>() : 1];
     project_bwd_geo_rows<DEG, FUSED_ADAM, kRowThreads>(a, blockIdx.x, s_mv);
 }
@@ -152,18 +156,18 @@ cudaError_t launch_project(const ProjectArgs& a, int deg, cudaStream_t st) {
     const unsigned blocks = (unsigned)((a.n + threads - 1) / threads);
     if (blocks == 0) return cudaSuccess;
     switch (deg) {
-        case 0: project_kernel<0><<<blocks, threads, 0, st>>>(a); break;
-        case 1: project_kernel<1><<<blocks, threads, 0, st>>>(a); break;
-        case 2: project_kernel<2><<<blocks, threads, 0, st>>>(a); break;
-        default: project_kernel<3><<<blocks, threads, 0, st>>>(a); break;
+        case 0: launch_pdl(project_kernel<0>, blocks, threads, 0, st, a); break;
+        case 1: launch_pdl(project_kernel<1>, blocks, threads, 0, st, a); break;
+        case 2: launch_pdl(project_kernel<2>, blocks, threads, 0, st, a); break;
+        default: launch_pdl(project_kernel<3>, blocks, threads, 0, st, a); break;
     }
     return cudaGetLastError();
 }
 
 template <int DEG, bool FUSED_ADAM>
 static cudaError_t launch_project_bwd_d(const ProjectBwdArgs& a, unsigned blocks, cudaStream_t st) {
-    project_bwd_sh_kernel<DEG, FUSED_ADAM><<<blocks, kRowThreads, 0, st>>>(a);
-    project_bwd_geo_kernel<DEG, FUSED_ADAM><<<blocks, kRowThreads, 0, st>>>(a);
+    launch_pdl_small(project_bwd_sh_kernel<DEG, FUSED_ADAM>, blocks, kRowThreads, 0, st, a);
+    launch_pdl_small(project_bwd_geo_kernel<DEG, FUSED_ADAM>, blocks, kRowThreads, 0, st, a);
     return cudaGetLastError();
 }
 
@@ -182,7 +186,7 @@ static cudaError_t launch_project_bwd_t(const ProjectBwdArgs& a, int deg, cudaSt
 cudaError_t launch_project_bwd(const ProjectBwdArgs& a, int deg, cudaStream_t st) {
     // entry part (persistent grid over the device-side entry count), then the row part's SH
     // and geometry kernels
-    project_bwd_entry_kernel<<<device_sms() * 12, kEntryThreads, 0, st>>>(a);
+    launch_pdl(project_bwd_entry_kernel, device_sms() * 12, kEntryThreads, 0, st, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return a.fused_adam ? launch_project_bwd_t<true>(a, deg, st) : launch_project_bwd_t<false>(a, deg, st);

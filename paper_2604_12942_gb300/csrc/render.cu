@@ -24,6 +24,7 @@ __device__ __forceinline__ int view_of_tile(const View* views, int n_views, int 
 // ----------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) loss_count_kernel(const View* views, const float* tgt_depth,
                                                          const uint8_t* mask, uint32_t* counts) {
+    pdl_begin();
     const int v = blockIdx.y;
     const View& V = views[v];
     const int64_t P = (int64_t)V.W * V.H;
@@ -81,13 +82,14 @@ cudaError_t launch_loss_count(const View* views, int n_views, const int64_t* pix
 
 __global__ void loss_finalize_kernel(const double* sums, const uint32_t* counts, int n_views, float lambda_rgb,
                                      float lambda_depth, float lambda_ssim, int has_depth, float* loss_out) {
+    pdl_begin();
     if (threadIdx.x == 0)
         loss_finalize_one(sums, counts, n_views, lambda_rgb, lambda_depth, lambda_ssim, has_depth, loss_out);
 }
 
 cudaError_t launch_loss_finalize(const double* sums, const uint32_t* counts, int n_views, float lambda_rgb,
                                  float lambda_depth, float lambda_ssim, int has_depth, float* loss_out, cudaStream_t st) {
-    loss_finalize_kernel<<<1, 32, 0, st>>>(sums, counts, n_views, lambda_rgb, lambda_depth, lambda_ssim, has_depth,
+    launch_pdl(loss_finalize_kernel, 1, 32, 0, st, sums, counts, n_views, lambda_rgb, lambda_depth, lambda_ssim, has_depth,
                                            loss_out);
     return cudaGetLastError();
 }
@@ -489,6 +491,7 @@ __device__ __forceinline__ void render_fwd_tile(const FwdArgs& a, int item, FwdS
 template <int TILE, int CHUNK, bool COUNT>
 __global__ void __launch_bounds__(TileMap<TILE, kFwdPPT>::NT, kFwdThreadsPerSM / TileMap<TILE, kFwdPPT>::NT)
     render_fwd_kernel(FwdArgs a) {
+    pdl_begin();
     __shared__ FwdSmem<TILE, CHUNK> S;
     render_fwd_tile<TILE, CHUNK, COUNT>(a, blockIdx.x, S);
 }
@@ -558,6 +561,7 @@ __device__ __forceinline__ void warp_reduce10(float (&v)[10], float& out8, float
 
 template <int TILE, int CHUNK, bool COUNT>
 __global__ void __launch_bounds__(TileMap<TILE, kBwdPPT>::NT) render_bwd_kernel(BwdArgs a) {
+    pdl_begin();
     constexpr int kPPT = kBwdPPT;
     using TM = TileMap<TILE, kPPT>;
     constexpr int NT = TM::NT;
@@ -985,6 +989,7 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
 
 template <bool COUNT>
 __global__ void __launch_bounds__(32, 32) render_bwd_warp_kernel(BwdArgs a) {
+    pdl_begin();
     __shared__ BwdWarpSmem S;
     render_bwd_region<COUNT>(a, blockIdx.x, S);
 }
@@ -992,8 +997,11 @@ __global__ void __launch_bounds__(32, 32) render_bwd_warp_kernel(BwdArgs a) {
 template <int TILE, int CHUNK>
 static void launch_fwd_c(const FwdArgs& a, int total_tiles, cudaStream_t st) {
     constexpr int NT = TileMap<TILE, kFwdPPT>::NT;
-    if (a.op.count) render_fwd_kernel<TILE, CHUNK, true><<<total_tiles, NT, 0, st>>>(a);
-    else render_fwd_kernel<TILE, CHUNK, false><<<total_tiles, NT, 0, st>>>(a);
+    // (without a target the kernel may follow the join of a captured step's upload branch: a plain
+    // launch there, as of the loss count that follows it otherwise)
+    auto kernel = a.op.count ? render_fwd_kernel<TILE, CHUNK, true> : render_fwd_kernel<TILE, CHUNK, false>;
+    if (a.tgt_rgb) launch_pdl_small(kernel, total_tiles, NT, 0, st, a);
+    else kernel<<<total_tiles, NT, 0, st>>>(a);
 }
 
 template <int TILE>
@@ -1010,8 +1018,8 @@ static cudaError_t launch_fwd_t(const FwdArgs& a, int total_tiles, int chunk, cu
 template <int TILE, int CHUNK>
 static void launch_bwd_c(const BwdArgs& a, int total_tiles, cudaStream_t st) {
     constexpr int NT = TileMap<TILE, kBwdPPT>::NT;
-    if (a.op.count) render_bwd_kernel<TILE, CHUNK, true><<<total_tiles, NT, 0, st>>>(a);
-    else render_bwd_kernel<TILE, CHUNK, false><<<total_tiles, NT, 0, st>>>(a);
+    if (a.op.count) launch_pdl_small(render_bwd_kernel<TILE, CHUNK, true>, total_tiles, NT, 0, st, a);
+    else launch_pdl_small(render_bwd_kernel<TILE, CHUNK, false>, total_tiles, NT, 0, st, a);
 }
 
 template <int TILE>
@@ -1043,6 +1051,7 @@ cudaError_t launch_render_fwd(const FwdArgs& a, int total_tiles, cudaStream_t st
 // as the separate loss kernel) and its Adam step counter (adam_ctr non-null).
 __global__ void __launch_bounds__(256) clear_grad2d_kernel(BwdArgs a, Counters* adam_ctr, float b1, float b2,
                                                            LossFinal lf) {
+    pdl_begin();
     if (lf.loss_out && blockIdx.x == 0 && threadIdx.x == 0)
         loss_finalize_one(lf.sums, lf.counts, lf.n_views, lf.lambda_rgb, lf.lambda_depth, 0.f, lf.has_depth,
                           lf.loss_out);
@@ -1066,12 +1075,12 @@ __global__ void __launch_bounds__(256) clear_grad2d_kernel(BwdArgs a, Counters* 
 
 cudaError_t launch_render_bwd(const BwdArgs& a, int total_tiles, cudaStream_t st, Counters* adam_ctr, float b1,
                               float b2, const LossFinal& lf) {
-    clear_grad2d_kernel<<<device_sms() * 12, 256, 0, st>>>(a, adam_ctr, b1, b2, lf);
+    launch_pdl(clear_grad2d_kernel, device_sms() * 12, 256, 0, st, a, adam_ctr, b1, b2, lf);
     if (total_tiles <= 0) return cudaGetLastError();
     // 16 x 16 tiles: one independent warp per 8 x 8 region (8 x 8 tiles are one warp already)
     if (a.op.tile == 16) {
-        if (a.op.count) render_bwd_warp_kernel<true><<<4 * total_tiles, 32, 0, st>>>(a);
-        else render_bwd_warp_kernel<false><<<4 * total_tiles, 32, 0, st>>>(a);
+        if (a.op.count) launch_pdl_small(render_bwd_warp_kernel<true>, 4 * total_tiles, 32, 0, st, a);
+        else launch_pdl_small(render_bwd_warp_kernel<false>, 4 * total_tiles, 32, 0, st, a);
         return cudaGetLastError();
     }
     return launch_bwd_t<8>(a, total_tiles, a.op.chunk, st);
