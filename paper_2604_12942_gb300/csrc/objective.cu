@@ -23,44 +23,57 @@ constexpr int kInW = kObjTX + 2 * kHalo, kInH = kObjH + 2 * kHalo;
 constexpr float kSsimC1 = 0.01f * 0.01f, kSsimC2 = 0.03f * 0.03f;
 
 // Interior mask: [1 - T >= tau] eroded by the radius-r disk (outside the image counts as
-// outside the support), and the caller's mask.  The block thresholds its 32 x 8 pixels and a
-// halo of r once into shared memory, then every pixel tests the disk there.
+// outside the support), and the caller's mask.  A block takes 32 x 32 pixels: a warp thresholds a
+// row of them and 16 pixels either side into one 64-bit word (two ballots), and a pixel then
+// tests each row of the disk as a run of bits, one 64-bit operation a row.  (With bytes
+// in shared memory, 13 tests at radius 2, it took 38 us for 3.1 Mpx, now 26.)
 constexpr int kMaskMaxR = 16;
+constexpr int kMaskRows = 4, kMaskH = kObjTY * kMaskRows;   // rows per thread and per block
 __global__ void __launch_bounds__(kObjTX * kObjTY) render_mask_kernel(ObjArgs a) {
     pdl_begin();
-    __shared__ uint8_t s_geo[kObjTY + 2 * kMaskMaxR][kObjTX + 2 * kMaskMaxR];
+    __shared__ unsigned long long s_row[kMaskH + 2 * kMaskMaxR];
     __shared__ int s_w[2 * kMaskMaxR + 1];   // half-width of the disk in each row
     const View& V = a.views[blockIdx.z];
-    const int x0 = blockIdx.x * kObjTX, y0 = blockIdx.y * kObjTY;
+    const int x0 = blockIdx.x * kObjTX, y0 = blockIdx.y * kMaskH;
     if (x0 >= V.W || y0 >= V.H) return;   // (the whole block)
     const int r = a.r_erode;
-    const int tw = kObjTX + 2 * r, th = kObjTY + 2 * r;
     const float* T = a.T_final + V.pix_off;
-    const int t = threadIdx.y * kObjTX + threadIdx.x;
+    const int lane = threadIdx.x, w = threadIdx.y, t = w * kObjTX + lane;
     if (t <= 2 * r) {
         const int dy = t - r;
-        int w = 0;
-        while ((w + 1) * (w + 1) + dy * dy <= r * r) w++;
-        s_w[t] = w;
+        int k = 0;
+        while ((k + 1) * (k + 1) + dy * dy <= r * r) k++;
+        s_w[t] = k;
     }
-    for (int i = t; i < tw * th; i += kObjTX * kObjTY) {
-        const int iy = i / tw, ix = i - iy * tw;
-        const int gx = x0 - r + ix, gy = y0 - r + iy;
-        const bool inside = gx >= 0 && gx < V.W && gy >= 0 && gy < V.H;
-        s_geo[iy][ix] = inside && __fsub_rn(1.f, __ldg(T + (int64_t)gy * V.W + gx)) >= a.tau;
+    for (int iy = w; iy < kMaskH + 2 * r; iy += kObjTY) {
+        const int gy = y0 - r + iy;
+        uint32_t bits[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int gx = x0 - kMaskMaxR + 32 * h + lane;
+            const bool inside = gx >= 0 && gx < V.W && gy >= 0 && gy < V.H;
+            const bool geo = inside && __fsub_rn(1.f, __ldg(T + (int64_t)gy * V.W + gx)) >= a.tau;
+            bits[h] = __ballot_sync(0xffffffffu, geo);
+        }
+        if (lane == 0) s_row[iy] = (unsigned long long)bits[1] << 32 | bits[0];
     }
     __syncthreads();
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-    if (x >= V.W || y >= V.H) return;
-    bool in = true;
-    for (int dy = -r; dy <= r; dy++) {
-        const int w = s_w[dy + r];   // the largest w with w^2 + dy^2 <= r^2
-        const uint8_t* row = &s_geo[threadIdx.y + r + dy][threadIdx.x + r];
-        for (int dx = -w; dx <= w; dx++) in = in && row[dx];
+    const int x = x0 + lane;
+    if (x >= V.W) return;
+#pragma unroll
+    for (int k = 0; k < kMaskRows; k++) {
+        const int oy = w * kMaskRows + k, y = y0 + oy;
+        if (y >= V.H) return;
+        bool in = true;
+        for (int dy = -r; dy <= r; dy++) {
+            const int hw = s_w[dy + r];   // the largest half-width with hw^2 + dy^2 <= r^2
+            const unsigned long long run = (1ull << (2 * hw + 1)) - 1ull;
+            in = in && ((s_row[oy + r + dy] >> (lane + kMaskMaxR - hw)) & run) == run;
+        }
+        const int64_t g = V.pix_off + (int64_t)y * V.W + x;
+        if (a.caller_mask) in = in && a.caller_mask[g] != 0;
+        a.mask_out[g] = in ? 1 : 0;
     }
-    const int64_t g = V.pix_off + (int64_t)y * V.W + x;
-    if (a.caller_mask) in = in && a.caller_mask[g] != 0;
-    a.mask_out[g] = in ? 1 : 0;
 }
 
 // Block sums of two per-thread values, one FP64 atomic each (every thread of the block calls
@@ -335,7 +348,7 @@ static dim3 obj_grid(const ObjArgs& a, int tile_h) {
 
 cudaError_t launch_render_mask(const ObjArgs& a, cudaStream_t st) {
     if (a.n_views <= 0) return cudaSuccess;
-    launch_pdl_small(render_mask_kernel, obj_grid(a, kObjTY), dim3(kObjTX, kObjTY), 0, st, a);
+    launch_pdl_small(render_mask_kernel, obj_grid(a, kMaskH), dim3(kObjTX, kObjTY), 0, st, a);
     return cudaGetLastError();
 }
 
