@@ -315,7 +315,7 @@ gs_status gs_objective(const gs_camera *cams, const gs_render_opts *opts, const 
 
 /* f2 -- Map-size updates between mapping iterations (§III-C, optimization: new Gaussians pass
  * a 3-D Euclidean proximity test before insertion; low-opacity Gaussians are pruned under a
- * bounded removal ratio).  The three calls below read counts back and so synchronize `stream`.
+ * bounded removal ratio).  The calls below read counts back and so synchronize `stream`.
  * They share one caller-owned device scratch buffer of gs_map_update_scratch_bytes(n_map,
  * n_new) bytes (256-byte multiple); calls that overlap on the GPU must not share it. */
 size_t gs_map_update_scratch_bytes(int64_t n_map, int64_t n_new);
@@ -335,6 +335,12 @@ gs_status gs_prune_plan(const gs_gaussians *g, float opacity_min, double max_rat
 gs_status gs_dedup_plan(const gs_gaussians *map, const float *new_means, int64_t n_new, float radius,
                         uint8_t *accept, void *scratch, size_t scratch_bytes, int64_t *n_accept,
                         void *stream);
+
+/* Rows that gs_map_update with these flags keeps and accepts (accept NULL: all n_new), for the
+ * caller to size its outputs. */
+gs_status gs_map_update_counts(const uint8_t *keep, int64_t n, const uint8_t *accept, int64_t n_new,
+                               void *scratch, size_t scratch_bytes, int64_t *n_keep,
+                               int64_t *n_accept, void *stream);
 
 /* Update: out = the rows of `in` with keep != 0, in order, then the rows of new_rows (may be
  * NULL) with accept != 0 (accept may be NULL = all), in order; m_out / v_out carry the kept

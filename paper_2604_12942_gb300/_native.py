@@ -109,6 +109,8 @@ _SIGS = {
                        C.POINTER(C.c_int64), C.c_void_p], C.c_int),
     "gs_dedup_plan": ([C.POINTER(Gaussians), C.c_void_p, C.c_int64, C.c_float, C.c_void_p, C.c_void_p, C.c_size_t,
                        C.POINTER(C.c_int64), C.c_void_p], C.c_int),
+    "gs_map_update_counts": ([C.c_void_p, C.c_int64, C.c_void_p, C.c_int64, C.c_void_p, C.c_size_t,
+                              C.POINTER(C.c_int64), C.POINTER(C.c_int64), C.c_void_p], C.c_int),
     "gs_map_update": ([C.POINTER(Gaussians)] * 3 + [C.c_void_p, C.POINTER(Gaussians), C.c_void_p, C.c_void_p, C.c_void_p] +
                       [C.POINTER(Gaussians)] * 3 + [C.c_void_p, C.c_void_p, C.c_size_t, C.c_void_p], C.c_int),
     "gs_gicp_scratch_bytes": ([C.c_int64], C.c_size_t),

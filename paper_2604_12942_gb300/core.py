@@ -451,12 +451,16 @@ def map_update(planes, m, v, sh_degree, keep, new_planes=None, accept=None, tags
     moments)."""
     n = planes.shape[1]
     n_new = 0 if new_planes is None else new_planes.shape[1]
-    n_out = int(keep.sum()) + (0 if new_planes is None else (n_new if accept is None else int(accept.sum())))
     P = planes.shape[0]
     dev = planes.device
+    scratch = map_update_scratch(n, n_new, dev) if scratch is None else scratch
+    nk, na = C.c_int64(), C.c_int64()
+    N.check(N.lib().gs_map_update_counts(_ptr(keep), n, _ptr(accept) if new_planes is not None else None, n_new,
+                                         _ptr(scratch), scratch.numel(), C.byref(nk), C.byref(na), _stream()),
+            "gs_map_update_counts")
+    n_out = nk.value + na.value
     out, m_out, v_out = (torch.empty(P, n_out, device=dev) for _ in range(3))
     tags_out = torch.empty(n_out, dtype=torch.int32, device=dev) if tags is not None else None
-    scratch = map_update_scratch(n, n_new, dev) if scratch is None else scratch
     gs_ = [gaussians_struct(t, sh_degree) for t in (planes, m, v)]
     go = [gaussians_struct(t, sh_degree) for t in (out, m_out, v_out)]
     gn = gaussians_struct(new_planes.contiguous(), sh_degree) if new_planes is not None else None

@@ -1182,6 +1182,23 @@ gs_status gs_dedup_plan(const gs_gaussians* map, const float* new_means, int64_t
     return GS_OK;
 }
 
+gs_status gs_map_update_counts(const uint8_t* keep, int64_t n, const uint8_t* accept, int64_t n_new, void* scratch,
+                               size_t scratch_bytes, int64_t* n_keep, int64_t* n_accept, void* stream) {
+    if (n < 0 || n_new < 0 || (n > 0 && !keep) || !scratch || !n_keep || !n_accept)
+        return fail(GS_ERR_INVALID_ARG, "keep, scratch, n_keep and n_accept are required");
+    if (n >= (int64_t)0x7FFFFFFFll || n_new >= (int64_t)0x7FFFFFFFll) return fail(GS_ERR_INVALID_ARG, "sizes must be < 2^31");
+    if (scratch_bytes < map_update_scratch_bytes(n, n_new)) return fail(GS_ERR_INVALID_ARG, "scratch too small");
+    cudaStream_t st = (cudaStream_t)stream;
+    uint32_t totals[2] = {0, 0};
+    const uint32_t* pos = nullptr;
+    GS_CUDA(launch_map_scan(keep, n, accept, n_new, scratch, &pos, totals, st));
+    const gs_status s = sync_counts(st);
+    if (s != GS_OK) return s;
+    *n_keep = (int64_t)totals[0];
+    *n_accept = accept ? (int64_t)totals[1] : n_new;
+    return GS_OK;
+}
+
 gs_status gs_map_update(const gs_gaussians* in, const gs_gaussians* m_in, const gs_gaussians* v_in, const uint8_t* keep,
                         const gs_gaussians* new_rows, const uint8_t* accept, const uint32_t* tags_in,
                         const uint32_t* new_tags, gs_gaussians* out, gs_gaussians* m_out, gs_gaussians* v_out,
@@ -1204,15 +1221,15 @@ gs_status gs_map_update(const gs_gaussians* in, const gs_gaussians* m_in, const 
     MapUpdateArgs a;
     memset(&a, 0, sizeof(a));
     uint32_t totals[2] = {0, 0};
-    uint32_t *pk = nullptr, *pn = nullptr;
-    GS_CUDA(launch_map_scan(keep, in->n, new_rows ? accept : nullptr, n_new, scratch, &pk, &pn, totals, st));
+    const uint32_t* pos = nullptr;
+    GS_CUDA(launch_map_scan(keep, in->n, new_rows ? accept : nullptr, n_new, scratch, &pos, totals, st));
     if ((s = sync_counts(st)) != GS_OK) return s;
     const int64_t n_acc = new_rows ? (accept ? (int64_t)totals[1] : n_new) : 0;
     if (out->n != (int64_t)totals[0] + n_acc)
         return fail(GS_ERR_INVALID_ARG, "out->n must be %lld (kept %u + accepted %lld), got %lld",
                     (long long)((int64_t)totals[0] + n_acc), totals[0], (long long)n_acc, (long long)out->n);
     a.n = in->n; a.n_new = n_new; a.n_out = out->n; a.n_keep = totals[0];
-    a.keep = keep; a.accept = new_rows ? accept : nullptr; a.pos_keep = pk; a.pos_new = pn;
+    a.keep = keep; a.accept = new_rows ? accept : nullptr; a.chunk_pos = pos;
     a.n_planes = map_planes(in, in->n, a.in);
     map_planes(m_in, in->n, a.m_in);
     map_planes(v_in, in->n, a.v_in);

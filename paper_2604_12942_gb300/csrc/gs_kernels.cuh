@@ -186,10 +186,10 @@ constexpr int kMapMaxPlanes = 11 + 3 * 16;
 struct MapUpdateArgs {
     int64_t n, n_new, n_out, n_keep;
     int n_planes;
+    uint32_t n_chunks;           // chunks of the n rows (launch_compact sets it)
     const uint8_t* keep;         // [n]
     const uint8_t* accept;       // [n_new] or null (all accepted)
-    const uint32_t* pos_keep;    // exclusive scan of keep
-    const uint32_t* pos_new;     // exclusive scan of accept (null: identity)
+    const uint32_t* chunk_pos;   // place of each chunk's first row: the map's, then the new rows' (from 0)
     const float* in[kMapMaxPlanes];
     const float* m_in[kMapMaxPlanes];
     const float* v_in[kMapMaxPlanes];
@@ -206,8 +206,8 @@ cudaError_t launch_prune_plan(const float* logits, int64_t n, float thr, double 
 cudaError_t launch_dedup_plan(const float* map_means, int64_t n, const float* new_means, int64_t nq, float radius,
                               uint8_t* accept, void* scratch, unsigned long long* accepted_host, cudaStream_t st);
 cudaError_t launch_map_scan(const uint8_t* keep, int64_t n, const uint8_t* accept, int64_t n_new, void* scratch,
-                            uint32_t** pos_keep, uint32_t** pos_new, uint32_t* totals_host, cudaStream_t st);
-cudaError_t launch_compact(const MapUpdateArgs& a, cudaStream_t st);
+                            const uint32_t** chunk_pos, uint32_t* totals_host, cudaStream_t st);
+cudaError_t launch_compact(MapUpdateArgs& a, cudaStream_t st);
 // exclusive scan of n uint32 (bsum: ceil(n / 1024) + 1 words of scratch; total may be null)
 cudaError_t exclusive_scan_u32(const uint32_t* x, int64_t n, uint32_t* out, uint32_t* bsum, uint32_t* total,
                                cudaStream_t st);
