@@ -859,7 +859,7 @@ def main():
         table[k]["traffic"] = stage_traffic(k, args.tile, args.chunk, args.n)
     cp = compute_peaks(pk, r["sms"])
     roof = dict(table[dom])
-    roof.update({"kernel": {"composite_bwd": "render_bwd_warp_kernel" if args.tile == 16 else "render_bwd_kernel",
+    roof.update({"kernel": {"composite_bwd": "render_bwd_warp_kernel",
                             "render_fwd": "render_fwd_kernel",
                             "project_bwd_adam": "project_bwd_{entry,sh,geo}_kernel (fused Adam)", "project": "project_kernel",
                             "bin_sort": "scan/emit/radix/ranges kernels"}[dom],

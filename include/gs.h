@@ -96,7 +96,7 @@ typedef struct {
     float lambda_rgb;   /* default 1 */
     float lambda_depth; /* default 0.1 */
     int32_t tile;       /* default 16 */
-    int32_t chunk;      /* default 64; with 16-pixel tiles every value runs chunks of 256 */
+    int32_t chunk;      /* default 64; forward of 8-pixel tiles; 16-pixel tiles run 256 */
     int32_t count_fragments; /* 1: the compositing kernels fill the frag_* and visits_* counters
                                 of gs_counters (a few percent slower); 0 (default): those
                                 counters stay 0 */

@@ -509,269 +509,21 @@ __global__ void __launch_bounds__(TileMap<TILE, kFwdPPT>::NT, kFwdThreadsPerSM /
 //   r0 = (sum h h_x, sum h h_y, sum h dx^2, sum h dx dy)
 //   r1 = (sum h dy^2, sum dL/dalpha G, sum g_D w, 0), r2 = (sum g_C w, 0)
 // (h_x, h_y from frag_exponent) and the projection backward applies the constant factors.
-// A lane first sums its two pixels; the warp's 10 sums are then reduced (warp_reduce10) and
-// written by 10 lanes with one atomic each -- or, when at most kBwdDirectLanes lanes
-// contribute, added by those lanes directly with vector atomics.
+// A lane first sums its two pixels; the warp's sums are then reduced (bwd_reduce) and written by
+// 10 lanes with one atomic each -- or, when at most kBwdDirectLanes lanes contribute, added by
+// those lanes directly with vector atomics.
+//
+// One independent warp per (tile, 8 x 8 region).  The warp walks the tile's
+// list back to front 32 positions at a time: each lane tests the stored region mask of one
+// position, the hits are compacted in order (a ballot) and only their records are copied
+// (cp.async) into the warp's own double buffer while the previous window's records are
+// composited.  No block barrier: every warp proceeds at its own pace.
 // ----------------------------------------------------------------------------------------
-// Warp sums of 10 per-lane values by transpose reductions: values 0..7 halve their count at
-// each of the lane-xor 16, 8, 4 exchanges and finish with two butterflies (lane l ends with
-// the total of value (l >> 2) & 7); values 8..9 take one exchange and four butterflies (lane
-// l ends with value 8 + (l >> 4)).  44 shuffle / select / add instructions instead of 62 for
-// a 16-padded transpose.
-__device__ __forceinline__ void warp_reduce10(float (&v)[10], float& out8, float& out2) {
-    const int lane = threadIdx.x & 31;
-    {
-        const bool hi = lane & 16;
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const float mine = hi ? v[4 + k] : v[k];
-            const float other = hi ? v[k] : v[4 + k];
-            v[k] = mine + __shfl_xor_sync(0xffffffffu, other, 16);
-        }
-    }
-    {
-        const bool hi = lane & 8;
-#pragma unroll
-        for (int k = 0; k < 2; k++) {
-            const float mine = hi ? v[2 + k] : v[k];
-            const float other = hi ? v[k] : v[2 + k];
-            v[k] = mine + __shfl_xor_sync(0xffffffffu, other, 8);
-        }
-    }
-    {
-        const bool hi = lane & 4;
-        const float mine = hi ? v[1] : v[0];
-        const float other = hi ? v[0] : v[1];
-        v[0] = mine + __shfl_xor_sync(0xffffffffu, other, 4);
-    }
-    float a = v[0];
-    a += __shfl_xor_sync(0xffffffffu, a, 2);
-    a += __shfl_xor_sync(0xffffffffu, a, 1);
-    out8 = a;
-    const bool hi = lane & 16;
-    const float mine = hi ? v[9] : v[8];
-    const float other = hi ? v[8] : v[9];
-    float b = mine + __shfl_xor_sync(0xffffffffu, other, 16);
-    b += __shfl_xor_sync(0xffffffffu, b, 8);
-    b += __shfl_xor_sync(0xffffffffu, b, 4);
-    b += __shfl_xor_sync(0xffffffffu, b, 2);
-    b += __shfl_xor_sync(0xffffffffu, b, 1);
-    out2 = b;
-}
-
-template <int TILE, int CHUNK, bool COUNT>
-__global__ void __launch_bounds__(TileMap<TILE, kBwdPPT>::NT) render_bwd_kernel(BwdArgs a) {
-    pdl_begin();
-    constexpr int kPPT = kBwdPPT;
-    using TM = TileMap<TILE, kPPT>;
-    constexpr int NT = TM::NT;
-    // two chunk buffers: while the warps walk one, cp.async fills the other
-    __shared__ float4 s_rec[2][CHUNK][3];   // raw projected records (u, v, z, o), (a, b, c, rx), (r, g, b, ry)
-    __shared__ uint32_t s_id[2][CHUNK];
-    __shared__ uint32_t s_mask[2][CHUNK];
-    __shared__ uint16_t s_list[NT / 32][CHUNK];   // per warp: the chunk's records that reach its region
-    __shared__ uint32_t s_max;
-    const uint32_t status = a.counters->status;
-    const int gt = a.order ? (int)a.order[blockIdx.x] : (int)blockIdx.x;
-    if (status != 0) return;
-    const uint2 rg = a.ranges[gt];
-    const int v = view_of_tile(a.views, a.n_views, gt);
-    const View& V = a.views[v];
-    const int lt = gt - V.tile_off;
-    const int tx = lt % V.tiles_x, ty = lt / V.tiles_x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int rx0 = tx * TILE + (w % TM::WX) * 8, ry0 = ty * TILE + (w / TM::WX) * TM::RH;
-    const float amin = a.op.alpha_min, amax = a.op.alpha_max;
-    uint32_t n_eval = 0, n_add = 0, n_visit = 0;
-    float px[kPPT], py[kPPT], T[kPPT], S[kPPT], gc0[kPPT], gc1[kPPT], gc2[kPPT], gd[kPPT];
-    uint32_t last[kPPT];
-    uint32_t mylast = 0;
-#pragma unroll
-    for (int q = 0; q < kPPT; q++) {
-        const int xi = rx0 + (lane & 7), yi = ry0 + (lane >> 3) + 4 * q;
-        px[q] = (float)xi + 0.5f;
-        py[q] = (float)yi + 0.5f;
-        T[q] = 0.f; gc0[q] = gc1[q] = gc2[q] = gd[q] = 0.f;
-        last[q] = 0;
-        if (xi < V.W && yi < V.H) {
-            const int64_t P = (int64_t)V.W * V.H;
-            const int64_t p = (int64_t)yi * V.W + xi;
-            const int64_t g = V.pix_off + p;
-            T[q] = a.T_final[g];
-            last[q] = a.n_contrib[g];
-            const float* d = a.dl_drgb + 3 * V.pix_off;
-            gc0[q] = d[p];
-            gc1[q] = d[P + p];
-            gc2[q] = d[2 * P + p];
-            gd[q] = a.dl_ddepth ? a.dl_ddepth[g] : 0.f;
-            if (gc0[q] == 0.f && gc1[q] == 0.f && gc2[q] == 0.f && gd[q] == 0.f) last[q] = 0;
-        }
-        S[q] = (gc0[q] * a.op.bg0 + gc1[q] * a.op.bg1 + gc2[q] * a.op.bg2) * T[q];
-        mylast = max(mylast, last[q]);
-    }
-    const uint32_t wtop = __reduce_max_sync(0xffffffffu, mylast);
-    int top_all;
-    if constexpr (NT == 32) {
-        top_all = (int)wtop;   // one warp: no block reduction
-    } else {
-        if (threadIdx.x == 0) s_max = 0;
-        __syncthreads();
-        if (lane == 0 && wtop) atomicMax(&s_max, wtop);
-        __syncthreads();
-        top_all = (int)s_max;
-    }
-    // Chunk c covers list positions [max(0, top_all - (c + 1) CHUNK), top_all - c CHUNK).
-    // Pipeline: the ids and masks of chunk c + 2 are loaded into registers and the records of
-    // chunk c + 1 are copied asynchronously while chunk c is composited.
-    const int nchunks = (top_all + CHUNK - 1) / CHUNK;
-    constexpr int R = (CHUNK + NT - 1) / NT;   // staged records per thread
-    uint32_t pid[R];
-    uint32_t pmsk[R];
-    auto fetch_ids = [&](int c) {
-        const int top = top_all - c * CHUNK, lo = max(0, top - CHUNK);
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            const int k = (int)threadIdx.x + r * NT;
-            if (c < nchunks && k < top - lo) {
-                pid[r] = a.vals[rg.x + lo + k];
-                pmsk[r] = a.pair_mask[rg.x + lo + k];
-            }
-        }
-    };
-    auto stage = [&](int c, int b) {
-        const int top = top_all - c * CHUNK, lo = max(0, top - CHUNK);
-#pragma unroll
-        for (int r = 0; r < R; r++) {
-            const int k = (int)threadIdx.x + r * NT;
-            if (c < nchunks && k < top - lo) {
-                s_id[b][k] = pid[r];
-                s_mask[b][k] = bwd_mask_from_fwd<TILE>(pmsk[r]);
-                const float4* src = a.proj + 3 * (size_t)pid[r];
-#pragma unroll
-                for (int h = 0; h < 3; h++) cp_async16(&s_rec[b][k][h], src + h);
-            }
-        }
-        cp_async_commit();
-    };
-    fetch_ids(0);
-    stage(0, 0);
-    fetch_ids(1);
-    for (int c = 0; c < nchunks; c++) {
-        const int b = c & 1;
-        const int top = top_all - c * CHUNK, lo = max(0, top - CHUNK);
-        stage(c + 1, b ^ 1);
-        fetch_ids(c + 2);
-        cp_async_wait_prior();   // chunk c has landed (chunk c + 1 may still be in flight)
-        __syncthreads();
-        uint32_t ltm;
-        asm("mov.u32 %0, %%lanemask_lt;" : "=r"(ltm));
-        // this warp's records of the chunk, back to front: positions below its pixels' last
-        // added fragment whose alpha >= alpha_min region reaches the warp's pixels
-        const int kstart = min(top, (int)wtop) - 1 - lo;
-        int cnt = 0;
-        for (int k0 = kstart; k0 >= 0; k0 -= 32) {
-            const int kk = k0 - lane;
-            const bool hit = kk >= 0 && ((s_mask[b][kk] >> w) & 1u);
-            const uint32_t bal = __ballot_sync(0xffffffffu, hit);
-            if (hit) s_list[w][cnt + __popc(bal & ltm)] = (uint16_t)kk;
-            cnt += __popc(bal);
-        }
-        __syncwarp();
-        if constexpr (COUNT) n_visit += cnt;
-        for (int t = 0; t < cnt; t++) {
-            const int k = s_list[w][t];
-            const int j = lo + k;
-            const float4 r0 = s_rec[b][k][0], r1 = s_rec[b][k][1];
-            const float2 bx = make_float2(r0.x, r0.y);
-            const float4 co = make_float4(r1.x, r1.y, r1.z, r0.w);
-            float val[10];
-#pragma unroll
-            for (int q = 0; q < 10; q++) val[q] = 0.f;
-            bool contrib = false;
-            const float4 r2 = s_rec[b][k][2];
-            const float4 cz = make_float4(r2.x, r2.y, r2.z, r0.z);
-            // Branch-free per pixel: every lane computes the fragment and commits it with
-            // selects (adding exact zeros where it does not contribute), so the warp runs one
-            // straight path instead of re-converging around per-pixel branches.
-#pragma unroll
-            for (int q = 0; q < kPPT; q++) {
-                const bool live = (uint32_t)j < last[q];
-                const float dx = px[q] - bx.x, dy = py[q] - bx.y;
-                const FragE fe = frag_exponent(dx, dy, co.x, co.y, co.z);
-                const float G = ex2_approx(fe.e);
-                const float a0 = co.w * G;
-                const float alpha = fminf(amax, a0);
-                const bool c = live && !(alpha < amin);
-                if constexpr (COUNT) {
-                    n_eval += live;
-                    n_add += c;
-                }
-                contrib |= c;
-                const float rom = rcp_approx(1.f - alpha);
-                const float Tn = T[q] * rom;
-                const float wgt = alpha * Tn;
-                const float gcz = gc0[q] * cz.x + gc1[q] * cz.y + gc2[q] * cz.z + gd[q] * cz.w;
-                const float dLda = Tn * gcz - S[q] * rom;
-                S[q] = c ? fmaf(gcz, wgt, S[q]) : S[q];
-                T[q] = c ? Tn : T[q];
-                const float wc = c ? wgt : 0.f;
-                val[7] = fmaf(gc0[q], wc, val[7]);
-                val[8] = fmaf(gc1[q], wc, val[8]);
-                val[9] = fmaf(gc2[q], wc, val[9]);
-                val[6] = fmaf(gd[q], wc, val[6]);
-                const float gl = (c && a0 < amax) ? dLda : 0.f;   // the 0.99 clamp stops the gradient
-                const float h = gl * a0;
-                const float hdx = h * dx;
-                val[0] = fmaf(h, fe.hx, val[0]);
-                val[1] = fmaf(h, fe.hy, val[1]);
-                val[2] = fmaf(hdx, dx, val[2]);
-                val[3] = fmaf(hdx, dy, val[3]);
-                val[4] = fmaf(h * dy, dy, val[4]);
-                val[5] = fmaf(gl, G, val[5]);
-            }
-            const uint32_t cmask = __ballot_sync(0xffffffffu, contrib);
-            if (cmask) {
-                float4* rec4 = a.grad2d + 3 * (size_t)s_id[b][k];
-                if (__popc(cmask) <= kBwdDirectLanes) {
-                    // few contributing lanes: each adds its own sums with three vector atomics
-                    // (slots 7 and 11 of the record are padding and receive zeros)
-                    if (contrib) {
-                        atomicAdd(rec4, make_float4(val[0], val[1], val[2], val[3]));
-                        atomicAdd(rec4 + 1, make_float4(val[4], val[5], val[6], 0.f));
-                        atomicAdd(rec4 + 2, make_float4(val[7], val[8], val[9], 0.f));
-                    }
-                } else {
-                    float t8, t2;
-                    warp_reduce10(val, t8, t2);
-                    float* rec = reinterpret_cast<float*>(rec4);
-                    // value index -> record slot: 0..6 -> 0..6, 7..9 -> 8..10
-                    if ((lane & 3) == 0) {
-                        const int idx = lane >> 2;
-                        atomicAdd(rec + (idx < 7 ? idx : idx + 1), t8);
-                    }
-                    if ((lane & 15) == 0) atomicAdd(rec + 9 + (lane >> 4), t2);
-                }
-            }
-        }
-        __syncthreads();   // buffer b is refilled with chunk c + 2 in the next iteration
-    }
-    cp_async_wait_all();
-    if constexpr (COUNT) {
-        warp_count_add(&a.counters->frag_bwd_eval, n_eval);
-        warp_count_add(&a.counters->frag_bwd_add, n_add);
-        if (lane == 0 && n_visit) atomicAdd(&a.counters->visits_bwd, n_visit);
-    }
-}
-
-// ----------------------------------------------------------------------------------------
-// Backward compositing, one independent warp per (16 x 16 tile, 8 x 8 region).  The warp walks
-// the tile's list back to front 32 positions at a time: each lane tests the stored region mask
-// of one position, the hits are compacted in order (a ballot) and only their records are
-// copied (cp.async) into the warp's own double buffer while the previous window's records are
-// composited.  No block barrier: every warp proceeds at its own pace.  The per-record
-// arithmetic is that of render_bwd_kernel.
-// ----------------------------------------------------------------------------------------
-constexpr int kWin = 32;   // list positions per window
+constexpr int kWin = 32;            // list positions per window
+// Items a resident warp from which two visits reduce together (render_bwd_region's JOINT): at 19.7
+// (95,680 items) it is better on two scenes (4055 and 4089, 3521 and 3555 us a step), at 9.5 better on
+// one and worse on the other (1439 and 1448, 1864 and 1820), at 2 worse.
+constexpr int kBwdJointWaves = 16;
 
 // A warp's shared memory: its two windows of staged records, their ids and list positions.
 struct BwdWarpSmem {
@@ -780,17 +532,90 @@ struct BwdWarpSmem {
     int pos[2][kWin];
 };
 
-// The backward of work item `item` = 4 t + w: region w of the t-th tile of the work order, by
-// one warp with its own shared memory S.
-template <bool COUNT>
+// Keeps `own`, sends `other` to the lane at distance `x`, and adds what that lane sends.
+__device__ __forceinline__ float fold(float own, float other, int x) {
+    return own + __shfl_xor_sync(0xffffffffu, other, x);
+}
+
+// What a visit adds to its Gaussian's record, from lane sums over the lane's two pixels, which lie
+// in one column of the region (one dx):
+//   A0 = sum h, A1 = sum h dy, A2 = sum h dy^2, D = sum g_D w, c0..c2 = sum g_C w.
+struct BwdSums {
+    float A0, A1, A2, D, c0, c1, c2;
+    float dx, a, b, c, inv_o;   // the column's dx; the record's conic and 1 / o
+};
+
+// Warp totals of N visits, stage by stage over all of them so that their shuffles overlap.  The
+// sums over rows come first (lane distances 16 and 8), on seven values a visit instead of ten; dx
+// and the conic (a, b, c) then turn the three geometry sums of a column into its six terms, and
+// the lanes 8 r + x of row r hold three (r = 0, 1) or two terms for the sums over columns:
+//   r = 0: h h_x, h h_y, h dx dy   r = 1: dL/dalpha G, h dx^2, h dy^2   r = 2: D, c0   r = 3: c1, c2
+// z[k] is the total for record slot bwd_slot(lane) of visit k.
+template <int N>
+__device__ __forceinline__ void bwd_reduce(int lane, const BwdSums (&s)[N], float (&z)[N]) {
+    const bool hi = lane & 16, odd = lane & 8, x4 = lane & 4, x2 = lane & 2;
+    const bool r0 = !hi && !odd, r1 = !hi && odd;
+    float k0[N], k1[N], k2[N], k3[N], p[N], q[N], v0[N], v1[N], v2[N];
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        k0[k] = fold(hi ? s[k].D : s[k].A0, hi ? s[k].A0 : s[k].D, 16);
+        k1[k] = fold(hi ? s[k].c1 : s[k].A1, hi ? s[k].A1 : s[k].c1, 16);
+        k2[k] = fold(hi ? s[k].c2 : s[k].A2, hi ? s[k].A2 : s[k].c2, 16);
+        k3[k] = fold(s[k].c0, s[k].c0, 16);
+    }
+    // p: A0, A0, D, c1 and q: A1, A2, c0, c2 of rows 0 .. 3
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        p[k] = fold(hi && odd ? k1[k] : k0[k], hi && !odd ? k1[k] : k0[k], 8);
+        const float e = hi ? k3[k] : k1[k];
+        q[k] = fold(odd ? k2[k] : e, odd ? e : k2[k], 8);
+    }
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        // (dx times a, b and dx do not wait for the sums)
+        v0[k] = r0 ? fmaf(s[k].a * s[k].dx, p[k], s[k].b * q[k]) : (r1 ? p[k] * s[k].inv_o : p[k]);
+        v1[k] = r0 ? fmaf(s[k].b * s[k].dx, p[k], s[k].c * q[k]) : (r1 ? s[k].dx * s[k].dx * p[k] : q[k]);
+        v2[k] = r0 ? s[k].dx * q[k] : q[k];
+    }
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+        v0[k] = fold(x4 ? v2[k] : v0[k], x4 ? v0[k] : v2[k], 4);
+        v1[k] = fold(v1[k], v1[k], 4);
+    }
+#pragma unroll
+    for (int k = 0; k < N; k++) z[k] = fold(x2 ? v1[k] : v0[k], x2 ? v0[k] : v1[k], 2);
+#pragma unroll
+    for (int k = 0; k < N; k++) z[k] = fold(z[k], z[k], 1);
+}
+
+// The record slot whose total bwd_reduce leaves in this lane, or -1.
+__device__ __forceinline__ int bwd_slot(int lane) {
+    const int r = lane >> 3, x = lane & 7;
+    if (x == 0) return r == 0 ? 0 : (r == 1 ? 5 : (r == 2 ? 6 : 9));
+    if (x == 2) return r == 0 ? 1 : (r == 1 ? 2 : (r == 2 ? 8 : 10));
+    if (x == 4) return r == 0 ? 3 : (r == 1 ? 4 : -1);
+    return -1;
+}
+
+// The backward of work item `item` = R t + w: region w of the R = (TILE / 8)^2 regions of the t-th
+// tile of the work order, by one warp with its own shared memory W.
+//
+// What bounds it: the issue slots while the chip is full (73% busy, 61 registers, 32 one-warp blocks
+// an SM), then the longest lists, each walked by one warp.  Sums by columns and alpha = 0 in place
+// of three selects a pixel save about 17 of 175 instructions a visit.  JOINT reduces two visits at
+// once, so that their shuffles overlap: better while many warps share an SM, worse where a lone
+// warp's list sets the time.  Whole steps, ten values reduced / by columns / JOINT: 2M Gaussians, 8
+// views 4100, 4089, 4055 us; 200k, 8 small views 868, 860, 894; 1M, 2 views 1348, 1327, 1344.  8 x 8
+// tiles, 1M, 2 views, as blocks with shared chunks / this: 1176, 1130.
+template <int TILE, bool JOINT, bool COUNT>
 __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, BwdWarpSmem& W) {
-    constexpr int TILE = 16, kPPT = kBwdPPT;
+    constexpr int kPPT = kBwdPPT, WX = TILE / 8, R = WX * WX;
     auto& s_rec = W.rec;
     auto& s_id = W.id;
     auto& s_pos = W.pos;
     const uint32_t status = a.counters->status;
-    const int gt = a.order ? (int)a.order[item >> 2] : (item >> 2);
-    const int w = item & 3;   // region: column w % 2, row w / 2 (the forward's mask order)
+    const int gt = a.order ? (int)a.order[item / R] : item / R;
+    const int w = item % R;   // region: column w % WX, row w / WX (the forward's mask order)
     if (status != 0) return;
     const uint2 rg = a.ranges[gt];
     const int v = view_of_tile(a.views, a.n_views, gt);
@@ -798,7 +623,7 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
     const int lt = gt - V.tile_off;
     const int tx = lt % V.tiles_x, ty = lt / V.tiles_x;
     const int lane = threadIdx.x & 31;
-    const int rx0 = tx * TILE + (w & 1) * 8, ry0 = ty * TILE + (w >> 1) * 8;
+    const int rx0 = tx * TILE + (w % WX) * 8, ry0 = ty * TILE + (w / WX) * 8;
     const float amin = a.op.alpha_min, amax = a.op.alpha_max;
     uint32_t n_eval = 0, n_add = 0, n_visit = 0;
     float px[kPPT], py[kPPT], T[kPPT], S[kPPT], gc0[kPPT], gc1[kPPT], gc2[kPPT], gd[kPPT];
@@ -828,11 +653,9 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
         mylast = max(mylast, last[q]);
     }
     const int wtop = (int)__reduce_max_sync(0xffffffffu, mylast);
-    // the lane's two pixels (rows y and y + 4 of the region) as packed pairs
-    const float2 px2 = make_float2(px[0], px[1]), py2 = make_float2(py[0], py[1]);
-    const float2 g0 = make_float2(gc0[0], gc0[1]), g1 = make_float2(gc1[0], gc1[1]);
-    const float2 g2 = make_float2(gc2[0], gc2[1]), gd2 = make_float2(gd[0], gd[1]);
-    float2 T2 = make_float2(T[0], T[1]), S2 = make_float2(S[0], S[1]);
+    // the rows y and y + 4 of the lane's two pixels as a packed pair (their column is one)
+    const float2 py2 = make_float2(py[0], py[1]);
+    const int slot = bwd_slot(lane);
     uint32_t ltm;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(ltm));
     // window starting (from the back) at position k0: this warp's hits, copied into buffer b
@@ -872,108 +695,111 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
         if (lane < cnt) s_rec[b][lane][2].w = s_rec[b][lane][0].z;
         __syncwarp();
         if constexpr (COUNT) n_visit += cnt;
-        // the alphas of the lane's two pixels of record t, as one packed pair: a record that no
-        // pixel of the warp adds (all below alpha_min or past their pixels' last fragment)
+        // the alphas of the lane's two pixels of record t (the exponent as a packed pair): a record
+        // that no pixel of the warp adds (all below alpha_min or past their pixels' last fragment)
         // changes nothing and is skipped whole
         struct Alphas {
-            float2 dx, dy, hx, hy, G, a0, al;
+            float dx;
+            float2 dy, a0;
             bool c0, c1;
         };
         auto alphas = [&](int t, Alphas& P) {
             const uint32_t j = (uint32_t)s_pos[b][t];
             const float4 r0 = s_rec[b][t][0], r1 = s_rec[b][t][1];
-            P.dx = __fadd2_rn(px2, dup2(-r0.x));
+            P.dx = px[0] - r0.x;
             P.dy = __fadd2_rn(py2, dup2(-r0.y));
-            const FragE2 fe = frag_exponent2(P.dx, P.dy, dup2(r1.x), dup2(r1.y), dup2(r1.z));
-            P.hx = fe.hx;
-            P.hy = fe.hy;
-            P.G = make_float2(ex2_approx(fe.e.x), ex2_approx(fe.e.y));
-            P.a0 = __fmul2_rn(dup2(r0.w), P.G);
-            P.al = make_float2(fminf(amax, P.a0.x), fminf(amax, P.a0.y));
-            P.c0 = j < last[0] && !(P.al.x < amin);
-            P.c1 = j < last[1] && !(P.al.y < amin);
+            const FragE2 fe = frag_exponent2(dup2(P.dx), P.dy, dup2(r1.x), dup2(r1.y), dup2(r1.z));
+            P.a0 = __fmul2_rn(dup2(r0.w), make_float2(ex2_approx(fe.e.x), ex2_approx(fe.e.y)));
+            P.c0 = j < last[0] && !(fminf(amax, P.a0.x) < amin);
+            P.c1 = j < last[1] && !(fminf(amax, P.a0.y) < amin);
             if constexpr (COUNT) {
                 n_eval += (j < last[0]) + (j < last[1]);
                 n_add += P.c0 + P.c1;
             }
         };
         // back to front, each pixel of the lane in turn: T in front of the fragment from the one
-        // behind it, weight, the colour / depth adjoint and dL/dalpha; pixels that do not add it
-        // keep T and S (scalar arithmetic: packing these pairs measured slower)
+        // behind it, weight, the colour / depth adjoint and dL/dalpha; a pixel that does not add
+        // the fragment takes alpha = 0, which leaves T and S as they are (rcp(1) = 1) and adds
+        // exact zeros
         auto adjoint = [&](int t, const Alphas& P) {
-            const bool contrib = P.c0 || P.c1;
-            const float dxs[2] = {P.dx.x, P.dx.y}, dys[2] = {P.dy.x, P.dy.y}, hxs[2] = {P.hx.x, P.hx.y},
-                        hys[2] = {P.hy.x, P.hy.y};
-            const float Gs[2] = {P.G.x, P.G.y}, a0s[2] = {P.a0.x, P.a0.y}, als[2] = {P.al.x, P.al.y};
-            const float4 r2 = s_rec[b][t][2];
-            const float4 cz = r2;   // colour and depth
-            float val[10];
-#pragma unroll
-            for (int q = 0; q < 10; q++) val[q] = 0.f;
-            const float Ts[2] = {T2.x, T2.y}, Ss[2] = {S2.x, S2.y};
-            const float g0s[2] = {g0.x, g0.y}, g1s[2] = {g1.x, g1.y}, g2s[2] = {g2.x, g2.y}, gds[2] = {gd2.x, gd2.y};
-            float Tn_[2], Sn_[2];
+            const float4 cz = s_rec[b][t][2];   // colour and depth
+            const float a0s[2] = {P.a0.x, P.a0.y}, dys[2] = {P.dy.x, P.dy.y};
             const bool cq[2] = {P.c0, P.c1};
+            BwdSums s = {};
 #pragma unroll
-            for (int q = 0; q < 2; q++) {
-                const float dxv = dxs[q], dyv = dys[q], Gv = Gs[q], a0v = a0s[q], alpha = als[q];
-                const bool c = cq[q];
+            for (int q = 0; q < kPPT; q++) {
+                const float a0 = a0s[q];
+                const float alpha = cq[q] ? fminf(amax, a0) : 0.f;
                 const float rom = rcp_approx(1.f - alpha);
-                const float Tn = Ts[q] * rom;
+                const float Tn = T[q] * rom;
                 const float wgt = alpha * Tn;
-                const float gcz = g0s[q] * cz.x + g1s[q] * cz.y + g2s[q] * cz.z + gds[q] * cz.w;
-                const float dLda = Tn * gcz - Ss[q] * rom;
-                Sn_[q] = c ? fmaf(gcz, wgt, Ss[q]) : Ss[q];
-                Tn_[q] = c ? Tn : Ts[q];
-                const float wc = c ? wgt : 0.f;
-                val[7] = fmaf(g0s[q], wc, val[7]);
-                val[8] = fmaf(g1s[q], wc, val[8]);
-                val[9] = fmaf(g2s[q], wc, val[9]);
-                val[6] = fmaf(gds[q], wc, val[6]);
-                const float gl = (c && a0v < amax) ? dLda : 0.f;   // the 0.99 clamp stops the gradient
-                const float h = gl * a0v;
-                const float hdx = h * dxv;
-                val[0] = fmaf(h, hxs[q], val[0]);
-                val[1] = fmaf(h, hys[q], val[1]);
-                val[2] = fmaf(hdx, dxv, val[2]);
-                val[3] = fmaf(hdx, dyv, val[3]);
-                val[4] = fmaf(h * dyv, dyv, val[4]);
-                val[5] = fmaf(gl, Gv, val[5]);
+                const float gcz = gc0[q] * cz.x + gc1[q] * cz.y + gc2[q] * cz.z + gd[q] * cz.w;
+                const float dLda = Tn * gcz - S[q] * rom;
+                S[q] = fmaf(gcz, wgt, S[q]);
+                T[q] = Tn;
+                s.c0 = fmaf(gc0[q], wgt, s.c0);
+                s.c1 = fmaf(gc1[q], wgt, s.c1);
+                s.c2 = fmaf(gc2[q], wgt, s.c2);
+                s.D = fmaf(gd[q], wgt, s.D);
+                const float h = cq[q] && a0 < amax ? dLda * a0 : 0.f;   // the 0.99 clamp stops the gradient
+                const float hy = h * dys[q];
+                s.A0 += h;
+                s.A1 += hy;
+                s.A2 = fmaf(hy, dys[q], s.A2);
             }
-            S2 = make_float2(Sn_[0], Sn_[1]);
-            T2 = make_float2(Tn_[0], Tn_[1]);
-            const uint32_t cmask = __ballot_sync(0xffffffffu, contrib);
+            const float4 r1 = s_rec[b][t][1];
+            s.dx = P.dx;
+            s.a = r1.x;
+            s.b = r1.y;
+            s.c = r1.z;
+            s.inv_o = rcp_approx(s_rec[b][t][0].w);   // sum dL/dalpha G = sum h / o
+            return s;
+        };
+        // one record added by the lanes of cm
+        auto visit = [&](int t, const Alphas& P, uint32_t cm) {
+            const BwdSums s[1] = {adjoint(t, P)};
             float4* rec4 = a.grad2d + 3 * (size_t)s_id[b][t];
-            if (__popc(cmask) <= kBwdDirectLanes) {
-                if (contrib) {
-                    atomicAdd(rec4, make_float4(val[0], val[1], val[2], val[3]));
-                    atomicAdd(rec4 + 1, make_float4(val[4], val[5], val[6], 0.f));
-                    atomicAdd(rec4 + 2, make_float4(val[7], val[8], val[9], 0.f));
+            if (__popc(cm) <= kBwdDirectLanes) {
+                if (P.c0 || P.c1) {
+                    const float u = s[0].dx * s[0].A0;
+                    atomicAdd(rec4, make_float4(fmaf(s[0].a, u, s[0].b * s[0].A1), fmaf(s[0].b, u, s[0].c * s[0].A1),
+                                                s[0].dx * u, s[0].dx * s[0].A1));
+                    atomicAdd(rec4 + 1, make_float4(s[0].A2, s[0].A0 * s[0].inv_o, s[0].D, 0.f));
+                    atomicAdd(rec4 + 2, make_float4(s[0].c0, s[0].c1, s[0].c2, 0.f));
                 }
             } else {
-                float t8, t2;
-                warp_reduce10(val, t8, t2);
-                float* rec = reinterpret_cast<float*>(rec4);
-                if ((lane & 3) == 0) {
-                    const int idx = lane >> 2;
-                    atomicAdd(rec + (idx < 7 ? idx : idx + 1), t8);
-                }
-                if ((lane & 15) == 0) atomicAdd(rec + 9 + (lane >> 4), t2);
+                float z[1];
+                bwd_reduce(lane, s, z);
+                if (slot >= 0) atomicAdd(reinterpret_cast<float*>(rec4) + slot, z[0]);
             }
         };
-        // two records per iteration: their alphas are independent (the adjoints are not)
+        // two records per iteration: their alphas are independent (the adjoints are not), and so are
+        // their reductions
         int t = 0;
         for (; t + 1 < cnt; t += 2) {
             Alphas A, B;
             alphas(t, A);
             alphas(t + 1, B);
-            if (__any_sync(0xffffffffu, A.c0 || A.c1)) adjoint(t, A);
-            if (__any_sync(0xffffffffu, B.c0 || B.c1)) adjoint(t + 1, B);
+            const uint32_t ca = __ballot_sync(0xffffffffu, A.c0 || A.c1);
+            const uint32_t cb = __ballot_sync(0xffffffffu, B.c0 || B.c1);
+            if (JOINT && min(__popc(ca), __popc(cb)) > kBwdDirectLanes) {
+                const BwdSums s[2] = {adjoint(t, A), adjoint(t + 1, B)};
+                float z[2];
+                bwd_reduce(lane, s, z);
+                if (slot >= 0) {
+                    atomicAdd(reinterpret_cast<float*>(a.grad2d + 3 * (size_t)s_id[b][t]) + slot, z[0]);
+                    atomicAdd(reinterpret_cast<float*>(a.grad2d + 3 * (size_t)s_id[b][t + 1]) + slot, z[1]);
+                }
+                continue;
+            }
+            if (ca) visit(t, A, ca);
+            if (cb) visit(t + 1, B, cb);
         }
         if (t < cnt) {
             Alphas A;
             alphas(t, A);
-            if (__any_sync(0xffffffffu, A.c0 || A.c1)) adjoint(t, A);
+            const uint32_t ca = __ballot_sync(0xffffffffu, A.c0 || A.c1);
+            if (ca) visit(t, A, ca);
         }
         __syncwarp();   // every lane is done with buffer b before it is refilled
         cnt = cnt_next;
@@ -987,11 +813,11 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
     }
 }
 
-template <bool COUNT>
+template <int TILE, bool JOINT, bool COUNT>
 __global__ void __launch_bounds__(32, 32) render_bwd_warp_kernel(BwdArgs a) {
     pdl_begin();
     __shared__ BwdWarpSmem S;
-    render_bwd_region<COUNT>(a, blockIdx.x, S);
+    render_bwd_region<TILE, JOINT, COUNT>(a, blockIdx.x, S);
 }
 
 template <int TILE, int CHUNK>
@@ -1015,21 +841,14 @@ static cudaError_t launch_fwd_t(const FwdArgs& a, int total_tiles, int chunk, cu
     return cudaGetLastError();
 }
 
-template <int TILE, int CHUNK>
-static void launch_bwd_c(const BwdArgs& a, int total_tiles, cudaStream_t st) {
-    constexpr int NT = TileMap<TILE, kBwdPPT>::NT;
-    if (a.op.count) launch_pdl_small(render_bwd_kernel<TILE, CHUNK, true>, total_tiles, NT, 0, st, a);
-    else launch_pdl_small(render_bwd_kernel<TILE, CHUNK, false>, total_tiles, NT, 0, st, a);
-}
-
 template <int TILE>
-static cudaError_t launch_bwd_t(const BwdArgs& a, int total_tiles, int chunk, cudaStream_t st) {
-    switch (chunk) {
-        case 32: launch_bwd_c<TILE, 32>(a, total_tiles, st); break;
-        case 64: launch_bwd_c<TILE, 64>(a, total_tiles, st); break;
-        case 128: launch_bwd_c<TILE, 128>(a, total_tiles, st); break;
-        default: launch_bwd_c<TILE, 256>(a, total_tiles, st); break;
-    }
+static cudaError_t launch_bwd_t(const BwdArgs& a, int total_tiles, cudaStream_t st) {
+    const int items = total_tiles * (TILE / 8) * (TILE / 8);
+    const bool joint = items >= kBwdJointWaves * 32 * device_sms();
+    auto kernel = a.op.count ? render_bwd_warp_kernel<TILE, false, true>
+                  : joint    ? render_bwd_warp_kernel<TILE, true, false>
+                             : render_bwd_warp_kernel<TILE, false, false>;
+    launch_pdl_small(kernel, items, 32, 0, st, a);
     return cudaGetLastError();
 }
 
@@ -1077,13 +896,8 @@ cudaError_t launch_render_bwd(const BwdArgs& a, int total_tiles, cudaStream_t st
                               float b2, const LossFinal& lf) {
     launch_pdl(clear_grad2d_kernel, device_sms() * 12, 256, 0, st, a, adam_ctr, b1, b2, lf);
     if (total_tiles <= 0) return cudaGetLastError();
-    // 16 x 16 tiles: one independent warp per 8 x 8 region (8 x 8 tiles are one warp already)
-    if (a.op.tile == 16) {
-        if (a.op.count) launch_pdl_small(render_bwd_warp_kernel<true>, 4 * total_tiles, 32, 0, st, a);
-        else launch_pdl_small(render_bwd_warp_kernel<false>, 4 * total_tiles, 32, 0, st, a);
-        return cudaGetLastError();
-    }
-    return launch_bwd_t<8>(a, total_tiles, a.op.chunk, st);
+    if (a.op.tile == 16) return launch_bwd_t<16>(a, total_tiles, st);
+    return launch_bwd_t<8>(a, total_tiles, st);
 }
 
 // ----------------------------------------------------------------------------------------
@@ -1223,7 +1037,7 @@ __global__ void __launch_bounds__(kPersistThreads, 2) step_persistent_kernel(Per
         if (lane == 0) item = atomicAdd(&P.sync->q_bwd, 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
         if (item >= 4u * (unsigned int)P.total_tiles) break;
-        render_bwd_region<false>(P.bwd, (int)item, S.u.bwd[warp]);
+        render_bwd_region<16, false, false>(P.bwd, (int)item, S.u.bwd[warp]);
     }
     if (!grid_barrier<DEG>(P, true, S)) return;
     project_bwd_entry_part(P.pb, blockIdx.x, gridDim.x, S.tw);   // phase 3
