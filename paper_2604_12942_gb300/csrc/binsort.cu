@@ -137,11 +137,13 @@ __global__ void __launch_bounds__(kEntryThreads, 4) entry_compact_kernel(BinArgs
     __shared__ uint32_t s_hist[kSortBins];
     __shared__ bool s_ok;
     static_assert(kEntryThreads == kSortBins, "a thread per digit");
-    if (a.counters->status != 0) return;
     s_hist[threadIdx.x] = 0;
     if (LOOKBACK) {
-        if (threadIdx.x == 0) s_chunk = atomicAdd(&a.tickets[0], 1u);
+        if (threadIdx.x == 0) s_chunk = lb_ticket(&a.tickets[0], a.counters);
         __syncthreads();
+        if (s_chunk == kLbStop) return;
+    } else if (a.counters->status != 0) {   // (this form does not set it)
+        return;
     }
     const int64_t chunk = LOOKBACK ? s_chunk : blockIdx.x, word = chunk * WPB + threadIdx.x;
     const uint32_t b = (int)threadIdx.x < WPB && word < n_words ? a.vis_bits[word] : 0u;
@@ -266,15 +268,14 @@ __global__ void __launch_bounds__(kPairScanThreads) pair_offsets_kernel(BinArgs 
     __shared__ uint32_t s[33], s_chunk;
     __shared__ unsigned long long s_base;
     __shared__ bool s_ok;
-    if (a.counters->status != 0) return;
     const int64_t E = (int64_t)a.counters->n_entries, VN = (int64_t)a.n_views * a.n;
     const int64_t n_chunks = (E + kPairScanChunk - 1) / kPairScanChunk;
     const uint64_t emit_chunks = ((uint64_t)a.max_pairs + kEmitChunk - 1) / kEmitChunk;
     for (;;) {
-        if (threadIdx.x == 0) s_chunk = atomicAdd(&a.tickets[1], 1u);
+        if (threadIdx.x == 0) s_chunk = lb_ticket(&a.tickets[1], a.counters);
         __syncthreads();
         const int64_t ch = s_chunk;
-        if (ch >= n_chunks) return;
+        if (ch >= n_chunks) return;   // (kLbStop is past every chunk)
         // thread t takes entries 4 t .. 4 t + 3 of the chunk
         const int64_t e0 = ch * kPairScanChunk + (int64_t)threadIdx.x * kPairScanItems;
         uint32_t c[kPairScanItems], t[kPairScanItems], sum = 0;

@@ -503,6 +503,16 @@ __device__ __forceinline__ uint32_t lb_state(uint32_t w, uint32_t tag) {
 }
 __device__ __forceinline__ uint32_t lb_value(uint32_t w) { return w & 0xFFFFFFu; }
 
+// The next chunk's ticket, or kLbStop once the status is set.  One thread of a block calls it and
+// hands the result to the others: a kernel that can itself set the status (a time-out, the pair
+// capacity) while blocks of it start must not let every thread read it, for threads of one block
+// could then disagree and part of it would go on without the rest.
+constexpr uint32_t kLbStop = 0xFFFFFFFFu;
+__device__ __forceinline__ uint32_t lb_ticket(uint32_t* ticket, const Counters* c) {
+    const uint32_t t = atomicAdd(ticket, 1u), s = *(const volatile uint32_t*)&c->status;
+    return s != 0 ? kLbStop : t;
+}
+
 // One warp: publishes the chunk's total, sums the totals of the chunks before it (128 at a time:
 // the chunks of the first wave publish together and none has a prefix yet) and publishes the
 // inclusive prefix.  Returns the exclusive prefix; ok is cleared if a wait gave up (the status
