@@ -122,11 +122,13 @@ __device__ __forceinline__ void entry_geometry_bwd(const float (&mu)[3], const C
 constexpr int kEntryThreads = 256;
 
 // The entry part over the block's share of the entries (block `blk` of `nblk`, kEntryThreads
-// threads); s_tw: the block's GS_MAX_VIEWS * 6 floats of shared memory.
+// threads); s_tw: the block's GS_MAX_VIEWS * 6 floats of shared memory.  CHECK, here and below:
+// leave if the status is set (off where the caller has checked it for the whole block).
+template <bool CHECK = true>
 __device__ __forceinline__ void project_bwd_entry_part(const ProjectBwdArgs& a, int64_t blk, int64_t nblk,
                                                        float* s_tw) {
     // a failed earlier stage (capacity, non-finite input) leaves the screen-space sums undefined
-    if (a.counters->status != 0) return;
+    if (CHECK && a.counters->status != 0) return;
     for (int t = threadIdx.x; t < a.n_views * 6; t += kEntryThreads) s_tw[t] = 0.f;
     __syncthreads();
     const int64_t E = (int64_t)a.counters->n_entries;
@@ -204,10 +206,10 @@ constexpr int sh_mv_floats() { return 2 * 2 * (DEG + 1) * (DEG + 1) * T; }
 // s_cam: GS_MAX_VIEWS * 12 floats of shared memory, each view's camera centre and rotation
 // (cw, R) copied there when the block starts, so the walk over a row's views reads them without
 // a trip to L2 (the streamed planes keep little of the view table in L1).
-template <int DEG, bool FUSED_ADAM, int T>
+template <int DEG, bool FUSED_ADAM, int T, bool CHECK = true>
 __device__ __forceinline__ void project_bwd_sh_rows(const ProjectBwdArgs& a, int64_t blk, float* s_tw, float* s_mv,
                                                     float* s_cam) {
-    if (a.counters->status != 0) return;   // no gradient (and no Adam update) after a failed stage
+    if (CHECK && a.counters->status != 0) return;   // no gradient (and no Adam update) after a failed stage
     constexpr int K = (DEG + 1) * (DEG + 1);
     for (int t = threadIdx.x; t < a.n_views * 6; t += T) s_tw[t] = 0.f;
     for (int t = threadIdx.x; t < a.n_views * 12; t += T) {
@@ -381,9 +383,9 @@ __device__ __forceinline__ void adam_planes(float* P, float* M, float* V, int64_
 template <int T>
 constexpr int geo_mv_floats() { return 2 * 11 * T; }
 
-template <int DEG, bool FUSED_ADAM, int T>
+template <int DEG, bool FUSED_ADAM, int T, bool CHECK = true>
 __device__ __forceinline__ void project_bwd_geo_rows(const ProjectBwdArgs& a, int64_t blk, float* s_mv) {
-    if (a.counters->status != 0) return;
+    if (CHECK && a.counters->status != 0) return;
     const int64_t n = a.n;
     const int64_t i = blk * T + threadIdx.x;
     const bool live = i < n && a.visible[i] != 0;

@@ -254,7 +254,9 @@ struct FwdSmem {
 
 // The forward of work item `item` (the item-th tile of the work order), by the CTA's NT threads.
 // COUNT: fill the fragment and visit counters (a diagnostic option; off in the step).
-template <int TILE, int CHUNK, bool COUNT>
+// CHECK: leave if the status is set; off where the caller has checked it for the whole block, in a
+// kernel that can set it while it runs (threads that read it themselves could then disagree).
+template <int TILE, int CHUNK, bool COUNT, bool CHECK = true>
 __device__ __forceinline__ void render_fwd_tile(const FwdArgs& a, int item, FwdSmem<TILE, CHUNK>& S) {
     using TM = TileMap<TILE, kFwdPPT>;
     constexpr int NT = TM::NT;
@@ -266,7 +268,7 @@ __device__ __forceinline__ void render_fwd_tile(const FwdArgs& a, int item, FwdS
     auto& s_tgt = S.tgt;
     // (loads ordered so that the dependent chain order -> ranges / view -> ids -> records is
     // as short as possible: CTAs are short and this latency is paid once per tile)
-    const uint32_t status = a.counters->status;
+    const uint32_t status = CHECK ? a.counters->status : 0u;
     const int gt = a.order ? (int)a.order[item] : item;
     if (status != 0) return;
     const uint2 rg = a.ranges[gt];
@@ -607,13 +609,13 @@ __device__ __forceinline__ int bwd_slot(int lane) {
 // warp's list sets the time.  Whole steps, ten values reduced / by columns / JOINT: 2M Gaussians, 8
 // views 4100, 4089, 4055 us; 200k, 8 small views 868, 860, 894; 1M, 2 views 1348, 1327, 1344.  8 x 8
 // tiles, 1M, 2 views, as blocks with shared chunks / this: 1176, 1130.
-template <int TILE, bool JOINT, bool COUNT>
+template <int TILE, bool JOINT, bool COUNT, bool CHECK = true>
 __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, BwdWarpSmem& W) {
     constexpr int kPPT = kBwdPPT, WX = TILE / 8, R = WX * WX;
     auto& s_rec = W.rec;
     auto& s_id = W.id;
     auto& s_pos = W.pos;
-    const uint32_t status = a.counters->status;
+    const uint32_t status = CHECK ? a.counters->status : 0u;
     const int gt = a.order ? (int)a.order[item / R] : item / R;
     const int w = item % R;   // region: column w % WX, row w / WX (the forward's mask order)
     if (status != 0) return;
@@ -1004,7 +1006,11 @@ template <int DEG>
 __global__ void __launch_bounds__(kPersistThreads, 2) step_persistent_kernel(PersistentArgs P) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     PersistSmem<DEG>& S = *reinterpret_cast<PersistSmem<DEG>*>(s_raw);
-    if (P.counters->status != 0) return;   // failed earlier stage: every block leaves at once
+    // failed earlier stage: the block leaves at once.  One thread decides, here as in grid_barrier: a
+    // wait that gives up sets the status while other blocks start or work on a phase.
+    if (threadIdx.x == 0) S.ok = *(volatile uint32_t*)&P.counters->status == 0u;
+    __syncthreads();
+    if (!S.ok) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     {   // phase 0
         const int64_t E = (int64_t)P.counters->n_entries;
@@ -1023,7 +1029,7 @@ __global__ void __launch_bounds__(kPersistThreads, 2) step_persistent_kernel(Per
         const unsigned int t = S.item;
         __syncthreads();
         if (t >= (unsigned int)P.total_tiles) break;
-        render_fwd_tile<16, 256, false>(P.fwd, (int)t, S.u.fwd);
+        render_fwd_tile<16, 256, false, false>(P.fwd, (int)t, S.u.fwd);
     }
     if (!grid_barrier<DEG>(P, (int)blockIdx.x != P.skip_block, S)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -1037,18 +1043,18 @@ __global__ void __launch_bounds__(kPersistThreads, 2) step_persistent_kernel(Per
         if (lane == 0) item = atomicAdd(&P.sync->q_bwd, 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
         if (item >= 4u * (unsigned int)P.total_tiles) break;
-        render_bwd_region<16, false, false>(P.bwd, (int)item, S.u.bwd[warp]);
+        render_bwd_region<16, false, false, false>(P.bwd, (int)item, S.u.bwd[warp]);
     }
     if (!grid_barrier<DEG>(P, true, S)) return;
-    project_bwd_entry_part(P.pb, blockIdx.x, gridDim.x, S.tw);   // phase 3
+    project_bwd_entry_part<false>(P.pb, blockIdx.x, gridDim.x, S.tw);   // phase 3
     if (!grid_barrier<DEG>(P, true, S)) return;
     for (int64_t blk = blockIdx.x; blk * kPersistThreads < P.pb.n; blk += gridDim.x) {   // phase 4a
-        project_bwd_sh_rows<DEG, true, kPersistThreads>(P.pb, blk, S.tw, S.u.mv, S.cam);
+        project_bwd_sh_rows<DEG, true, kPersistThreads, false>(P.pb, blk, S.tw, S.u.mv, S.cam);
         __syncthreads();
     }
     if (!grid_barrier<DEG>(P, true, S)) return;
     for (int64_t blk = blockIdx.x; blk * kPersistThreads < P.pb.n; blk += gridDim.x)   // phase 4b
-        project_bwd_geo_rows<DEG, true, kPersistThreads>(P.pb, blk, S.u.gmv);
+        project_bwd_geo_rows<DEG, true, kPersistThreads, false>(P.pb, blk, S.u.gmv);
 }
 
 template <int DEG>
