@@ -22,9 +22,10 @@
 namespace gs {
 
 // ----------------------------------------------------------------------------------------
-// Block-wide scans.
+// Block-wide scans.  The sums of a warp are taken in 32 bits, those across warps in U.
 // ----------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t block_exclusive_scan_1024(uint32_t x, uint32_t* s_warp, uint32_t& total) {
+template <typename U>
+__device__ __forceinline__ U block_exclusive_scan_1024(uint32_t x, U* s_warp, U& total) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t inc = x;
 #pragma unroll
@@ -35,11 +36,11 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_1024(uint32_t x, uint32
     if (lane == 31) s_warp[w] = inc;
     __syncthreads();
     if (w == 0) {
-        uint32_t t = lane < (int)(blockDim.x >> 5) ? s_warp[lane] : 0u;
-        uint32_t ti = t;
+        U t = lane < (int)(blockDim.x >> 5) ? s_warp[lane] : U(0);
+        U ti = t;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, ti, o);
+            const U y = __shfl_up_sync(0xffffffffu, ti, o);
             if (lane >= o) ti += y;
         }
         s_warp[lane] = ti - t;
@@ -47,7 +48,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_1024(uint32_t x, uint32
     }
     __syncthreads();
     total = s_warp[32];
-    const uint32_t r = s_warp[w] + inc - x;
+    const U r = s_warp[w] + (inc - x);
     __syncthreads();
     return r;
 }
@@ -265,8 +266,8 @@ __device__ __forceinline__ uint32_t rect_count(uint2 r) { return (r.y & 0xFFFFu)
 // blocks take chunks of kPairScanChunk entries in turn.
 __global__ void __launch_bounds__(kPairScanThreads) pair_offsets_kernel(BinArgs a) {
     pdl_begin();
-    __shared__ uint32_t s[33], s_chunk;
-    __shared__ unsigned long long s_base;
+    __shared__ unsigned long long s[33], s_base;
+    __shared__ uint32_t s_chunk;
     __shared__ bool s_ok;
     const int64_t E = (int64_t)a.counters->n_entries, VN = (int64_t)a.n_views * a.n;
     const int64_t n_chunks = (E + kPairScanChunk - 1) / kPairScanChunk;
@@ -299,8 +300,10 @@ __global__ void __launch_bounds__(kPairScanThreads) pair_offsets_kernel(BinArgs 
                 a.srt[2 * VN + e0 + k] = r[k].z;
             }
         }
-        uint32_t tot;
-        const uint32_t local = block_exclusive_scan_1024(sum, s, tot);
+        // an entry covers at most (16384 / 8)^2 = 2^22 tiles: a warp's 128 entries fit 32 bits, the
+        // chunk's 2048 do not
+        unsigned long long tot;
+        const unsigned long long local = block_exclusive_scan_1024(sum, s, tot);
         if (threadIdx.x < 32) {
             bool ok = true;
             const unsigned long long before = lb_scan_warp(a.pair_scan, ch, tot, a.counters, ok);
