@@ -481,7 +481,7 @@ cudaError_t launch_emit(const BinArgs& a, cudaStream_t st) {
 // Radix sort with BITS-bit digits (8 or 9), keys K = uint32_t or unsigned long long.
 // ----------------------------------------------------------------------------------------
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kItemsPerWarp = kSortChunk / kSortWarps;   // 512
+constexpr int kItemsPerWarp = kSortChunk / kSortWarps;   // 256
 constexpr int kHistThreads = 512;
 constexpr int kHistItems = kSortChunk / kHistThreads;    // 8
 
@@ -582,16 +582,6 @@ __device__ __forceinline__ void block_exclusive_scan_dpt(const uint32_t (&x)[DPT
         r += x[q];
     }
     __syncthreads();
-}
-
-constexpr int kSortBlocksPerSM = kSortThreads == 256 ? 3 : 2;
-
-// Blocks of a pass: at most the resident ones, which bounds the look-back.
-static int sort_grid(int64_t capacity) {
-    int64_t g = (int64_t)device_sms() * kSortBlocksPerSM;
-    if (g > kSortMaxGrid) g = kSortMaxGrid;
-    const int64_t chunks = sort_chunks(capacity);
-    return (int)(chunks < 1 ? 1 : (chunks < g ? chunks : g));
 }
 
 constexpr int kLbBatch = 8;   // look-back words loaded at a time
@@ -848,7 +838,7 @@ static cudaError_t launch_pass(const SortArgs& a, int in_buf, int shift, int pas
         return cudaFuncSetAttribute(sort_pass_kernel<K, BITS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     });
     if (e != cudaSuccess) return e;
-    launch_pdl(sort_pass_kernel<K, BITS>, sort_grid(a.capacity), kSortThreads, smem, st, a, in_buf, shift, pass, next_shift,
+    launch_pdl(sort_pass_kernel<K, BITS>, sort_grid(a.capacity, device_sms()), kSortThreads, smem, st, a, in_buf, shift, pass, next_shift,
                                                                               next_mask);
     return cudaGetLastError();
 }
@@ -879,7 +869,7 @@ cudaError_t launch_sort64(const SortArgs& a, int n_passes, const int* shifts, cu
 }
 
 cudaError_t launch_sort_count64(const SortArgs& a, int shift, cudaStream_t st) {
-    sort_count_kernel<<<sort_grid(a.capacity), kHistThreads, 0, st>>>(a, shift);
+    sort_count_kernel<<<sort_grid(a.capacity, device_sms()), kHistThreads, 0, st>>>(a, shift);
     return cudaGetLastError();
 }
 

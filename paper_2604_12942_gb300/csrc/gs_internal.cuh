@@ -16,6 +16,7 @@ constexpr int kSortBins = 256;                    // 8-bit digits (64-bit keys)
 constexpr int kSortMaxBins = 512;                 // up to 9-bit digits (32-bit keys)
 constexpr int kSortThreads = 512;
 constexpr int kSortItems = 8;                      // per thread per chunk
+constexpr int kSortBlocksPerSM = 2;                // resident blocks of a pass
 constexpr int kSortGroup = 16;                     // blocks per look-back group
 constexpr int kSortMaxGrid = 512;                  // blocks of a sort pass (at most)
 constexpr int kSortChunk = kSortThreads * kSortItems;
@@ -487,7 +488,7 @@ __device__ __forceinline__ uint32_t lb_state(lbword w, uint32_t tag) {
     return (t >> 2) == tag ? (t & 3u) : 0u;
 }
 __device__ __forceinline__ unsigned long long lb_value(lbword w) { return w & ((1ull << 56) - 1); }
-// the same in 32 bits, for totals below 2^24 (state and tag in the top byte)
+// the same in 32 bits, for totals below 2^24 (state and tag in the top byte; sort_grid sees to it)
 __device__ __forceinline__ void lb_store(uint32_t* p, uint32_t tag, uint32_t state, uint32_t v) {
     const uint32_t w = ((tag * 4 + state) << 24) | v;
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(w) : "memory");

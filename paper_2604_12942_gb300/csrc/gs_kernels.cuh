@@ -97,6 +97,19 @@ inline size_t sort_lookback_bytes(int64_t capacity, int bits) {
     return kSortGroupBytes + ((sizeof(uint32_t) * (size_t)blocks) << bits);
 }
 
+// Blocks of a pass: the resident ones, or, on a device (or a partition of one) too small for its
+// capacity, as many as keep a block's run below the 2^24 keys that its look-back words can count.
+// Blocks beyond the resident ones start as others end: a block only waits for earlier tickets.
+inline int sort_grid(int64_t capacity, int sms) {
+    constexpr int64_t kMaxRun = ((1 << 24) - 1) / kSortChunk;   // chunks of a block
+    static_assert(kSortMaxGrid * kMaxRun * kSortChunk >= (int64_t)1 << 32, "the largest capacity");
+    const int64_t chunks = sort_chunks(capacity), need = (chunks + kMaxRun - 1) / kMaxRun;
+    int64_t g = (int64_t)sms * kSortBlocksPerSM;
+    g = g < need ? need : g;
+    g = g > kSortMaxGrid ? kSortMaxGrid : g;
+    return (int)(chunks < 1 ? 1 : (chunks < g ? chunks : g));
+}
+
 struct RangeArgs {
     const uint32_t* keys;      // sorted global tile ids
     uint2* ranges;
