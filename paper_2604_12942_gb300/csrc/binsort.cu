@@ -587,10 +587,10 @@ __device__ __forceinline__ void block_exclusive_scan_dpt(const uint32_t (&x)[DPT
 constexpr int kLbBatch = 8;   // look-back words loaded at a time
 
 // Sum of the words col[j << bits], j = last, last - 1, ..., first, up to and including the first
-// that holds an inclusive prefix (state 2).  ok is cleared if a wait gave up.
+// that holds an inclusive prefix (state 2).  ok is cleared after `limit` polls of words not there.
 template <typename W>
-__device__ __forceinline__ uint32_t lb_sum(const W* col, int bits, int64_t last, int64_t first, uint32_t tag,
-                                           const Counters* c, bool& ok) {
+__device__ __forceinline__ uint32_t lb_sum(const W* col, int bits, int64_t last, int64_t first, uint32_t tag, int limit,
+                                           bool& ok) {
     uint32_t sum = 0;
     int spin = 0;
     for (int64_t j = last; j >= first && ok; j -= kLbBatch) {
@@ -603,7 +603,7 @@ __device__ __forceinline__ uint32_t lb_sum(const W* col, int bits, int64_t last,
             if (full || j - u < first || !ok) continue;
             uint32_t st = lb_state(wd[u], tag);
             while (st == 0) {
-                if (++spin > kLbSpin || ((spin & 1023) == 0 && *(const volatile uint32_t*)&c->status != 0)) {
+                if (++spin > limit) {
                     ok = false;
                     break;
                 }
@@ -628,7 +628,9 @@ __device__ __forceinline__ uint32_t lb_sum(const W* col, int bits, int64_t last,
 // most of the pass.  At 7k / 356k / 1.9M entries a pass takes 9 / 12 / 27 us, at 8.7M pairs 77 to 90
 // (separate kernels: 20 / 26 / 38, 76).  (Chunks dealt out one by one, each with a look-back of its own, lose at large
 // counts: a look-back step is about a microsecond across the two dies, 85 against 60 us a pass at
-// 8.7M pairs.)  The next pass's digits are counted on the way out.
+// 8.7M pairs.)  The next pass's digits are counted on the way out.  Every wait is bounded, and a
+// block whose wait gives up counts the keys before its run itself, so that a pass has one result:
+// the callers that sort without a status word to report would have nothing to tell a failure by.
 template <typename K, int BITS>
 __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSM)
     sort_pass_kernel(SortArgs a, int in_buf, int shift, int pass, int next_shift, uint32_t next_mask) {
@@ -712,7 +714,6 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSM)
         lb_store(words + ((size_t)t << BITS) + d0 + q, tag, 1, mine[q]);
         S.next[d0 + q] = 0;
     }
-    bool ok = true;
     for (int64_t base = lo; base < hi; base += kSortChunk) {
         const int m = chunk_size(base);
         for (int k = threadIdx.x; k < kSortWarps * BINS; k += kSortThreads) (&S.wcnt[0][0])[k] = 0;
@@ -774,22 +775,34 @@ __global__ void __launch_bounds__(kSortThreads, kSortBlocksPerSM)
             // counts of the blocks before this one: those of its group, then the groups before
             const int64_t g = t / kSortGroup;
             const bool last = t % kSortGroup == kSortGroup - 1;
+            bool ok = a.spin > 0;
 #pragma unroll
             for (int q = 0; q < DPT; q++) {
                 const int d = d0 + q;
                 if (d >= BINS) continue;
-                uint32_t before = lb_sum(words + d, BITS, t - 1, g * kSortGroup, tag, a.counters, ok);
+                uint32_t before = lb_sum(words + d, BITS, t - 1, g * kSortGroup, tag, a.spin, ok);
                 if (last && ok)
                     lb_store(groups + ((size_t)g << BITS) + d, tag, g == 0 ? 2u : 1u, (unsigned long long)(before + mine[q]));
                 if (g > 0 && ok) {
-                    before += lb_sum(groups + d, BITS, g - 1, 0, tag, a.counters, ok);
+                    before += lb_sum(groups + d, BITS, g - 1, 0, tag, a.spin, ok);
                     if (last && ok) lb_store(groups + ((size_t)g << BITS) + d, tag, 2, (unsigned long long)(before + mine[q]));
                 }
                 S.run[d] = dbase[q] + before;
             }
+            // a wait that gives up: the counts from the keys before the run, which the pass only reads
             if (__syncthreads_or(!ok)) {
-                if (threadIdx.x == 0) set_status(a.counters, GS_ERR_TIMEOUT);
-                return;
+                for (int d = threadIdx.x; d < BINS; d += kSortThreads) S.run[d] = 0;
+                __syncthreads();
+                for (int64_t i = threadIdx.x; i < lo; i += kSortThreads)
+                    atomicAdd(&S.run[digit_of<BITS>(kin[i], shift, a.digit_mask)], 1u);
+                __syncthreads();
+#pragma unroll
+                for (int q = 0; q < DPT; q++) {
+                    const int d = d0 + q;
+                    if (d >= BINS) continue;
+                    if (last) lb_store(groups + ((size_t)g << BITS) + d, tag, 2, (unsigned long long)(S.run[d] + mine[q]));
+                    S.run[d] += dbase[q];
+                }
             }
         }
 #pragma unroll

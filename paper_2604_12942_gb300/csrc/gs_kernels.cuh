@@ -85,6 +85,7 @@ struct SortArgs {
     Counters* counters;        // status word (a set status skips the sort)
     const unsigned long long* count;   // element count, read on the device
     int64_t capacity;          // upper bound of it (grid sizes)
+    int spin = kLbSpin;        // polls of a wait before a block counts the keys before it itself
     uint32_t tag = 1;          // look-back tags tag .. tag + passes - 1 (below 64)
     uint32_t digit_mask = 0xFFFFFFFFu;  // ANDed into every digit of the pass (a partial top digit)
 };
