@@ -11,10 +11,9 @@
 // The proximity test hashes the map means into cubic cells of side 1.001 * radius; a new mean
 // looks at the 27 cells around its own and is redundant if any map mean there lies strictly
 // within radius (squared distance summed in FP32 in x, y, z order).
-#include "gs_internal.cuh"
-#include "gs_kernels.cuh"
 #include <cstddef>
 #include <math_constants.h>
+
 #include "gs_kernels.cuh"
 
 namespace gs {
@@ -341,8 +340,8 @@ cudaError_t exclusive_scan_u32(const uint32_t* x, int64_t n, uint32_t* out, uint
 }
 
 // ---------------------------------------------------------------------------------------
-// Positions of the update: the flags of each chunk of 1024 rows are summed (by value: a row moves
-// on the rows behind it by its flag) by a warp, and the block that finishes last scans the sums,
+// Positions of the update: the rows of each chunk of 1024 whose flag is not 0 are counted by a
+// warp, and the block that finishes last scans the counts,
 // first those of the map, then those of the new rows.  The compaction ranks the rows inside their
 // chunk itself, so that no position per row is written (9 us for 2M + 200k flags; the scans of
 // all rows took 37).
@@ -386,10 +385,10 @@ __global__ void __launch_bounds__(kMuThreads) chunk_sum_kernel(const uint8_t* ke
             const int64_t i = i0 + k * 256;
             if (((uintptr_t)f & 7) == 0 && i + 8 <= m) {
                 const uint2 w = *reinterpret_cast<const uint2*>(f + i);
-                x = __dp4a(w.x, 0x01010101u, __dp4a(w.y, 0x01010101u, x));
+                x = __dp4a(__vsetne4(w.x, 0u), 0x01010101u, __dp4a(__vsetne4(w.y, 0u), 0x01010101u, x));
             } else {
                 for (int j = 0; j < 8; j++)
-                    if (i + j < m) x += f[i + j];
+                    if (i + j < m) x += f[i + j] != 0;
             }
         }
         x = warp_sum(x);
@@ -416,12 +415,12 @@ __global__ void __launch_bounds__(kMuThreads) compact_kernel(MapUpdateArgs a) {
     const int64_t c = old ? (int64_t)blockIdx.x : (int64_t)blockIdx.x - a.n_chunks;
     const int64_t i0 = c * kChunkRows + threadIdx.x, n = old ? a.n : a.n_new;
     const uint8_t* flag = old ? a.keep : a.accept;
-    // the flags of the 4 rows in 16-bit fields (a field's sum over the block is at most 255 * 256)
+    // the flags of the 4 rows in 16-bit fields (a field's sum over the block is at most 256)
     unsigned long long f = 0, tot;
 #pragma unroll
     for (int k = 0; k < kRowsPerThread; k++) {
         const int64_t i = i0 + k * kMuThreads;
-        if (i < n) f |= (unsigned long long)(flag ? flag[i] : 1u) << (16 * k);
+        if (i < n) f |= (unsigned long long)(!flag || flag[i]) << (16 * k);
     }
     const unsigned long long rank = block_scan_excl(f, tot);
     int64_t o[kRowsPerThread], base = (old ? 0 : a.n_keep) + (flag ? (int64_t)a.chunk_pos[blockIdx.x] : c * kChunkRows);
