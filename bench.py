@@ -324,10 +324,8 @@ def run_gpu(args, rank, world):
     if args.tile == 0 or args.chunk == 0:
         from paper_2604_12942_gb300 import autotune
         key = autotune.cache_key(torch.cuda.get_device_name(dev), n, SIZES, 3)
-        tiles = (args.tile,) if args.tile else autotune.TILES
-        chunks = (args.chunk,) if args.chunk else autotune.CHUNKS
         ch = autotune.tune(lambda t, c: autotune.time_mapping_step(planes0, 3, cams, (trgb, tdep), t, c, cap),
-                           key, [(t, c) for t in tiles for c in chunks], force=args.retune)
+                           key, autotune.step_candidates(args.tile, args.chunk), force=args.retune)
         args.tile, args.chunk = ch.tile, ch.chunk
         tune = {"tile": ch.tile, "chunk": ch.chunk, "ms_per_step": round(ch.ms, 4), "table": ch.table, "key": key}
     opts = gs.default_opts(tile=args.tile, chunk=args.chunk)
@@ -533,9 +531,9 @@ def a9_measure(args, planes0, cams, trgb, tdep, cap, st, graph_ms):
     import torch
 
     import paper_2604_12942_gb300 as gs
-    if args.tile != 16 or args.chunk != 256:
-        return {"note": f"persistent form needs 16x256 (the autotuned shape is {args.tile}x{args.chunk})"}
-    opts = gs.default_opts(tile=16, chunk=256, persistent=1)
+    if args.tile != 16:
+        return {"note": f"persistent form needs 16 x 16 tiles (the autotuned shape is {args.tile}x{args.chunk})"}
+    opts = gs.default_opts(tile=16, chunk=args.chunk, persistent=1)
     ps = gs.MappingStep(planes0.clone(), 3, cams, opts, max_pairs=cap)
     for _ in range(2):
         ps(trgb, tdep)

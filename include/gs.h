@@ -110,7 +110,7 @@ typedef struct {
     /* Launch form of gs_step's compositing, backward and update stages (a9):                   */
     int32_t persistent;      /* 1: forward compositing, backward compositing, projection backward
                                 and Adam run as ONE cooperative persistent kernel whose phases are
-                                separated by bounded grid barriers (needs tile 16, chunk 256, the
+                                separated by bounded grid barriers (needs tile 16, the
                                 fused L1 loss and optimize = 1; else gs_step returns
                                 GS_ERR_UNSUPPORTED); 0 (default): one kernel per stage */
     int32_t sync_spin_limit; /* polls (about 0.1 us apart) before a grid-barrier wait gives up and

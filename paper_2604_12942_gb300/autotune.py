@@ -1,7 +1,7 @@
 """Autotuner of the batched mapping step's kernel shape.
 
-Picks the tile size (8x8 or 16x16 pixels) and the per-CTA Gaussian chunk staged in shared
-memory (32, 64, 128 or 256) by timing whole steps on the device with CUDA events, and
+Picks the tile size (8x8 or 16x16 pixels) and, for 8x8 tiles, the Gaussian chunk that the forward
+stages in shared memory (32, 64, 128 or 256; 16x16 tiles always run 256) by timing whole steps on the device with CUDA events, and
 caches the choice in a JSON file keyed by (GPU name, Gaussian-count bucket, image-size
 set, SH degree).  Host logic only; the timed work is the library's kernels.
 """
@@ -16,6 +16,20 @@ from dataclasses import dataclass
 TILES = (8, 16)
 CHUNKS = (32, 64, 128, 256)
 _lock = threading.Lock()
+
+
+def step_candidates(tile: int = 0, chunk: int = 0) -> list:
+    """The (tile, chunk) shapes of the mapping step that differ in what they run, within the given
+    tile or chunk (0: any)."""
+    return [(t, c) for t in TILES if tile in (0, t)
+            for c in ((chunk,) if chunk else CHUNKS if t == 8 else (256,))]
+
+
+def step_candidates(tile: int = 0, chunk: int = 0) -> list:
+    """The (tile, chunk) shapes of the mapping step that differ in what they run, within the given
+    tile or chunk (0: any)."""
+    return [(t, c) for t in TILES if tile in (0, t)
+            for c in ((chunk,) if chunk else CHUNKS if t == 8 else (256,))]
 
 
 def cache_path() -> str:

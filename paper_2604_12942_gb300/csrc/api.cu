@@ -756,10 +756,10 @@ static gs_status check_step(gs_gaussians* params, gs_gaussians* grads, gs_gaussi
     if ((s = check_adam(params, grads, m, v, io->lr, io->b1, io->b2, io->eps)) != GS_OK) return s;
     if (params->n != L->n) return fail(GS_ERR_INVALID_ARG, "n does not match the layout");
     if (opts->persistent &&
-        (opts->tile != 16 || opts->chunk != 256 || !io->optimize || opts->lambda_ssim > 0.f || opts->mask_erode >= 0 ||
+        (opts->tile != 16 || !io->optimize || opts->lambda_ssim > 0.f || opts->mask_erode >= 0 ||
          opts->count_fragments))
-        return fail(GS_ERR_UNSUPPORTED, "the persistent step needs tile 16, chunk 256, optimize = 1, the fused L1 loss "
-                                        "and no fragment counters");
+        return fail(GS_ERR_UNSUPPORTED, "the persistent step needs tile 16, optimize = 1, the fused L1 loss and no "
+                                        "fragment counters");
     return geometry_for(L, cams, opts, G);
 }
 
