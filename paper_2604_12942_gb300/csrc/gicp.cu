@@ -351,7 +351,10 @@ __global__ void __launch_bounds__(kGThreads) gicp_search_kernel(GicpMap src, int
 // at a small fraction of the FP32 rate, so the kernel is written for few FP64 instructions:
 // a block first lists its matched pairs, so that warps are full, and the algebra is taken apart.
 // The planar covariance R diag(1, 1, 1e-3) R^T is I - 0.999 n n^T with n the column of R that
-// gets 1e-3, so Sigma~_n + R Sigma~_m R^T = 2 I - 0.999 (n n^T + m m^T), m = R n_m; with O its
+// gets 1e-3, so Sigma~_n + R Sigma~_m R^T = I + R R^T - 0.999 (n n^T + m m^T), m = R n_m (R R^T is
+// formed once a thread and not taken for I: the caller's first transform is a rotation to its own
+// rounding only, and every later one keeps what it had; with 2 I in its place a transform given in
+// FP32 left ten times the error, and one 1e-3 off a rotation met another minimum); with O its
 // inverse and q^ the cross-product matrix of T mu_m the blocks of J^T O J (J = [-I | q^]) are
 // O, -O q^ and -q^ O q^, those of J^T O r are -O r and -q^ O r.  About 190 FP64 operations a
 // pair where the matrix products spelled out took about 700: 41 us an evaluation at 80k source
@@ -480,6 +483,9 @@ __global__ void __launch_bounds__(kNormalThreads) gicp_normal_kernel(GicpMap src
     double T[12];
 #pragma unroll
     for (int k = 0; k < 12; k++) T[k] = st->T[k];
+    // I + R R^T: xx xy xz yy yz zz
+    auto rr = [&](int a, int b) { return T[4 * a] * T[4 * b] + T[4 * a + 1] * T[4 * b + 1] + T[4 * a + 2] * T[4 * b + 2]; };
+    const double B0 = 1.0 + rr(0, 0), B1 = rr(0, 1), B2 = rr(0, 2), B3 = 1.0 + rr(1, 1), B4 = rr(1, 2), B5 = 1.0 + rr(2, 2);
     const uint32_t cnt = st->n_list;
     const int64_t ns = src.n, nt = tar.n;
     double acc[32];
@@ -512,12 +518,12 @@ __global__ void __launch_bounds__(kNormalThreads) gicp_normal_kernel(GicpMap src
             planar_normal(tar, j, n);
 #pragma unroll
             for (int e = 0; e < 3; e++) mr[e] = T[4 * e] * nm[0] + T[4 * e + 1] * nm[1] + T[4 * e + 2] * nm[2];
-            // A = 2 I - 0.999 (n n^T + m m^T): xx xy xz yy yz zz
+            // A = I + R R^T - 0.999 (n n^T + m m^T): xx xy xz yy yz zz
             const double kn[3] = {kPlanar * n[0], kPlanar * n[1], kPlanar * n[2]};
             const double km[3] = {kPlanar * mr[0], kPlanar * mr[1], kPlanar * mr[2]};
-            const double A0 = 2.0 - kn[0] * n[0] - km[0] * mr[0], A1 = -kn[0] * n[1] - km[0] * mr[1],
-                         A2 = -kn[0] * n[2] - km[0] * mr[2], A3 = 2.0 - kn[1] * n[1] - km[1] * mr[1],
-                         A4 = -kn[1] * n[2] - km[1] * mr[2], A5 = 2.0 - kn[2] * n[2] - km[2] * mr[2];
+            const double A0 = B0 - kn[0] * n[0] - km[0] * mr[0], A1 = B1 - kn[0] * n[1] - km[0] * mr[1],
+                         A2 = B2 - kn[0] * n[2] - km[0] * mr[2], A3 = B3 - kn[1] * n[1] - km[1] * mr[1],
+                         A4 = B4 - kn[1] * n[2] - km[1] * mr[2], A5 = B5 - kn[2] * n[2] - km[2] * mr[2];
             // inverse by the adjugate
             const double c0 = A3 * A5 - A4 * A4, c1 = A2 * A4 - A1 * A5, c2 = A1 * A4 - A2 * A3;
             const double id = 1.0 / (A0 * c0 + A1 * c1 + A2 * c2);
