@@ -541,43 +541,47 @@ __device__ __forceinline__ float fold(float own, float other, int x) {
 
 // What a visit adds to its Gaussian's record, from lane sums over the lane's two pixels, which lie
 // in one column of the region (one dx):
-//   A0 = sum h, A1 = sum h dy, A2 = sum h dy^2, D = sum g_D w, c0..c2 = sum g_C w.
+//   X = sum h h_x, Y = sum h h_y, A0 = sum h, A1 = sum h dy, A2 = sum h dy^2, D = sum g_D w,
+//   c0..c2 = sum g_C w.
+// X and Y are summed pixel by pixel: from A0 and A1 (a dx A0 + b A1 a column) two large sums would
+// cancel for a thin slanted Gaussian, after their rounding instead of before it (for axes 10 : 1,
+// 1.4 times the error).
 struct BwdSums {
-    float A0, A1, A2, D, c0, c1, c2;
-    float dx, a, b, c, inv_o;   // the column's dx; the record's conic and 1 / o
+    float X, Y, A0, A1, A2, D, c0, c1, c2;
+    float dx, inv_o;   // the column's dx; 1 / the record's o
 };
 
 // Warp totals of N visits, stage by stage over all of them so that their shuffles overlap.  The
-// sums over rows come first (lane distances 16 and 8), on seven values a visit instead of ten; dx
-// and the conic (a, b, c) then turn the three geometry sums of a column into its six terms, and
-// the lanes 8 r + x of row r hold three (r = 0, 1) or two terms for the sums over columns:
+// sums over rows come first (lane distances 16 and 8), on nine values a visit instead of ten; dx
+// then makes h dx^2 and h dx dy of a column's A0 and A1, and the lanes 8 r + x of row r hold three
+// (r = 0, 1) or two terms for the sums over columns:
 //   r = 0: h h_x, h h_y, h dx dy   r = 1: dL/dalpha G, h dx^2, h dy^2   r = 2: D, c0   r = 3: c1, c2
 // z[k] is the total for record slot bwd_slot(lane) of visit k.
 template <int N>
 __device__ __forceinline__ void bwd_reduce(int lane, const BwdSums (&s)[N], float (&z)[N]) {
     const bool hi = lane & 16, odd = lane & 8, x4 = lane & 4, x2 = lane & 2;
     const bool r0 = !hi && !odd, r1 = !hi && odd;
-    float k0[N], k1[N], k2[N], k3[N], p[N], q[N], v0[N], v1[N], v2[N];
+    float k0[N], k1[N], k2[N], k3[N], k4[N], p[N], q[N], v0[N], v1[N], v2[N];
 #pragma unroll
     for (int k = 0; k < N; k++) {
-        k0[k] = fold(hi ? s[k].D : s[k].A0, hi ? s[k].A0 : s[k].D, 16);
-        k1[k] = fold(hi ? s[k].c1 : s[k].A1, hi ? s[k].A1 : s[k].c1, 16);
-        k2[k] = fold(hi ? s[k].c2 : s[k].A2, hi ? s[k].A2 : s[k].c2, 16);
-        k3[k] = fold(s[k].c0, s[k].c0, 16);
+        k0[k] = fold(hi ? s[k].D : s[k].X, hi ? s[k].X : s[k].D, 16);
+        k1[k] = fold(hi ? s[k].c0 : s[k].Y, hi ? s[k].Y : s[k].c0, 16);
+        k2[k] = fold(hi ? s[k].c1 : s[k].A0, hi ? s[k].A0 : s[k].c1, 16);
+        k3[k] = fold(hi ? s[k].c2 : s[k].A2, hi ? s[k].A2 : s[k].c2, 16);
+        k4[k] = fold(s[k].A1, s[k].A1, 16);
     }
-    // p: A0, A0, D, c1 and q: A1, A2, c0, c2 of rows 0 .. 3
+    // p: X, A0, D, c1 and q: Y, A2, c0, c2 of rows 0 .. 3
 #pragma unroll
     for (int k = 0; k < N; k++) {
-        p[k] = fold(hi && odd ? k1[k] : k0[k], hi && !odd ? k1[k] : k0[k], 8);
-        const float e = hi ? k3[k] : k1[k];
-        q[k] = fold(odd ? k2[k] : e, odd ? e : k2[k], 8);
+        p[k] = fold(odd ? k2[k] : k0[k], odd ? k0[k] : k2[k], 8);
+        q[k] = fold(odd ? k3[k] : k1[k], odd ? k1[k] : k3[k], 8);
+        k4[k] = fold(k4[k], k4[k], 8);
     }
 #pragma unroll
     for (int k = 0; k < N; k++) {
-        // (dx times a, b and dx do not wait for the sums)
-        v0[k] = r0 ? fmaf(s[k].a * s[k].dx, p[k], s[k].b * q[k]) : (r1 ? p[k] * s[k].inv_o : p[k]);
-        v1[k] = r0 ? fmaf(s[k].b * s[k].dx, p[k], s[k].c * q[k]) : (r1 ? s[k].dx * s[k].dx * p[k] : q[k]);
-        v2[k] = r0 ? s[k].dx * q[k] : q[k];
+        v0[k] = r1 ? p[k] * s[k].inv_o : p[k];
+        v1[k] = r1 ? s[k].dx * s[k].dx * p[k] : q[k];
+        v2[k] = r0 ? s[k].dx * k4[k] : q[k];
     }
 #pragma unroll
     for (int k = 0; k < N; k++) {
@@ -602,13 +606,16 @@ __device__ __forceinline__ int bwd_slot(int lane) {
 // The backward of work item `item` = R t + w: region w of the R = (TILE / 8)^2 regions of the t-th
 // tile of the work order, by one warp with its own shared memory W.
 //
-// What bounds it: the issue slots while the chip is full (73% busy, 61 registers, 32 one-warp blocks
-// an SM), then the longest lists, each walked by one warp.  Sums by columns and alpha = 0 in place
-// of three selects a pixel save about 17 of 175 instructions a visit.  JOINT reduces two visits at
-// once, so that their shuffles overlap: better while many warps share an SM, worse where a lone
-// warp's list sets the time.  Whole steps, ten values reduced / by columns / JOINT: 2M Gaussians, 8
-// views 4100, 4089, 4055 us; 200k, 8 small views 868, 860, 894; 1M, 2 views 1348, 1327, 1344.  8 x 8
-// tiles, 1M, 2 views, as blocks with shared chunks / this: 1176, 1130.
+// What bounds it: issue slots and the latency of a visit's chain while the chip is full (63 registers,
+// 32 one-warp blocks an SM; a tenth fewer instructions a visit moved the largest step by 1%), then
+// the longest lists, each walked by one warp.  alpha = 0 takes the place of three selects a pixel,
+// and sums by columns that of three products a pixel and two shuffles a visit.  JOINT reduces two
+// visits at once, so that their shuffles overlap: better while many warps share an SM, worse where a
+// lone warp's list sets the time.  Whole steps, ten values reduced / seven, h_x and h_y by columns too
+// / that with JOINT: 2M Gaussians, 8 views 4100, 4089, 4055 us; 200k, 8 small views 868, 860, 894;
+// 1M, 2 views 1348, 1327, 1344.  The nine values of this form against the seven, on one card: 3717
+// and 3730, 839 and 841, 1298 and 1298 us.  8 x 8 tiles, 1M, 2 views, as blocks with shared chunks /
+// this: 1176, 1130.
 template <int TILE, bool JOINT, bool COUNT, bool CHECK = true>
 __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, BwdWarpSmem& W) {
     constexpr int kPPT = kBwdPPT, WX = TILE / 8, R = WX * WX;
@@ -702,7 +709,7 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
         // changes nothing and is skipped whole
         struct Alphas {
             float dx;
-            float2 dy, a0;
+            float2 dy, hx, hy, a0;
             bool c0, c1;
         };
         auto alphas = [&](int t, Alphas& P) {
@@ -711,6 +718,8 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
             P.dx = px[0] - r0.x;
             P.dy = __fadd2_rn(py2, dup2(-r0.y));
             const FragE2 fe = frag_exponent2(dup2(P.dx), P.dy, dup2(r1.x), dup2(r1.y), dup2(r1.z));
+            P.hx = fe.hx;
+            P.hy = fe.hy;
             P.a0 = __fmul2_rn(dup2(r0.w), make_float2(ex2_approx(fe.e.x), ex2_approx(fe.e.y)));
             P.c0 = j < last[0] && !(fminf(amax, P.a0.x) < amin);
             P.c1 = j < last[1] && !(fminf(amax, P.a0.y) < amin);
@@ -726,6 +735,7 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
         auto adjoint = [&](int t, const Alphas& P) {
             const float4 cz = s_rec[b][t][2];   // colour and depth
             const float a0s[2] = {P.a0.x, P.a0.y}, dys[2] = {P.dy.x, P.dy.y};
+            const float hxs[2] = {P.hx.x, P.hx.y}, hys[2] = {P.hy.x, P.hy.y};
             const bool cq[2] = {P.c0, P.c1};
             BwdSums s = {};
 #pragma unroll
@@ -744,16 +754,14 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
                 s.c2 = fmaf(gc2[q], wgt, s.c2);
                 s.D = fmaf(gd[q], wgt, s.D);
                 const float h = cq[q] && a0 < amax ? dLda * a0 : 0.f;   // the 0.99 clamp stops the gradient
-                const float hy = h * dys[q];
+                const float hdy = h * dys[q];
+                s.X = fmaf(h, hxs[q], s.X);
+                s.Y = fmaf(h, hys[q], s.Y);
                 s.A0 += h;
-                s.A1 += hy;
-                s.A2 = fmaf(hy, dys[q], s.A2);
+                s.A1 += hdy;
+                s.A2 = fmaf(hdy, dys[q], s.A2);
             }
-            const float4 r1 = s_rec[b][t][1];
             s.dx = P.dx;
-            s.a = r1.x;
-            s.b = r1.y;
-            s.c = r1.z;
             s.inv_o = rcp_approx(s_rec[b][t][0].w);   // sum dL/dalpha G = sum h / o
             return s;
         };
@@ -763,9 +771,7 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
             float4* rec4 = a.grad2d + 3 * (size_t)s_id[b][t];
             if (__popc(cm) <= kBwdDirectLanes) {
                 if (P.c0 || P.c1) {
-                    const float u = s[0].dx * s[0].A0;
-                    atomicAdd(rec4, make_float4(fmaf(s[0].a, u, s[0].b * s[0].A1), fmaf(s[0].b, u, s[0].c * s[0].A1),
-                                                s[0].dx * u, s[0].dx * s[0].A1));
+                    atomicAdd(rec4, make_float4(s[0].X, s[0].Y, s[0].dx * (s[0].dx * s[0].A0), s[0].dx * s[0].A1));
                     atomicAdd(rec4 + 1, make_float4(s[0].A2, s[0].A0 * s[0].inv_o, s[0].D, 0.f));
                     atomicAdd(rec4 + 2, make_float4(s[0].c0, s[0].c1, s[0].c2, 0.f));
                 }
