@@ -11,7 +11,7 @@ namespace gs {
 // Backward of the projection.  Screen-space sums per (view, Gaussian) come from the
 // backward compositing kernel (see render.cu for their definition):
 //   r0 = (sum h h_x, sum h h_y, sum h dx^2, sum h dx dy)
-//   r1 = (sum h dy^2, dL/do, dL/dz, 0), r2 = (dL/dr, dL/dg, dL/db, 0)
+//   r1 = (sum h dy^2, sum h = o dL/do, dL/dz, 0), r2 = (dL/dr, dL/dg, dL/db, 0)
 // with h = dL/dalpha * o * G and e = dx h_x + dy h_y.  Since dalpha/de = ln2 o G and
 // de/du = -2 h_x, de/dv = -2 h_y, de/dA = k dx^2, de/dB = 2 k dx dy, de/dC = k dy^2
 // (k = -log2(e)/2, ln2 log2(e) = 1): dL/du = -2 ln2 r0.x, dL/dv = -2 ln2 r0.y,
@@ -425,13 +425,13 @@ __device__ __forceinline__ void project_bwd_geo_rows(const ProjectBwdArgs& a, in
         for (int k = 0; k < 3; k++) g_mu[k] = a.dirgrad[k * n + i];
     }
     float gS[6] = {0, 0, 0, 0, 0, 0};   // dL/dSigma as a symmetric matrix: xx xy xz yy yz zz
-    float g_o = 0.f;
+    float g_h = 0.f;   // o dL/do
     for (uint64_t todo = vmask; todo; todo &= todo - 1) {
         const int v = __ffsll((long long)todo) - 1;
         const int64_t idx = (int64_t)v * n + i;
         const float4* geo = a.geo2d + 3 * idx;
         const float4 q0 = geo[0], q1 = geo[1], q2 = geo[2];
-        g_o += reinterpret_cast<const float*>(a.grad2d + 3 * idx + 1)[1];
+        g_h += reinterpret_cast<const float*>(a.grad2d + 3 * idx + 1)[1];
         g_mu[0] += q0.x; g_mu[1] += q0.y; g_mu[2] += q0.z;
         gS[0] += q0.w; gS[1] += q1.x; gS[2] += q1.y; gS[3] += q1.z; gS[4] += q1.w; gS[5] += q2.x;
     }
@@ -466,7 +466,7 @@ __device__ __forceinline__ void project_bwd_geo_rows(const ProjectBwdArgs& a, in
     for (int k = 0; k < 3; k++) { g[k] = g_mu[k]; g[3 + k] = gls[k]; }
 #pragma unroll
     for (int k = 0; k < 4; k++) g[6 + k] = (gq[k] - qn[k] * dq) * cv.qinv;
-    g[10] = g_o * o * (1.f - o);
+    g[10] = g_h * (1.f - o);
     // element i of geometry plane k (means 0-2, log-scales 3-5, quats 6-9, logit 10)
     auto at = [&](float* const* grp, int k) -> float& {
         return k < 3 ? grp[0][k * n + i] : k < 6 ? grp[1][(k - 3) * n + i] : k < 10 ? grp[2][(k - 6) * n + i]

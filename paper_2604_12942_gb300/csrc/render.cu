@@ -509,8 +509,9 @@ __global__ void __launch_bounds__(TileMap<TILE, kFwdPPT>::NT, kFwdThreadsPerSM /
 // If o G < alpha_max (the clamp is inactive), alpha = o 2^e gives dalpha/do = G and
 // dalpha/de = ln2 o G.  Per (view, Gaussian) the kernel accumulates, with h = dL/dalpha o G:
 //   r0 = (sum h h_x, sum h h_y, sum h dx^2, sum h dx dy)
-//   r1 = (sum h dy^2, sum dL/dalpha G, sum g_D w, 0), r2 = (sum g_C w, 0)
-// (h_x, h_y from frag_exponent) and the projection backward applies the constant factors.
+//   r1 = (sum h dy^2, sum h, sum g_D w, 0), r2 = (sum g_C w, 0)
+// (h_x, h_y from frag_exponent) and the projection backward applies the constant factors (sum h is
+// o times the opacity's gradient, and the logit's is o (1 - o) times that: nothing is divided by o).
 // A lane first sums its two pixels; the warp's sums are then reduced (bwd_reduce) and written by
 // 10 lanes with one atomic each -- or, when at most kBwdDirectLanes lanes contribute, added by
 // those lanes directly with vector atomics.
@@ -548,14 +549,14 @@ __device__ __forceinline__ float fold(float own, float other, int x) {
 // 1.4 times the error).
 struct BwdSums {
     float X, Y, A0, A1, A2, D, c0, c1, c2;
-    float dx, inv_o;   // the column's dx; 1 / the record's o
+    float dx;   // the column's
 };
 
 // Warp totals of N visits, stage by stage over all of them so that their shuffles overlap.  The
 // sums over rows come first (lane distances 16 and 8), on nine values a visit instead of ten; dx
 // then makes h dx^2 and h dx dy of a column's A0 and A1, and the lanes 8 r + x of row r hold three
 // (r = 0, 1) or two terms for the sums over columns:
-//   r = 0: h h_x, h h_y, h dx dy   r = 1: dL/dalpha G, h dx^2, h dy^2   r = 2: D, c0   r = 3: c1, c2
+//   r = 0: h h_x, h h_y, h dx dy   r = 1: h, h dx^2, h dy^2   r = 2: D, c0   r = 3: c1, c2
 // z[k] is the total for record slot bwd_slot(lane) of visit k.
 template <int N>
 __device__ __forceinline__ void bwd_reduce(int lane, const BwdSums (&s)[N], float (&z)[N]) {
@@ -579,7 +580,7 @@ __device__ __forceinline__ void bwd_reduce(int lane, const BwdSums (&s)[N], floa
     }
 #pragma unroll
     for (int k = 0; k < N; k++) {
-        v0[k] = r1 ? p[k] * s[k].inv_o : p[k];
+        v0[k] = p[k];
         v1[k] = r1 ? s[k].dx * s[k].dx * p[k] : q[k];
         v2[k] = r0 ? s[k].dx * k4[k] : q[k];
     }
@@ -762,7 +763,6 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
                 s.A2 = fmaf(hdy, dys[q], s.A2);
             }
             s.dx = P.dx;
-            s.inv_o = rcp_approx(s_rec[b][t][0].w);   // sum dL/dalpha G = sum h / o
             return s;
         };
         // one record added by the lanes of cm
@@ -772,7 +772,7 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
             if (__popc(cm) <= kBwdDirectLanes) {
                 if (P.c0 || P.c1) {
                     atomicAdd(rec4, make_float4(s[0].X, s[0].Y, s[0].dx * (s[0].dx * s[0].A0), s[0].dx * s[0].A1));
-                    atomicAdd(rec4 + 1, make_float4(s[0].A2, s[0].A0 * s[0].inv_o, s[0].D, 0.f));
+                    atomicAdd(rec4 + 1, make_float4(s[0].A2, s[0].A0, s[0].D, 0.f));
                     atomicAdd(rec4 + 2, make_float4(s[0].c0, s[0].c1, s[0].c2, 0.f));
                 }
             } else {
