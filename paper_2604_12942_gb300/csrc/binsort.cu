@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(kEntryThreads, 4) entry_compact_kernel(BinArgs
         }
     } else if (threadIdx.x < 32) {
         bool ok = true;
-        const unsigned long long before = lb_scan_warp(a.entry_scan, chunk, tot, a.counters, ok);
+        const unsigned long long before = lb_scan_warp(a.entry_scan, chunk, tot, a.counters, a.spin, ok);
         if (threadIdx.x == 0) {
             s_base = (uint32_t)before;
             s_ok = ok;
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kPairScanThreads) pair_offsets_kernel(BinArgs 
         const unsigned long long local = block_exclusive_scan_1024(sum, s, tot);
         if (threadIdx.x < 32) {
             bool ok = true;
-            const unsigned long long before = lb_scan_warp(a.pair_scan, ch, tot, a.counters, ok);
+            const unsigned long long before = lb_scan_warp(a.pair_scan, ch, tot, a.counters, a.spin, ok);
             if (threadIdx.x == 0) {
                 s_base = before;
                 s_ok = ok;

@@ -464,7 +464,8 @@ __device__ __forceinline__ void project_view(const float* mu, const Cov3& cv, fl
 }
 
 // ---------------------------------------------------------------------------------------
-// Decoupled look-back: one pass over chunks taken in ticket order, each publishing its total
+// Decoupled look-back (Merrill and Garland, "Single-pass Parallel Prefix Scan with Decoupled
+// Look-back", 2016): one pass over chunks taken in ticket order, each publishing its total
 // (state 1) and, once the totals before it are summed, its inclusive prefix (state 2) in one
 // 64-bit word: (tag * 4 + state) << 56 | value.  A chunk only waits for chunks with smaller
 // tickets, whose blocks are running, so every wait ends; a wait is bounded all the same: a scan's
@@ -516,10 +517,10 @@ __device__ __forceinline__ uint32_t lb_ticket(uint32_t* ticket, const Counters* 
 
 // One warp: publishes the chunk's total, sums the totals of the chunks before it (128 at a time:
 // the chunks of the first wave publish together and none has a prefix yet) and publishes the
-// inclusive prefix.  Returns the exclusive prefix; ok is cleared if a wait gave up (the status
-// word is then set).
+// inclusive prefix.  Returns the exclusive prefix; ok is cleared if a wait gave up, after `limit`
+// polls or because the status is set (it then is).
 __device__ __forceinline__ unsigned long long lb_scan_warp(lbword* words, int64_t chunk, unsigned long long total,
-                                                           Counters* c, bool& ok) {
+                                                           Counters* c, int limit, bool& ok) {
     const int lane = threadIdx.x & 31;
     if (chunk == 0) {
         if (lane == 0) lb_store(words, 0, 2, total);
@@ -551,7 +552,8 @@ __device__ __forceinline__ unsigned long long lb_scan_warp(lbword* words, int64_
                     done = full != 0;
                     break;
                 }
-                if (++spin > kLbSpin || ((spin & 1023) == 0 && *(volatile uint32_t*)&c->status != 0)) {
+                if (++spin > limit ||
+                    ((spin & 1023) == 0 && __any_sync(0xffffffffu, *(volatile uint32_t*)&c->status != 0))) {
                     if (lane == 0) set_status(c, GS_ERR_TIMEOUT);
                     ok = false;
                     return before;

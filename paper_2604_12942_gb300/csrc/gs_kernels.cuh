@@ -70,6 +70,7 @@ struct BinArgs {
     uint32_t* srt;                // [3][n_views * n] the depth-sorted entries' first tile ids,
                                   //   tile spans (wx | wy << 16) and view * n + index (scratch)
     Counters* counters;
+    int spin = kLbSpin;           // polls of a scan's wait before it gives up (GS_ERR_TIMEOUT)
 };
 
 // Stable LSD radix sort of (key, value) pairs; pass p reads buffer (p & 1) of keys / vals and
