@@ -336,7 +336,7 @@ def run_gpu(args, rank, world):
         torch.cuda.synchronize()
         c = step.ws.counters()
         print(json.dumps({"profile_step": args.profile_step, "status": int(c.status), "pairs": int(c.n_pairs),
-                          "kernels_per_step": launches_per_step(step.ws.layout)}), flush=True)
+                          "kernels_per_step": launches_per_step(step.ws.layout, sm_count(dev))}), flush=True)
         sys.exit(0 if c.status == 0 else 1)
     stages = ["project", "bin_sort", "render_fwd", "composite_bwd", "project_bwd_adam"]
     st = torch.cuda.current_stream()
@@ -413,8 +413,8 @@ def run_gpu(args, rank, world):
         return dict(f1=None, f23=None, a9=None, total_ms=total_ms, stage_ms=stage_ms, n_pairs=n_pairs, loss0=loss0,
                     loss_end=loss_end, tune=tune, adam_steps=adam_steps, eager_ms=None, h2d_ms=None, work=work,
                     clocks=clk.summary(), e2e_s=None, px=sum(w * h for w, h in SIZES), h2d=0, d2h=0, sc=sc,
-                    cams=cams, trgb=trgb, tdep=tdep, n=n, kernels=launches_per_step(step.ws.layout),
-                    sms=torch.cuda.get_device_properties(dev).multi_processor_count)
+                    cams=cams, trgb=trgb, tdep=tdep, n=n, kernels=launches_per_step(step.ws.layout, sm_count(dev)),
+                    sms=sm_count(dev))
     f1 = f1_measure(args, step, cams, trgb, tdep, planes0, cap, st, dev)
     f23 = f23_measure(step, cams, dev)
     a9 = a9_measure(args, planes0, cams, trgb, tdep, cap, st, total_ms / args.steps)
@@ -461,8 +461,8 @@ def run_gpu(args, rank, world):
                 tune=tune, adam_steps=adam_steps, eager_ms=eager_ms, h2d_ms=h2d_ms, work=work,
                 clocks=clk.summary(), e2e_s=e_dt, px=px, h2d=int(h_rgb.numel() * 4 + h_dep.numel() * 4),
                 d2h=int(h_loss.numel() * 4), sc=sc, cams=cams, trgb=trgb, tdep=tdep, n=n,
-                kernels=launches_per_step(step.ws.layout),
-                sms=torch.cuda.get_device_properties(dev).multi_processor_count)
+                kernels=launches_per_step(step.ws.layout, sm_count(dev)),
+                sms=sm_count(dev))
 
 
 F1_LAMBDA_SSIM, F1_ERODE = 0.2, 2
@@ -648,6 +648,11 @@ def f23_measure(step, cams, dev):
             "note": "calls between / beside mapping steps; each synchronizes its stream"}
 
 
+def sm_count(dev):
+    import torch
+    return torch.cuda.get_device_properties(dev).multi_processor_count
+
+
 def tile_sort_passes(L):
     """Radix passes of the pair sort: 8-bit digits, or 9-bit ones where that saves a pass."""
     tb = 0
@@ -667,8 +672,8 @@ def kernels_per_step(L):
     return 1 + 1 + 3 + 3 * 4 + 4 + 3 * tile_sort_passes(L) + 1 + 3 + 2 + 2 + 3
 
 
-def launches_per_step(L, sms=152):
-    """Kernels one gs_step launches (the graph replays exactly these)."""
+def launches_per_step(L, sms):
+    """Kernels one gs_step launches on a device of `sms` SMs (the graph replays exactly these)."""
     # setup (view table and clears), project, entry compaction (a count kernel before it once its
     # blocks of 64 words are more than 4 per SM), 4 depth-sort passes, pair offsets, emission, the
     # tile-sort passes, ranges, 2 tile-order kernels, loss count + composite, gradient-record

@@ -382,7 +382,7 @@ static cudaError_t run_bin_sort(const gs_render_opts* opts, const gs_ws_layout* 
     r.keys = static_cast<const uint32_t*>(sa.keys[np & 1]);
     r.ranges = at<uint2>(ws, L->ranges);
     r.counters = cnt;
-    if ((e = launch_ranges(r, L->total_tiles, st)) != cudaSuccess) return e;
+    if ((e = launch_ranges(r, st)) != cudaSuccess) return e;
     uint32_t* order = at<uint32_t>(ws, L->tile_order);
     return launch_tile_order(r.ranges, L->total_tiles, order, order + L->total_tiles, cnt, st);
 }

@@ -925,8 +925,7 @@ __global__ void __launch_bounds__(256) ranges_kernel(RangeArgs a) {
     }
 }
 
-cudaError_t launch_ranges(const RangeArgs& a, int n_tiles, cudaStream_t st) {
-    (void)n_tiles;
+cudaError_t launch_ranges(const RangeArgs& a, cudaStream_t st) {
     launch_pdl(ranges_kernel, device_sms() * 12, 256, 0, st, a);
     return cudaGetLastError();
 }

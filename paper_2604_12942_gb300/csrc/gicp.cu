@@ -83,7 +83,8 @@ __device__ __forceinline__ uint32_t g_hash(int cx, int cy, int cz, uint32_t mask
     return ((uint32_t)cx * 73856093u ^ (uint32_t)cy * 19349663u ^ (uint32_t)cz * 83492791u) & mask;
 }
 // buckets of the occupancy table, whose entries are the occupied cells of a 4 x 4 x 4 block
-// (bit x + 4 y + 16 z): other multipliers, so that they do not repeat the cells' collisions
+// (bit x + 4 y + 16 z): other multipliers (the first three primes of 32-bit xxHash), so that they
+// do not repeat the cells' collisions
 __device__ __forceinline__ uint32_t g_coarse(int cx, int cy, int cz, uint32_t mask) {
     return ((uint32_t)cx * 2654435761u ^ (uint32_t)cy * 2246822519u ^ (uint32_t)cz * 3266489917u) & mask;
 }

@@ -469,7 +469,8 @@ __device__ __forceinline__ void project_view(const float* mu, const Cov3& cv, fl
 // (state 1) and, once the totals before it are summed, its inclusive prefix (state 2) in one
 // 64-bit word: (tag * 4 + state) << 56 | value.  A chunk only waits for chunks with smaller
 // tickets, whose blocks are running, so every wait ends; a wait is bounded all the same: a scan's
-// then sets GS_ERR_TIMEOUT, a sort pass goes on without it (binsort.cu).  Words start at 0; the passes of one sort share words by tags.
+// then sets GS_ERR_TIMEOUT, a sort pass goes on without it (binsort.cu).  Words start at 0; the
+// passes of one sort share words by tags.
 // ---------------------------------------------------------------------------------------
 typedef unsigned long long lbword;
 constexpr int kLbSpin = 1 << 20;   // polls of a wait (about a second)

@@ -267,7 +267,7 @@ cudaError_t launch_sort32(const SortArgs& a, int n_passes, const int* shifts, co
 cudaError_t launch_sort64(const SortArgs& a, int n_passes, const int* shifts, cudaStream_t st);
 // digit counts of the first pass of a 64-bit sort (8 bits at `shift`)
 cudaError_t launch_sort_count64(const SortArgs& a, int shift, cudaStream_t st);
-cudaError_t launch_ranges(const RangeArgs& a, int n_tiles, cudaStream_t st);
+cudaError_t launch_ranges(const RangeArgs& a, cudaStream_t st);
 // tmp: kOrderTmpWords words, zero before the call
 constexpr int kOrderTmpWords = 2 * kOrderBuckets + 1;
 cudaError_t launch_tile_order(const uint2* ranges, int n_tiles, uint32_t* order, uint32_t* tmp, const Counters* c,

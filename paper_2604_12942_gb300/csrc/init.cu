@@ -1,9 +1,9 @@
 // a10-a11: voxel-PCA geometric fitting (RMGS-SLAM §III-A) and the cascaded Gaussian
 // initialisation (§III-B equations).  Points are grouped into cubic voxels by sorting their
-// voxel keys with the library's radix sort; one thread per voxel then computes the mean,
-// the covariance, a 3x3 Jacobi eigen-decomposition, the planar / linear classification and
-// the trace of the descriptor covariance, and writes the per-point features the learned
-// initialiser consumes.
+// voxel keys with the library's radix sort; a warp then takes the voxels that start among 32 sorted
+// points, for each the mean, the covariance, a 3x3 Jacobi eigen-decomposition, the planar / linear
+// classification and the trace of the descriptor covariance, and writes the per-point features the
+// learned initialiser consumes.
 #include <cstring>
 
 #include "gs_kernels.cuh"

@@ -198,7 +198,11 @@ __global__ void __launch_bounds__(kMuThreads) prune_mark_kernel(const unsigned l
 // with one atomic exchange a row, and a row's coordinates and link are one 16-byte record, so a
 // step along a list is one sector.  (A counting sort of the rows by slot took two passes with
 // two atomics a row and a scan of the table, and each visit then read four sectors: 200 us for
-// 2M means and 200k new ones, now 63.)  Eight cells along x share a 32-byte sector of slots, so
+// 2M means and 200k new ones, now 63.  Where very many map rows share a cell and none of them is
+// near, a list is a long chain of reads: 200k rows in dense cells and 50k new ones beside them take
+// 105, 115, 167, 542 and 3682 us at 1, 8, 64, 512 and 4096 rows a cell, the runs of the counting sort
+// took 146, 165, 275, 713 and 2180.  With the same rows spread evenly most new ones are near: 73 to
+// 86 us against 136 to 11137.)  Eight cells along x share a 32-byte sector of slots, so
 // the 27 cells are 9 reads of mostly one sector; 9 lanes take a new mean, each a row of three
 // cells whose lists it walks side by side, and all stop when one has found a near mean.  What
 // bounds both kernels is the rate of scattered sector reads and atomics at L2.

@@ -220,17 +220,6 @@ __device__ __forceinline__ uint32_t bwd_mask_from_fwd(uint32_t m) {
     return out;
 }
 
-__device__ __forceinline__ void load_record(const float4* proj, uint32_t gid, float2& uv, float4& co, float4& cz,
-                                            float& rx, float& ry) {
-    const float4* r = proj + 3 * (size_t)gid;
-    const float4 f0 = __ldg(r), f1 = __ldg(r + 1), f2 = __ldg(r + 2);
-    uv = make_float2(f0.x, f0.y);
-    co = make_float4(f1.x, f1.y, f1.z, f0.w);
-    cz = make_float4(f2.x, f2.y, f2.z, f0.z);
-    rx = (float)__float_as_int(f1.w);
-    ry = (float)__float_as_int(f2.w);
-}
-
 // ----------------------------------------------------------------------------------------
 // Forward compositing.
 // ----------------------------------------------------------------------------------------
