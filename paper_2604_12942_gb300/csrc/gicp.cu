@@ -417,9 +417,9 @@ __device__ __forceinline__ void se3_exp_dev(const double (&xi)[6], double (&E)[1
 // pivoting of the symmetric positive definite 6 x 6 system, a lane per entry), T <- Exp(xi) T,
 // and the next stage.  Stops without a step on fewer than 6 correspondences or a pivot that is
 // not positive.
-__device__ void gicp_step(GicpState* s, const double* acc, double (*A)[7]) {
+__device__ void gicp_step(GicpState* s, const double* acc, double (*A)[7], bool final_eval) {
     const int lane = threadIdx.x & 31;
-    if (s->stage == 1) {
+    if (final_eval) {
         if (lane == 0) s->stage = 2;
         return;
     }
@@ -589,7 +589,8 @@ __global__ void __launch_bounds__(kNormalThreads) gicp_normal_kernel(GicpMap src
     s_acc[0][lane] = __ldcg(&st->acc[lane]);
     __syncwarp();
     const bool final_eval = st->stage == 1;
-    gicp_step(st, s_acc[0], s_A);
+    __syncwarp();   // every lane has read the stage that lane 0 moves on
+    gicp_step(st, s_acc[0], s_A, final_eval);
     // the final evaluation's cost and count stay for the host
     if (!final_eval) st->acc[lane] = 0.0;
     if (lane == 0) st->blocks_done = 0;
