@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kGThreads) gicp_search_kernel(GicpMap src, int
 // a block first lists its matched pairs, so that warps are full, and the algebra is taken apart.
 // The planar covariance R diag(1, 1, 1e-3) R^T is I - 0.999 n n^T with n the column of R that
 // gets 1e-3, so Sigma~_n + R Sigma~_m R^T = I + R R^T - 0.999 (n n^T + m m^T), m = R n_m (R R^T is
-// formed once a thread and not taken for I: the caller's first transform is a rotation to its own
+// formed once a block and not taken for I: the caller's first transform is a rotation to its own
 // rounding only, and every later one keeps what it had; with 2 I in its place a transform given in
 // FP32 left ten times the error, and one 1e-3 off a rotation met another minimum); with O its
 // inverse and q^ the cross-product matrix of T mu_m the blocks of J^T O J (J = [-I | q^]) are
@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kNormalThreads) gicp_normal_kernel(GicpMap src
     if (st->stage == 2) return;
     __shared__ uint32_t s_li[kNormalRows], s_n;
     __shared__ double s_acc[kNormalThreads / 32][32];
-    __shared__ double s_A[6][7];
+    __shared__ double s_A[6][7], s_B[6];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     uint32_t ltm;
@@ -484,9 +484,14 @@ __global__ void __launch_bounds__(kNormalThreads) gicp_normal_kernel(GicpMap src
     double T[12];
 #pragma unroll
     for (int k = 0; k < 12; k++) T[k] = st->T[k];
-    // I + R R^T: xx xy xz yy yz zz
-    auto rr = [&](int a, int b) { return T[4 * a] * T[4 * b] + T[4 * a + 1] * T[4 * b + 1] + T[4 * a + 2] * T[4 * b + 2]; };
-    const double B0 = 1.0 + rr(0, 0), B1 = rr(0, 1), B2 = rr(0, 2), B3 = 1.0 + rr(1, 1), B4 = rr(1, 2), B5 = 1.0 + rr(2, 2);
+    // I + R R^T, xx xy xz yy yz zz, by six threads (18 operations a thread would be a twentieth of
+    // its pairs'); the barriers before the pairs order it
+    if (threadIdx.x < 6) {
+        const int k = threadIdx.x, a = k < 3 ? 0 : (k < 5 ? 1 : 2), b = k < 3 ? k : (k < 5 ? k - 2 : 2);
+        double v = a == b ? 1.0 : 0.0;
+        for (int e = 0; e < 3; e++) v += st->T[4 * a + e] * st->T[4 * b + e];
+        s_B[k] = v;
+    }
     const uint32_t cnt = st->n_list;
     const int64_t ns = src.n, nt = tar.n;
     double acc[32];
@@ -522,9 +527,11 @@ __global__ void __launch_bounds__(kNormalThreads) gicp_normal_kernel(GicpMap src
             // A = I + R R^T - 0.999 (n n^T + m m^T): xx xy xz yy yz zz
             const double kn[3] = {kPlanar * n[0], kPlanar * n[1], kPlanar * n[2]};
             const double km[3] = {kPlanar * mr[0], kPlanar * mr[1], kPlanar * mr[2]};
-            const double A0 = B0 - kn[0] * n[0] - km[0] * mr[0], A1 = B1 - kn[0] * n[1] - km[0] * mr[1],
-                         A2 = B2 - kn[0] * n[2] - km[0] * mr[2], A3 = B3 - kn[1] * n[1] - km[1] * mr[1],
-                         A4 = B4 - kn[1] * n[2] - km[1] * mr[2], A5 = B5 - kn[2] * n[2] - km[2] * mr[2];
+            // (read here each time: held over the loop they would take 16 registers, an eighth block of an SM)
+            const volatile double* B = s_B;
+            const double A0 = B[0] - kn[0] * n[0] - km[0] * mr[0], A1 = B[1] - kn[0] * n[1] - km[0] * mr[1],
+                         A2 = B[2] - kn[0] * n[2] - km[0] * mr[2], A3 = B[3] - kn[1] * n[1] - km[1] * mr[1],
+                         A4 = B[4] - kn[1] * n[2] - km[1] * mr[2], A5 = B[5] - kn[2] * n[2] - km[2] * mr[2];
             // inverse by the adjugate
             const double c0 = A3 * A5 - A4 * A4, c1 = A2 * A4 - A1 * A5, c2 = A1 * A4 - A2 * A3;
             const double id = 1.0 / (A0 * c0 + A1 * c1 + A2 * c2);
