@@ -512,10 +512,6 @@ __global__ void __launch_bounds__(TileMap<TILE, kFwdPPT>::NT, kFwdThreadsPerSM /
 // composited.  No block barrier: every warp proceeds at its own pace.
 // ----------------------------------------------------------------------------------------
 constexpr int kWin = 32;            // list positions per window
-// Items a resident warp from which two visits reduce together (render_bwd_region's JOINT): at 19.7
-// (95,680 items) it is better on two scenes (4055 and 4089, 3521 and 3555 us a step), at 9.5 better on
-// one and worse on the other (1439 and 1448, 1864 and 1820), at 2 worse.
-constexpr int kBwdJointWaves = 16;
 
 // A warp's shared memory: its two windows of staged records, their ids and list positions.
 struct BwdWarpSmem {
@@ -541,47 +537,23 @@ struct BwdSums {
     float dx;   // the column's
 };
 
-// Warp totals of N visits, stage by stage over all of them so that their shuffles overlap.  The
-// sums over rows come first (lane distances 16 and 8), on nine values a visit instead of ten; dx
-// then makes h dx^2 and h dx dy of a column's A0 and A1, and the lanes 8 r + x of row r hold three
+// Warp totals of a visit.  The sums over rows come first (lane distances 16 and 8), on nine values
+// instead of ten; dx then makes h dx^2 and h dx dy of a column's A0 and A1, and the lanes 8 r + x of row r hold three
 // (r = 0, 1) or two terms for the sums over columns:
 //   r = 0: h h_x, h h_y, h dx dy   r = 1: h, h dx^2, h dy^2   r = 2: D, c0   r = 3: c1, c2
-// z[k] is the total for record slot bwd_slot(lane) of visit k.
-template <int N>
-__device__ __forceinline__ void bwd_reduce(int lane, const BwdSums (&s)[N], float (&z)[N]) {
+// The result is the total for record slot bwd_slot(lane).
+__device__ __forceinline__ float bwd_reduce(int lane, const BwdSums& s) {
     const bool hi = lane & 16, odd = lane & 8, x4 = lane & 4, x2 = lane & 2;
     const bool r0 = !hi && !odd, r1 = !hi && odd;
-    float k0[N], k1[N], k2[N], k3[N], k4[N], p[N], q[N], v0[N], v1[N], v2[N];
-#pragma unroll
-    for (int k = 0; k < N; k++) {
-        k0[k] = fold(hi ? s[k].D : s[k].X, hi ? s[k].X : s[k].D, 16);
-        k1[k] = fold(hi ? s[k].c0 : s[k].Y, hi ? s[k].Y : s[k].c0, 16);
-        k2[k] = fold(hi ? s[k].c1 : s[k].A0, hi ? s[k].A0 : s[k].c1, 16);
-        k3[k] = fold(hi ? s[k].c2 : s[k].A2, hi ? s[k].A2 : s[k].c2, 16);
-        k4[k] = fold(s[k].A1, s[k].A1, 16);
-    }
+    const float k0 = fold(hi ? s.D : s.X, hi ? s.X : s.D, 16), k1 = fold(hi ? s.c0 : s.Y, hi ? s.Y : s.c0, 16);
+    const float k2 = fold(hi ? s.c1 : s.A0, hi ? s.A0 : s.c1, 16), k3 = fold(hi ? s.c2 : s.A2, hi ? s.A2 : s.c2, 16);
+    const float k4 = fold(s.A1, s.A1, 16);
     // p: X, A0, D, c1 and q: Y, A2, c0, c2 of rows 0 .. 3
-#pragma unroll
-    for (int k = 0; k < N; k++) {
-        p[k] = fold(odd ? k2[k] : k0[k], odd ? k0[k] : k2[k], 8);
-        q[k] = fold(odd ? k3[k] : k1[k], odd ? k1[k] : k3[k], 8);
-        k4[k] = fold(k4[k], k4[k], 8);
-    }
-#pragma unroll
-    for (int k = 0; k < N; k++) {
-        v0[k] = p[k];
-        v1[k] = r1 ? s[k].dx * s[k].dx * p[k] : q[k];
-        v2[k] = r0 ? s[k].dx * k4[k] : q[k];
-    }
-#pragma unroll
-    for (int k = 0; k < N; k++) {
-        v0[k] = fold(x4 ? v2[k] : v0[k], x4 ? v0[k] : v2[k], 4);
-        v1[k] = fold(v1[k], v1[k], 4);
-    }
-#pragma unroll
-    for (int k = 0; k < N; k++) z[k] = fold(x2 ? v1[k] : v0[k], x2 ? v0[k] : v1[k], 2);
-#pragma unroll
-    for (int k = 0; k < N; k++) z[k] = fold(z[k], z[k], 1);
+    const float p = fold(odd ? k2 : k0, odd ? k0 : k2, 8), q = fold(odd ? k3 : k1, odd ? k1 : k3, 8), a1 = fold(k4, k4, 8);
+    const float v1 = r1 ? s.dx * s.dx * p : q, v2 = r0 ? s.dx * a1 : q;
+    const float w0 = fold(x4 ? v2 : p, x4 ? p : v2, 4), w1 = fold(v1, v1, 4);
+    const float z = fold(x2 ? w1 : w0, x2 ? w0 : w1, 2);
+    return fold(z, z, 1);
 }
 
 // The record slot whose total bwd_reduce leaves in this lane, or -1.
@@ -599,14 +571,13 @@ __device__ __forceinline__ int bwd_slot(int lane) {
 // What bounds it: issue slots and the latency of a visit's chain while the chip is full (63 registers,
 // 32 one-warp blocks an SM; a tenth fewer instructions a visit moved the largest step by 1%), then
 // the longest lists, each walked by one warp.  alpha = 0 takes the place of three selects a pixel,
-// and sums by columns that of three products a pixel and two shuffles a visit.  JOINT reduces two
-// visits at once, so that their shuffles overlap: better while many warps share an SM, worse where a
-// lone warp's list sets the time.  Whole steps, ten values reduced / seven, h_x and h_y by columns too
-// / that with JOINT: 2M Gaussians, 8 views 4100, 4089, 4055 us; 200k, 8 small views 868, 860, 894;
-// 1M, 2 views 1348, 1327, 1344.  The nine values of this form against the seven, on one card: 3717
-// and 3730, 839 and 841, 1298 and 1298 us.  8 x 8 tiles, 1M, 2 views, as blocks with shared chunks /
-// this: 1176, 1130.
-template <int TILE, bool JOINT, bool COUNT, bool CHECK = true>
+// and sums by columns that of two products a pixel and two shuffles a visit.  Whole steps, ten values
+// reduced / seven, h_x and h_y by columns too: 2M Gaussians, 8 views 4100, 4089 us; 200k, 8 small
+// views 868, 860; 1M, 2 views 1348, 1327.  The nine values of this form against the seven, on one
+// card: 3717 and 3730, 839 and 841, 1298 and 1298 us.  (Two visits reduced together on large grids
+// paid with seven values, 34 of 4089 us; with nine it does not, 3933 and 3929.)  8 x 8 tiles, 1M, 2
+// views, as blocks with shared chunks / this: 1176, 1130.
+template <int TILE, bool COUNT, bool CHECK = true>
 __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, BwdWarpSmem& W) {
     constexpr int kPPT = kBwdPPT, WX = TILE / 8, R = WX * WX;
     auto& s_rec = W.rec;
@@ -756,22 +727,20 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
         };
         // one record added by the lanes of cm
         auto visit = [&](int t, const Alphas& P, uint32_t cm) {
-            const BwdSums s[1] = {adjoint(t, P)};
+            const BwdSums s = adjoint(t, P);
             float4* rec4 = a.grad2d + 3 * (size_t)s_id[b][t];
             if (__popc(cm) <= kBwdDirectLanes) {
                 if (P.c0 || P.c1) {
-                    atomicAdd(rec4, make_float4(s[0].X, s[0].Y, s[0].dx * (s[0].dx * s[0].A0), s[0].dx * s[0].A1));
-                    atomicAdd(rec4 + 1, make_float4(s[0].A2, s[0].A0, s[0].D, 0.f));
-                    atomicAdd(rec4 + 2, make_float4(s[0].c0, s[0].c1, s[0].c2, 0.f));
+                    atomicAdd(rec4, make_float4(s.X, s.Y, s.dx * (s.dx * s.A0), s.dx * s.A1));
+                    atomicAdd(rec4 + 1, make_float4(s.A2, s.A0, s.D, 0.f));
+                    atomicAdd(rec4 + 2, make_float4(s.c0, s.c1, s.c2, 0.f));
                 }
             } else {
-                float z[1];
-                bwd_reduce(lane, s, z);
-                if (slot >= 0) atomicAdd(reinterpret_cast<float*>(rec4) + slot, z[0]);
+                const float z = bwd_reduce(lane, s);
+                if (slot >= 0) atomicAdd(reinterpret_cast<float*>(rec4) + slot, z);
             }
         };
-        // two records per iteration: their alphas are independent (the adjoints are not), and so are
-        // their reductions
+        // two records per iteration: their alphas are independent (the adjoints are not)
         int t = 0;
         for (; t + 1 < cnt; t += 2) {
             Alphas A, B;
@@ -779,16 +748,6 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
             alphas(t + 1, B);
             const uint32_t ca = __ballot_sync(0xffffffffu, A.c0 || A.c1);
             const uint32_t cb = __ballot_sync(0xffffffffu, B.c0 || B.c1);
-            if (JOINT && min(__popc(ca), __popc(cb)) > kBwdDirectLanes) {
-                const BwdSums s[2] = {adjoint(t, A), adjoint(t + 1, B)};
-                float z[2];
-                bwd_reduce(lane, s, z);
-                if (slot >= 0) {
-                    atomicAdd(reinterpret_cast<float*>(a.grad2d + 3 * (size_t)s_id[b][t]) + slot, z[0]);
-                    atomicAdd(reinterpret_cast<float*>(a.grad2d + 3 * (size_t)s_id[b][t + 1]) + slot, z[1]);
-                }
-                continue;
-            }
             if (ca) visit(t, A, ca);
             if (cb) visit(t + 1, B, cb);
         }
@@ -810,11 +769,11 @@ __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, Bw
     }
 }
 
-template <int TILE, bool JOINT, bool COUNT>
+template <int TILE, bool COUNT>
 __global__ void __launch_bounds__(32, 32) render_bwd_warp_kernel(BwdArgs a) {
     pdl_begin();
     __shared__ BwdWarpSmem S;
-    render_bwd_region<TILE, JOINT, COUNT>(a, blockIdx.x, S);
+    render_bwd_region<TILE, COUNT>(a, blockIdx.x, S);
 }
 
 template <int TILE, int CHUNK>
@@ -841,10 +800,7 @@ static cudaError_t launch_fwd_t(const FwdArgs& a, int total_tiles, int chunk, cu
 template <int TILE>
 static cudaError_t launch_bwd_t(const BwdArgs& a, int total_tiles, cudaStream_t st) {
     const int items = total_tiles * (TILE / 8) * (TILE / 8);
-    const bool joint = items >= kBwdJointWaves * 32 * device_sms();
-    auto kernel = a.op.count ? render_bwd_warp_kernel<TILE, false, true>
-                  : joint    ? render_bwd_warp_kernel<TILE, true, false>
-                             : render_bwd_warp_kernel<TILE, false, false>;
+    auto kernel = a.op.count ? render_bwd_warp_kernel<TILE, true> : render_bwd_warp_kernel<TILE, false>;
     launch_pdl_small(kernel, items, 32, 0, st, a);
     return cudaGetLastError();
 }
@@ -1038,7 +994,7 @@ __global__ void __launch_bounds__(kPersistThreads, 2) step_persistent_kernel(Per
         if (lane == 0) item = atomicAdd(&P.sync->q_bwd, 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
         if (item >= 4u * (unsigned int)P.total_tiles) break;
-        render_bwd_region<16, false, false, false>(P.bwd, (int)item, S.u.bwd[warp]);
+        render_bwd_region<16, false, false>(P.bwd, (int)item, S.u.bwd[warp]);
     }
     if (!grid_barrier<DEG>(P, true, S)) return;
     project_bwd_entry_part<false>(P.pb, blockIdx.x, gridDim.x, S.tw);   // phase 3
