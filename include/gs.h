@@ -240,9 +240,11 @@ gs_status gs_workspace_init(const gs_ws_layout *L, void *ws, void *stream);
 
 /* Device-side failures.  The projection clears the status word; a stage that fails sets it
  * (GS_ERR_CAPACITY from the binning, GS_ERR_NONFINITE from the projection on a NaN or infinite
- * parameter) and every later stage of the step -- binning, compositing, backward, projection
- * backward, the fused Adam update and its step counter -- then does nothing, so a failed
- * step leaves the parameters, moments and Adam step unchanged.  gs_read_counters reports it. */
+ * parameter, GS_ERR_TIMEOUT from a scan or grid barrier whose bounded wait gave up; the sorts have
+ * no failure: a block whose wait gives up counts the keys before it itself) and every later stage
+ * of the step -- binning, compositing, backward, projection backward, the fused Adam update and its
+ * step counter -- then does nothing, so a failed step leaves the parameters, moments and Adam step
+ * unchanged.  gs_read_counters reports it. */
 
 /* a1 -- EWA projection with SH colour (§III-C "standard differentiable Gaussian splatting";
  * tile-based rasterizer of §II-A).  For every view v and Gaussian i: q = q/|q| -> R,

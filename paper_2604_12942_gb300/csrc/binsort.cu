@@ -138,13 +138,12 @@ __global__ void __launch_bounds__(kEntryThreads, 4) entry_compact_kernel(BinArgs
     __shared__ uint32_t s_hist[kSortBins];
     __shared__ bool s_ok;
     static_assert(kEntryThreads == kSortBins, "a thread per digit");
+    if (!LOOKBACK && a.counters->status != 0) return;   // (this form does not set it)
     s_hist[threadIdx.x] = 0;
     if (LOOKBACK) {
         if (threadIdx.x == 0) s_chunk = lb_ticket(&a.tickets[0], a.counters);
         __syncthreads();
         if (s_chunk == kLbStop) return;
-    } else if (a.counters->status != 0) {   // (this form does not set it)
-        return;
     }
     const int64_t chunk = LOOKBACK ? s_chunk : blockIdx.x, word = chunk * WPB + threadIdx.x;
     const uint32_t b = (int)threadIdx.x < WPB && word < n_words ? a.vis_bits[word] : 0u;
