@@ -568,15 +568,15 @@ __device__ __forceinline__ int bwd_slot(int lane) {
 // The backward of work item `item` = R t + w: region w of the R = (TILE / 8)^2 regions of the t-th
 // tile of the work order, by one warp with its own shared memory W.
 //
-// What bounds it: issue slots and the latency of a visit's chain while the chip is full (63 registers,
-// 32 one-warp blocks an SM; a tenth fewer instructions a visit moved the largest step by 1%), then
-// the longest lists, each walked by one warp.  alpha = 0 takes the place of three selects a pixel,
-// and sums by columns that of two products a pixel and two shuffles a visit.  Whole steps, ten values
-// reduced / seven, h_x and h_y by columns too: 2M Gaussians, 8 views 4100, 4089 us; 200k, 8 small
-// views 868, 860; 1M, 2 views 1348, 1327.  The nine values of this form against the seven, on one
-// card: 3717 and 3730, 839 and 841, 1298 and 1298 us.  (Two visits reduced together on large grids
-// paid with seven values, 34 of 4089 us; with nine it does not, 3933 and 3929.)  8 x 8 tiles, 1M, 2
-// views, as blocks with shared chunks / this: 1176, 1130.
+// What bounds it: the issue slots while the chip is full (79% of them taken; 62 registers, 32 one-warp
+// blocks an SM), then the longest lists, each walked by one warp.  alpha = 0 takes the place of three
+// selects a pixel, and sums by columns that of two products a pixel and two shuffles a visit: 884M
+// warp instructions and 900 us at 1M Gaussians and 8 views, 918M and 929 with ten values.  Whole
+// steps, ten values reduced / seven, h_x and h_y by columns too: 2M Gaussians, 8 views 4100, 4089 us;
+// 200k, 8 small views 868, 860; 1M, 2 views 1348, 1327.  The nine values of this form against the
+// seven, on one card: 3717 and 3730, 839 and 841, 1298 and 1298 us.  (Two visits reduced together on
+// large grids paid with seven values, 34 of 4089 us; with nine it does not, 3933 and 3929.)  8 x 8
+// tiles, 1M, 2 views, as blocks with shared chunks / this: 1176, 1130.
 template <int TILE, bool COUNT, bool CHECK = true>
 __device__ __forceinline__ void render_bwd_region(const BwdArgs& a, int item, BwdWarpSmem& W) {
     constexpr int kPPT = kBwdPPT, WX = TILE / 8, R = WX * WX;
